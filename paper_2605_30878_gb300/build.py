@@ -20,7 +20,7 @@ LIB = os.path.join(OUT_DIR, "liblbm.so")
 LIB_DEBUG = os.path.join(OUT_DIR, "liblbm_debug.so")
 SOURCES = ["lbm_api.cu", "lbm_kern_f32.cu", "lbm_kern_f64.cu", "lbm_kern_f16.cu", "lbm_noalloc.cu", "lbm_debug.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-# FP64 kernels round every multiply and add separately, as the FP64 oracle does.
+# FP64 kernels fuse a multiply and an add only where the source writes fma.
 EXTRA = {"lbm_kern_f64.cu": ["-fmad=false"]}
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall",
          "-I" + CSRC, "-I" + os.path.join(ROOT, "include")]

@@ -58,12 +58,12 @@ struct StepParams {
     T exp_eps;               // exp(eps), eps = -(4/W) cos(theta)
 };
 
-// Population storage.  S = double: full values (FP64 mode, rounding as the
-// oracle).  S = float: deviations from the rest state, N_i - chi_i and
-// B_i - chi_i/2 (FP32 mode); the step computes directly in these deviations,
+// Population storage.  N is stored as its deviation from the rest state,
+// N_i - chi_i, in every mode; the step computes directly in these deviations,
 // an exact rewrite because sum chi = 1, sum c chi = 0 and chi is isotropic, and
 // it keeps the small pressure of a dense liquid (p = p_h/rho ~ 1e-8 at density
-// ratio 1000) representable.  S = __half: the same deviations, the rest
+// ratio 1000) representable.  B: full values in S = double (FP64 mode),
+// B_i - chi_i/2 in S = float (FP32 mode).  S = __half: the same deviations, the rest
 // populations (i = 0, whose B deviation reaches chi_0/2 ~ 0.46) as float in the
 // first plane, the moving ones times 2^16 (N) and 2^7 (B) as FP16 in the
 // following Q-1 planes.
@@ -102,10 +102,10 @@ template <typename V> struct PlainStore {
     __device__ static void store_units(V* m, int idx, V v, V&) { m[idx] = v; }
 };
 template <> struct PopStore<double> : PlainStore<double> {
-    static constexpr bool kShift = false, kExact = true;
+    static constexpr bool kShift = true, kShiftB = false, kExact = true;
 };
 template <> struct PopStore<float> : PlainStore<float> {
-    static constexpr bool kShift = true, kExact = true;
+    static constexpr bool kShift = true, kShiftB = true, kExact = true;
     // two adjacent nodes (idx even, so 8-byte aligned): values in storage units
     __device__ static float2 load_units2(const float* m, int idx) {
         return __ldg(reinterpret_cast<const float2*>(m + idx));
@@ -116,7 +116,7 @@ template <> struct PopStore<float> : PlainStore<float> {
     __device__ static void store_zero2(float* m) { *reinterpret_cast<float2*>(m) = make_float2(0.f, 0.f); }
 };
 template <> struct PopStore<__half> {
-    static constexpr bool kShift = true, kExact = false;     // moving populations are rounded on store
+    static constexpr bool kShift = true, kShiftB = true, kExact = false;     // moving populations are rounded on store
     static constexpr int kRestBytes = 4, kMovingBytes = 2;
     __device__ static const float* rest(const __half* p) { return reinterpret_cast<const float*>(p); }
     __device__ static float* rest(__half* p) { return reinterpret_cast<float*>(p); }
@@ -186,7 +186,8 @@ struct StepBuffers {
 constexpr uint32_t MASK_NOT_FLUID = 0x80000000u;
 
 // Block tiles of the step kernels in the shapes the batch autotuner chooses
-// between (V = 0 is the one-node single-domain kernel's tile), in nodes:
+// between (V = 0 is the float one-node single-domain kernel's tile, V = 3 that
+// of FP64), in nodes:
 //   V                 0        1        2        3        4        5
 //   D3Q19           32x4x2   32x2x4   32x8x1   32x2x2   32x4x4   64x2x2
 //   D2Q9            32x8     64x4     128x2    32x4     32x16    64x4
@@ -408,16 +409,16 @@ __device__ __forceinline__ void phi_node(const StepParams<T>& P, const S* __rest
     // a grid coarse enough for their float sum to be exact, so the node's color
     // comes back as k_step wrote it.
     const T rest = (T)PS::load_rest(PS::rest(Bst), node);
-    T s = PS::kShift ? T(0) : rest;
+    T s = PS::kShiftB ? T(0) : rest;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const int idx = ((m >> i) & 1u) ? (L::opp(i) - 1) * pl + node
                                         : (i - 1) * pl + node + W.off(-L::cx(i), -L::cy(i), -L::cz(i));
         PS::accumulate(mv, idx_checked(idx, (long long)(Q - 1) * pl, err), s);
     }
-    if (PS::kShift) s = rest + (PS::kExact ? s : s * T(1.0 / kScaleB));
+    if (PS::kShiftB) s = rest + (PS::kExact ? s : s * T(1.0 / kScaleB));
     // stored deviations B_i - chi_i/2 sum to phi - 1/2
-    phi[node] = PS::kShift ? T(0.5) + s : s;
+    phi[node] = PS::kShiftB ? T(0.5) + s : s;
 }
 
 template <int Q, typename T, typename S>
@@ -461,7 +462,7 @@ __global__ void __launch_bounds__(256) k_ghost(int64_t n_ghosts, const int32_t* 
 // ---------------------------------------------------------------------------
 // k_step: stencils, forces, macroscopic fields, collision, segregation
 // ---------------------------------------------------------------------------
-// Reciprocals: FP64 divides exactly, as the oracle.  FP32 takes the hardware
+// Reciprocals: FP64 divides exactly.  FP32 takes the hardware
 // approximation (PTX rcp.approx, within 1 ulp): its operands here (the mixture
 // density, the mixture inverse viscosity, tau) are positive normal floats, so
 // the correctly rounded form's special-case handling buys nothing but
@@ -476,118 +477,10 @@ __device__ __forceinline__ float rcp(float v) {
     return r;
 }
 __device__ __forceinline__ double inv_norm_floor(double g2, double floor) {
-    const double gn = sqrt(g2);
-    return 1.0 / (gn > floor ? gn : floor);
+    return rsqrt(g2 > floor * floor ? g2 : floor * floor);
 }
 __device__ __forceinline__ float inv_norm_floor(float g2, float floor) {
     return rsqrtf(g2 > floor * floor ? g2 : floor * floor);
-}
-
-// FP64 node update written in the order the model is stated (Sec. II and
-// Appendix A), as the FP64 oracle evaluates it, so that FP64 results follow the
-// oracle to rounding; only the collision uses its closed form.  Inputs are the
-// lattice-order sums gs[a] = sum w c_a phi, ls = sum w (phi_i - phi),
-// us[a][b] = sum w c_a u_b.
-template <int Q, bool CONTRAST>
-__device__ __forceinline__ void node_update_literal(const StepParams<double>& P, const double* N, double phi,
-                                                    const double* gs, double ls, const double (*us)[3], double* Nst,
-                                                    double* Bst, double* u, double& p) {
-    using L = Lattice<Q>;
-    constexpr int D = L::D;
-    const double cs2 = 1.0 / 3.0;
-    const double w0 = L::w(0);
-    double gphi[3], gu[3][3];
-    for (int a = 0; a < 3; ++a) {
-        gphi[a] = gs[a] / cs2;
-        for (int c = 0; c < 3; ++c) gu[a][c] = us[a][c] / cs2;
-    }
-    const double lap = ls * (2.0 / cs2);
-    const double rho = P.rho_l * phi + P.rho_g * (1.0 - phi);
-    double grho[3];
-    for (int a = 0; a < 3; ++a) grho[a] = (P.rho_l - P.rho_g) * gphi[a];
-    const double nu = 1.0 / (phi / P.nu_l + (1.0 - phi) / P.nu_g);
-    const double tau = 0.5 + nu / cs2;
-    // force-free velocity and its pressure (Eq. pressureUpdate) for F_p
-    double u0[3] = {0.0, 0.0, 0.0};
-    double s = 0.0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        if (L::cx(i)) u0[0] += N[i] * L::cx(i);
-        if (L::cy(i)) u0[1] += N[i] * L::cy(i);
-        if (L::cz(i)) u0[2] += N[i] * L::cz(i);
-        if (i > 0) s += N[i];
-    }
-    const double uu0 = u0[0] * u0[0] + u0[1] * u0[1] + u0[2] * u0[2];
-    const double p0 = (-(w0 / 2.0) * uu0 - (1.0 - P.chi[0]) * cs2 + s * cs2) / (1.0 - w0);
-    // Eqs. (surfaceTensionForce), body force, (pressCorrection), (viscCorrection), (totalForce)
-    const double mu = (48.0 / P.W) * phi * (1.0 - phi) * (phi - 0.5) + (3.0 * P.W / 2.0) * lap;
-    double F[3];
-    for (int a = 0; a < 3; ++a) {
-        const double Fs = -P.sigma * mu * gphi[a];
-        const double Fb = rho * P.g[a];
-        double Fp = 0.0, Fv = 0.0;
-        if (CONTRAST) {
-            Fp = -p0 * grho[a];
-            for (int c = 0; c < 3; ++c) Fv += (gu[a][c] + gu[c][a]) * grho[c];
-            Fv *= cs2 * (tau - 0.5);
-        }
-        F[a] = Fv + Fp + Fs + Fb;
-    }
-    if (D == 2) F[2] = 0.0;
-    // Eqs. (velUpdate), (pressureUpdate)
-    for (int a = 0; a < 3; ++a) u[a] = u0[a] + F[a] / (2.0 * rho);
-    const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    p = (-(w0 / 2.0) * uu - (1.0 - P.chi[0]) * cs2 + s * cs2) / (1.0 - w0);
-    // Eq. (equilibriumDistribution), Eq. (forceGuo)
-    double neq[Q], Fi[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const double cu = L::cx(i) * u[0] + L::cy(i) * u[1] + L::cz(i) * u[2];
-        if (i == 0) neq[i] = P.chi[0] - (1.0 - w0) * p / cs2 - w0 * uu / (2.0 * cs2);
-        else neq[i] = P.chi[i] + L::w(i) * (p / cs2 + cu / cs2 + cu * cu / (2.0 * cs2 * cs2) - uu / (2.0 * cs2));
-        const double cF = L::cx(i) * F[0] + L::cy(i) * F[1] + L::cz(i) * F[2];
-        Fi[i] = (L::w(i) / cs2) * cF / rho;
-    }
-    // Eq. (MRTCOLL) in closed form: N* = Neq + F_i/2 + (1 - 1/tau) sum_k m_k (m_k . (N - Neq)) / |m_k|^2
-    // over the traceless second-order rows m_k
-    double mf[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
-        const double f = N[i] - neq[i];
-        if (D == 2) {
-            mf[0] += (cx * cx - cy * cy) * f;
-            mf[1] += (cx * cy) * f;
-        } else {
-            const int c2 = cx * cx + cy * cy + cz * cz;
-            mf[0] += (3 * cx * cx - c2) * f;
-            mf[1] += (cy * cy - cz * cz) * f;
-            mf[2] += (cx * cy) * f;
-            mf[3] += (cy * cz) * f;
-            mf[4] += (cx * cz) * f;
-        }
-    }
-    const double om = 1.0 - 1.0 / tau;
-    // segregation, Eq. (segragationStepBlue), n_phi = grad phi / max(|grad phi|, 1e-6)
-    const double gn = sqrt(gphi[0] * gphi[0] + gphi[1] * gphi[1] + gphi[2] * gphi[2]);
-    double n[3];
-    for (int a = 0; a < 3; ++a) n[a] = gphi[a] / (gn > 1e-6 ? gn : 1e-6);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
-        double proj;
-        if (D == 2) {
-            proj = (cx * cx - cy * cy) * mf[0] / 4.0 + (cx * cy) * mf[1] / 4.0;
-        } else {
-            const int c2 = cx * cx + cy * cy + cz * cz;
-            proj = (3 * cx * cx - c2) * mf[0] / 36.0 + (cy * cy - cz * cz) * mf[1] / 12.0 + (cx * cy) * mf[2] / 4.0 +
-                   (cy * cz) * mf[3] / 4.0 + (cx * cz) * mf[4] / 4.0;
-        }
-        Nst[i] = neq[i] + 0.5 * Fi[i] + om * proj;
-        const double cn = cx * n[0] + cy * n[1] + cz * n[2];
-        const double neq0 = P.chi[i] + L::w(i) * (p / cs2);
-        Bst[i] = phi * Nst[i] + 2.0 * (cn / P.W) * phi * (1.0 - phi) * neq0;
-    }
 }
 
 // The pull of the post-streaming populations N of node (x, y, z), issued
@@ -595,9 +488,9 @@ __device__ __forceinline__ void node_update_literal(const StepParams<double>& P,
 // always lies in the grid), then the directions whose neighbour is not fluid
 // are read again from the node's own opposite slot.  B enters the collision
 // only through phi = sum B, which k_phi computed.  Values come in storage
-// units (times kScaleN with FP16 storage).  Only the literal FP64 update reads
-// the rest population: in the deviation form the pressure and every moment
-// come from the moving populations (Eq. pressureUpdate), so N[0] is not read.
+// units (times kScaleN with FP16 storage).  In the deviation form the pressure
+// and every moment come from the moving populations (Eq. pressureUpdate), so
+// N[0] is not read.
 template <int Q, typename T, typename S>
 __device__ __forceinline__ void pull_streaming(const StepParams<T>& P, const S* __restrict__ Nin, int node, int x,
                                                int y, int z, T (&N)[Q], int* err) {
@@ -605,7 +498,7 @@ __device__ __forceinline__ void pull_streaming(const StepParams<T>& P, const S* 
     using PS = PopStore<S>;
     const Wrap Wr(x, y, z, P.nx, P.ny, P.nz, P.px);
     const int pl = (int)P.plane;
-    N[0] = PS::kShift ? T(0) : (T)PS::load_rest(PS::rest(Nin), idx_checked(node, P.plane, err));
+    N[0] = T(0);
     const auto* mv = PS::moving(Nin, pl);
 #pragma unroll
     for (int i = 1; i < Q; ++i)
@@ -635,6 +528,7 @@ __device__ __forceinline__ void pull_bounce_back(const StepParams<T>& P, const S
 // results to the bit, and the two-node kernel issues one float instruction
 // where the one-node kernel issues two.
 struct SF {
+    using Real = float;
     float v;
     __device__ __forceinline__ SF() {}
     __device__ __forceinline__ SF(float x) : v(x) {}
@@ -647,7 +541,25 @@ __device__ __forceinline__ SF fma(SF a, SF b, SF c) { return SF(fmaf(a.v, b.v, c
 __device__ __forceinline__ SF rcp(SF a) { return SF(rcp(a.v)); }
 __device__ __forceinline__ SF inv_norm_floor(SF g2, float floor) { return SF(inv_norm_floor(g2.v, floor)); }
 
+// SD is the FP64 modes' type: one double, fused where written as fma.
+struct SD {
+    using Real = double;
+    double v;
+    __device__ __forceinline__ SD() {}
+    __device__ __forceinline__ SD(double x) : v(x) {}
+};
+__device__ __forceinline__ SD operator+(SD a, SD b) { return SD(__dadd_rn(a.v, b.v)); }
+__device__ __forceinline__ SD operator-(SD a, SD b) { return SD(__dsub_rn(a.v, b.v)); }
+__device__ __forceinline__ SD operator*(SD a, SD b) { return SD(__dmul_rn(a.v, b.v)); }
+__device__ __forceinline__ SD operator-(SD a) { return SD(-a.v); }
+__device__ __forceinline__ SD fma(SD a, SD b, SD c) { return SD(::fma(a.v, b.v, c.v)); }
+__device__ __forceinline__ SD rcp(SD a) { return SD(rcp(a.v)); }
+__device__ __forceinline__ SD inv_norm_floor(SD g2, double floor) { return SD(inv_norm_floor(g2.v, floor)); }
+template <typename T> struct ScalarOf { using type = SF; };
+template <> struct ScalarOf<double> { using type = SD; };
+
 struct F2 {
+    using Real = float;
     unsigned long long v;                       // lane 0 (node A) low, lane 1 (node B) high
     __device__ __forceinline__ F2() {}
     __device__ __forceinline__ F2(float a) { asm("mov.b64 %0, {%1, %1};" : "=l"(v) : "f"(a)); }
@@ -697,23 +609,30 @@ __device__ __forceinline__ F2 inv_norm_floor(F2 g2, float floor) {
 // sum the same terms give in the same order, started from zero.
 template <typename V>
 struct Acc {
-    V v = V(0.f);
+    V v = V(typename V::Real(0));
     bool set = false;
     __device__ __forceinline__ void add(int k, V t) {
         if (k == 0) return;
         if (!set) {
-            v = k == 1 ? t : (k == -1 ? -t : V(float(k)) * t);
+            v = k == 1 ? t : (k == -1 ? -t : V(typename V::Real(k)) * t);
         } else {
-            v = k == 1 ? v + t : (k == -1 ? v - t : fma(V(float(k)), t, v));
+            v = k == 1 ? v + t : (k == -1 ? v - t : fma(V(typename V::Real(k)), t, v));
         }
         set = true;
     }
-    __device__ __forceinline__ V get() const { return set ? v : V(0.f); }
+    __device__ __forceinline__ V get() const { return set ? v : V(typename V::Real(0)); }
 };
 
 // ---------------------------------------------------------------------------
-// Float arithmetic of one fluid node (V = SF), or of the two nodes of a pair
-// (V = F2, one packed lane each), written once so that the one-node and the
+// FP64 runs it too: this GPU's FP64 rate (two lanes per clock and SM) makes the
+// FP64 step bound by its FP64 instructions alone, so what counts is how few a
+// node takes: ~580 in D3Q19 and ~280 in D2Q9 in this form, against ~2400 and
+// ~1150 for the model's expressions evaluated as printed (a division by each
+// constant, no fused multiply-add): 64^3 1237 -> 240 us per step, 500 x 300
+// 308 -> 71 us.
+//
+// Arithmetic of one fluid node (V = SF, or SD in FP64), or of the two nodes of a
+// pair (V = F2, one packed lane each), written once so that the one-node and the
 // two-node kernels round alike.  Inputs: the pulled populations N
 // (deviations, in storage units with FP16 storage), the color phi at the node
 // and its isotropic stencils gp = grad phi, lap = lap phi and gu[a][b] = d_a u_b
@@ -724,21 +643,24 @@ struct Acc {
 // this code computes the same values.
 // ---------------------------------------------------------------------------
 template <int Q, bool UNITS, bool CONTRAST, typename V>
-struct FloatNode {
+struct NodeUpdate {
     using L = Lattice<Q>;
+    using R = typename V::Real;
     static constexpr int D = L::D;
     static constexpr double w0 = L::w(0);
     // storage units: times sN (N) and sB (B), 2^16 and 2^7 with FP16 storage,
     // else 1.  Being powers of two, the scales fold into the per-node factors
     // (the stress projections, the weights, phi, kseg) and the scaled values
     // round exactly as the unscaled ones would.
-    static constexpr float sN = UNITS ? kScaleN : 1.0f, sB = UNITS ? kScaleB : 1.0f;
+    static constexpr R sN = UNITS ? kScaleN : 1, sB = UNITS ? kScaleB : 1;
+    // B is stored in full in FP64, as its deviation from chi/2 in float
+    static constexpr bool kFullB = sizeof(R) == 8;
     V phi, u[3], uu, p;
     V F[3], gp[3];
     V A0, A1, Axy, Axz, Ayz;                   // stress projections of N - Neq, times (1 - 1/tau)
     V base0, base1, base2, three_p, halfF;
     V common1, common2, krc1, krc2;            // per direction class (1 axis, 2 diagonal/edge)
-    V shb1, shb2;                              // (phi - 1/2) chi_i per class, in B's units
+    V shb1, shb2;                              // (phi - 1/2) chi_i per class, in B's units (FP64: phi chi_i)
     V phiB;
 
     // raw moments of the pulled N (storage units): sum, first and second moments
@@ -774,14 +696,14 @@ struct FloatNode {
         m_xy = Pxy.get(); m_xz = Pxz.get(); m_yz = Pyz.get();
     }
 
-    __device__ __forceinline__ void compute(const StepParams<float>& P, const V (&N)[Q], V phi_, const V (&gp_)[3],
+    __device__ __forceinline__ void compute(const StepParams<R>& P, const V (&N)[Q], V phi_, const V (&gp_)[3],
                                             V lap, const V (&gu)[3][3]) {
         moments(N);
         compute(P, phi_, gp_, lap, gu);
     }
 
     // the rest of the node update, after moments()
-    __device__ __forceinline__ void compute(const StepParams<float>& P, V phi_, const V (&gp_)[3], V lap,
+    __device__ __forceinline__ void compute(const StepParams<R>& P, V phi_, const V (&gp_)[3], V lap,
                                             const V (&gu)[3][3]) {
         phi = phi_;
 #pragma unroll
@@ -791,16 +713,16 @@ struct FloatNode {
         const V rho = fma(V(P.drho), phi, V(P.rho_g));
         const V inv_rho = rcp(rho);
         const V nu = rcp(fma(phi, V(P.inv_nu_l - P.inv_nu_g), V(P.inv_nu_g)));   // 1 / (phi/nu_l + (1-phi)/nu_g)
-        const V tau = fma(V(3.0f), nu, V(0.5f));
+        const V tau = fma(V(R(3.0)), nu, V(R(0.5)));
 
         // FP16 storage: N came in storage units (times sN = 2^16); the moments are
         // linear in N, so the scale is taken out where each is used (exactly, a
         // power of two): here for u0 and the pressure, in the stress projections
         // below for the second moments
-        constexpr float r = 1.0f / sN;
+        constexpr R r = R(1) / sN;
         V u0[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) u0[a] = (a < D) ? (UNITS ? m_u0[a] * V(r) : m_u0[a]) : V(0.f);
+        for (int a = 0; a < 3; ++a) u0[a] = (a < D) ? (UNITS ? m_u0[a] * V(r) : m_u0[a]) : V(R(0));
         // Eq. (pressureUpdate) takes sum_{i>0} N_i - (1 - chi_0) with the exact
         // chi; the deviations are stored from the rounded chi of the storage, whose
         // moving values sum to 1 - chi[0], so the difference of the two is
@@ -808,22 +730,22 @@ struct FloatNode {
         // pressure would sit a constant ~4e-8 off, which F_p = -p grad(rho)
         // turns into a velocity error at a density contrast)
         const V pres_base = (UNITS ? fma(m_sum, V(r), V(P.chi_err[0])) : m_sum + V(P.chi_err[0])) *
-                            V(float(1.0 / 3.0));
-        const V inv_1mw0 = V(float(1.0 / (1.0 - w0)));
+                            V(R(1.0 / 3.0));
+        const V inv_1mw0 = V(R(1.0 / (1.0 - w0)));
 
         // forces: surface tension and body force, then (density contrast) the
         // pressure and viscous corrections
-        const V muc = fma(V(P.k3W2), lap, V(P.k48W) * phi * (V(1.0f) - phi) * (phi - V(0.5f)));   // chemical potential / sigma
+        const V muc = fma(V(P.k3W2), lap, V(P.k48W) * phi * (V(R(1.0)) - phi) * (phi - V(R(0.5))));   // chemical potential / sigma
         const V smu = V(-P.sigma) * muc;
 #pragma unroll
         for (int a = 0; a < D; ++a) F[a] = fma(smu, gp[a], rho * V(P.g[a]));
-        if (D == 2) F[2] = V(0.f);
+        if (D == 2) F[2] = V(R(0));
         if (CONTRAST) {
             // F_p = -p0 grad(rho), F_v = nu (grad u + grad u^T) . grad(rho), grad(rho) = drho grad(phi)
             const V uu0 = D == 2 ? fma(u0[0], u0[0], u0[1] * u0[1])
                                  : fma(u0[0], u0[0], fma(u0[1], u0[1], u0[2] * u0[2]));
-            const V p0 = fma(V(-float(0.5 * w0)), uu0, pres_base) * inv_1mw0;
-            const V kd = (tau - V(0.5f)) * V(float(1.0 / 3.0)) * V(P.drho), pd = -p0 * V(P.drho);
+            const V p0 = fma(V(-R(0.5 * w0)), uu0, pres_base) * inv_1mw0;
+            const V kd = (tau - V(R(0.5))) * V(R(1.0 / 3.0)) * V(P.drho), pd = -p0 * V(P.drho);
             V sv[3];
             if (D == 2) {
                 const V t01 = gu[0][1] + gu[1][0];
@@ -840,28 +762,28 @@ struct FloatNode {
         }
 
         // Eq. (velUpdate), Eq. (pressureUpdate)
-        const V hr = V(0.5f) * inv_rho;
+        const V hr = V(R(0.5)) * inv_rho;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) u[a] = (a < D) ? fma(F[a], hr, u0[a]) : V(0.f);
+        for (int a = 0; a < 3; ++a) u[a] = (a < D) ? fma(F[a], hr, u0[a]) : V(R(0));
         uu = D == 2 ? fma(u[0], u[0], u[1] * u[1]) : fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
-        p = fma(V(-float(0.5 * w0)), uu, pres_base) * inv_1mw0;
+        p = fma(V(-R(0.5 * w0)), uu, pres_base) * inv_1mw0;
 
         // collision: traceless second moments of N - Neq, with sum Neq c c = (c2chi + p) I + u u,
         // in N's storage units (the moments are raw, the u u terms take the scale)
-        const V omega1 = V(1.0f) - rcp(tau);                                        // 1 - s_nu
-        const V o4 = omega1 * V(0.25f);
-        base0 = V(3.0f) * u[0];
-        base1 = V(3.0f) * u[1];
-        base2 = V(3.0f) * u[2];
+        const V omega1 = V(R(1.0)) - rcp(tau);                                        // 1 - s_nu
+        const V o4 = omega1 * V(R(0.25));
+        base0 = V(R(3.0)) * u[0];
+        base1 = V(R(3.0)) * u[1];
+        base2 = V(R(3.0)) * u[2];
         if (D == 2) {
             A0 = o4 * fma(V(-sN), fma(u[0], u[0], -(u[1] * u[1])), m_xx - m_yy);   // m7 . f / |m7|^2
-            A1 = V(0.f);
+            A1 = V(R(0));
             Axy = o4 * fma(V(-sN) * u[0], u[1], m_xy);                              // m8 . f / |m8|^2
-            Axz = Ayz = V(0.f);
+            Axz = Ayz = V(R(0));
         } else {
             // 2 ux^2 - uy^2 - uz^2 = 3 ux^2 - u.u
-            A0 = (omega1 * V(float(1.0 / 36.0))) * fma(V(-sN), fma(base0, u[0], -uu), fma(V(2.0f), m_xx, -m_yy) - m_zz);
-            A1 = (omega1 * V(float(1.0 / 12.0))) * fma(V(-sN), fma(u[1], u[1], -(u[2] * u[2])), m_yy - m_zz);
+            A0 = (omega1 * V(R(1.0 / 36.0))) * fma(V(-sN), fma(base0, u[0], -uu), fma(V(R(2.0)), m_xx, -m_yy) - m_zz);
+            A1 = (omega1 * V(R(1.0 / 12.0))) * fma(V(-sN), fma(u[1], u[1], -(u[2] * u[2])), m_yy - m_zz);
             const V su0 = V(-sN) * u[0];
             Axy = o4 * fma(su0, u[1], m_xy);
             Axz = o4 * fma(su0, u[2], m_xz);
@@ -870,24 +792,24 @@ struct FloatNode {
 
         // segregation: n_phi = grad phi / max(|grad phi|, 1e-6)
         const V g2 = D == 2 ? fma(gp[0], gp[0], gp[1] * gp[1]) : fma(gp[0], gp[0], fma(gp[1], gp[1], gp[2] * gp[2]));
-        const V inv_gn = inv_norm_floor(g2, 1e-6f);
-        const V kseg = V(P.two_over_W) * phi * (V(1.0f) - phi) * inv_gn;
+        const V inv_gn = inv_norm_floor(g2, R(1e-6));
+        const V kseg = V(P.two_over_W) * phi * (V(R(1.0)) - phi) * inv_gn;
         const V ksegB = UNITS ? kseg * V(sB) : kseg;                        // recoloring in B's units
         phiB = UNITS ? phi * V(sB / sN) : phi;                              // phi N*, from N's units to B's
-        const V phmB = UNITS ? (phi - V(0.5f)) * V(sB) : phi - V(0.5f);
+        const V phmB = kFullB ? phi : (UNITS ? (phi - V(R(0.5))) * V(sB) : phi - V(R(0.5)));
         shb1 = phmB * V(P.chi[1]);
         shb2 = phmB * V(P.chi[D == 2 ? 5 : 7]);
-        three_p = V(3.0f) * p;
-        halfF = V(1.5f) * inv_rho;   // (1/2) F_i = (3/2) w_i (c_i . F)/rho
-        const V common = fma(V(-1.5f), uu, three_p);
+        three_p = V(R(3.0)) * p;
+        halfF = V(R(1.5)) * inv_rho;   // (1/2) F_i = (3/2) w_i (c_i . F)/rho
+        const V common = fma(V(R(-1.5)), uu, three_p);
         // per direction class (1 axis, 2 diagonal/edge): the equilibrium's constant
         // part w_i (3p - 3u^2/2) + (chi_i - stored chi_i), divided by w_i, and the
         // recolouring weight ksegB (chi_i + w_i 3p) with the exact chi_i
         constexpr double kW1 = L::w(1), kW2 = L::w(D == 2 ? 5 : 7);
-        common1 = fma(V(P.chi_err[1]), V(float(1.0 / kW1)), common);
-        common2 = fma(V(P.chi_err[2]), V(float(1.0 / kW2)), common);
-        krc1 = ksegB * fma(V(float(kW1)), three_p, V(P.chi[1] + P.chi_err[1]));
-        krc2 = ksegB * fma(V(float(kW2)), three_p, V(P.chi[D == 2 ? 5 : 7] + P.chi_err[2]));
+        common1 = fma(V(P.chi_err[1]), V(R(1.0 / kW1)), common);
+        common2 = fma(V(P.chi_err[2]), V(R(1.0 / kW2)), common);
+        krc1 = ksegB * fma(V(R(kW1)), three_p, V(P.chi[1] + P.chi_err[1]));
+        krc2 = ksegB * fma(V(R(kW2)), three_p, V(P.chi[D == 2 ? 5 : 7] + P.chi_err[2]));
     }
 
     // Direction i (opp(i) > i) and its opposite o, in storage units: the
@@ -896,7 +818,7 @@ struct FloatNode {
     // B* = phi N* + recolor, i.e. phi dN* + (phi - 1/2) chi_i + recolor.
     __device__ __forceinline__ void dir(int i, V& ni, V& no, V& bi, V& bo) const {
         const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
-        const float wiN = float(L::w(i)) * sN;
+        const R wiN = R(L::w(i)) * sN;
         // the stress projection, 3 c.u, c.F and c.grad phi, each without the terms
         // whose lattice coefficient is zero
         Acc<V> proj, cu3, cF, cg;
@@ -917,7 +839,7 @@ struct FloatNode {
         const bool axis = cx * cx + cy * cy + cz * cz == 1;
         const V krc = axis ? krc1 : krc2, g = cg.get();                // recoloring krc (c . grad phi), odd in c
         const V c3 = cu3.get();
-        const V even = fma(V(wiN), fma(V(0.5f) * c3, c3, axis ? common1 : common2), proj.get());
+        const V even = fma(V(wiN), fma(V(R(0.5)) * c3, c3, axis ? common1 : common2), proj.get());
         const V odd = fma(halfF, cF.get(), c3);                        // the odd part over wiN
         ni = fma(V(wiN), odd, even);
         no = fma(V(-wiN), odd, even);
@@ -928,11 +850,11 @@ struct FloatNode {
 
     // Rest direction (no forcing, no stress projection, no recoloring, c_0 = 0),
     // stored exactly (FP32): N*_0 - chi_0 and B*_0 - chi_0/2.
-    __device__ __forceinline__ V rest_N(const StepParams<float>& P) const {
-        return fma(V(-float(1.5 * w0)), uu, fma(V(-float(1.0 - w0)), three_p, V(P.chi_err[0])));
+    __device__ __forceinline__ V rest_N(const StepParams<R>& P) const {
+        return fma(V(-R(1.5 * w0)), uu, fma(V(-R(1.0 - w0)), three_p, V(P.chi_err[0])));
     }
-    __device__ __forceinline__ V rest_B(const StepParams<float>& P, V nst0) const {
-        return fma(phi, nst0, (phi - V(0.5f)) * V(P.chi[0]));
+    __device__ __forceinline__ V rest_B(const StepParams<R>& P, V nst0) const {
+        return fma(phi, nst0, (kFullB ? phi : phi - V(R(0.5))) * V(P.chi[0]));
     }
     // With FP16 storage the float rest populations take the node totals the
     // collision fixes less the moving populations as stored (sumN, sumB in
@@ -963,11 +885,8 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
     using PS = PopStore<S>;
     constexpr bool kShift = PS::kShift;
 
-    // isotropic stencils: grad f = 3 sum_i w_i c_i f(x+c_i), lap f = 6 sum_i w_i (f(x+c_i) - f(x)).
-    // FP32 sums over +/- pairs (half the multiply-adds); FP64, the mode checked
-    // against the FP64 oracle to 1e-12 over thousands of steps, sums in lattice
-    // order as the definition is written.
-    constexpr bool kPairs = sizeof(T) == 4;
+    // isotropic stencils: grad f = 3 sum_i w_i c_i f(x+c_i), lap f = 6 sum_i w_i (f(x+c_i) - f(x)),
+    // summed over +/- pairs (half the multiply-adds)
     const T phi = s_phi[idx_checked(hc, Tl::HN, err)];
     T gp[3] = {T(0), T(0), T(0)};
     T lsum = T(0);
@@ -975,82 +894,45 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
-        const T wi = T(L::w(i));
-        if (kPairs) {
-            if (L::opp(i) < i) continue;
-            const int hp = hc + Tl::off(cx, cy, cz), hm = hc - Tl::off(cx, cy, cz);
-            // each difference enters every component it feeds with one
-            // multiply-add by the constant c_ia w_i
-            const T pp = s_phi[idx_checked(hp, Tl::HN, err)], pm = s_phi[idx_checked(hm, Tl::HN, err)];
-            const T dphi = pp - pm;
-            // the weights carry the 3 of the gradient and the 6 of the laplacian
-            const T g3 = T(3.0 * L::w(i)), l6 = T(6.0 * L::w(i));
-            if (cx) gp[0] = fmadd(T(cx) * g3, dphi, gp[0]);
-            if (cy) gp[1] = fmadd(T(cy) * g3, dphi, gp[1]);
-            if (cz) gp[2] = fmadd(T(cz) * g3, dphi, gp[2]);
-            lsum = fmadd(l6, (pp - phi) + (pm - phi), lsum);
-            if (CONTRAST) {
+        if (L::opp(i) < i) continue;
+        const int hp = hc + Tl::off(cx, cy, cz), hm = hc - Tl::off(cx, cy, cz);
+        // each difference enters every component it feeds with one
+        // multiply-add by the constant c_ia w_i
+        const T pp = s_phi[idx_checked(hp, Tl::HN, err)], pm = s_phi[idx_checked(hm, Tl::HN, err)];
+        const T dphi = pp - pm;
+        // the weights carry the 3 of the gradient and the 6 of the laplacian
+        const T g3 = T(3.0 * L::w(i)), l6 = T(6.0 * L::w(i));
+        if (cx) gp[0] = fmadd(T(cx) * g3, dphi, gp[0]);
+        if (cy) gp[1] = fmadd(T(cy) * g3, dphi, gp[1]);
+        if (cz) gp[2] = fmadd(T(cz) * g3, dphi, gp[2]);
+        lsum = fmadd(l6, (pp - phi) + (pm - phi), lsum);
+        if (CONTRAST) {
 #pragma unroll
-                for (int bb = 0; bb < D; ++bb) {
-                    const T dub = s_u[idx_checked(bb * Tl::HN + hp, D * Tl::HN, err)] -
-                                  s_u[idx_checked(bb * Tl::HN + hm, D * Tl::HN, err)];
-                    if (cx) du[0][bb] = fmadd(T(cx) * g3, dub, du[0][bb]);
-                    if (cy) du[1][bb] = fmadd(T(cy) * g3, dub, du[1][bb]);
-                    if (cz) du[2][bb] = fmadd(T(cz) * g3, dub, du[2][bb]);
-                }
-            }
-        } else {
-            const int h = hc + Tl::off(cx, cy, cz);
-            const T ph = s_phi[idx_checked(h, Tl::HN, err)];
-            gp[0] += wi * T(cx) * ph;
-            gp[1] += wi * T(cy) * ph;
-            if (D == 3) gp[2] += wi * T(cz) * ph;
-            lsum += wi * (ph - phi);
-            if (CONTRAST) {
-#pragma unroll
-                for (int bb = 0; bb < D; ++bb) {
-                    const T ub = s_u[idx_checked(bb * Tl::HN + h, D * Tl::HN, err)];
-                    du[0][bb] += wi * T(cx) * ub;
-                    du[1][bb] += wi * T(cy) * ub;
-                    if (D == 3) du[2][bb] += wi * T(cz) * ub;
-                }
+            for (int bb = 0; bb < D; ++bb) {
+                const T dub = s_u[idx_checked(bb * Tl::HN + hp, D * Tl::HN, err)] -
+                              s_u[idx_checked(bb * Tl::HN + hm, D * Tl::HN, err)];
+                if (cx) du[0][bb] = fmadd(T(cx) * g3, dub, du[0][bb]);
+                if (cy) du[1][bb] = fmadd(T(cy) * g3, dub, du[1][bb]);
+                if (cz) du[2][bb] = fmadd(T(cz) * g3, dub, du[2][bb]);
             }
         }
     }
-    constexpr double w0 = L::w(0);
-    if constexpr (sizeof(T) == 8) {
-        double Ns[Q], Bs[Q], u[3], p;
-        node_update_literal<Q, CONTRAST>(P, N, phi, gp, lsum, du, Ns, Bs, u, p);
-        PS::store_rest(PS::rest(b.Nout), node, Ns[0]);
-        PS::store_rest(PS::rest(b.Bout), node, Bs[0]);
-        auto* Nmv = PS::moving(b.Nout, pl);
-        auto* Bmv = PS::moving(b.Bout, pl);
-#pragma unroll
-        for (int i = 1; i < Q; ++i) {
-            PS::store_moving(Nmv, (i - 1) * pl + node, Ns[i], kScaleN);
-            PS::store_moving(Bmv, (i - 1) * pl + node, Bs[i], kScaleB);
-        }
-#pragma unroll
-        for (int a = 0; a < D; ++a) b.u_out[a * pl + node] = u[a];
-        b.p[node] = p;
-        if (!(u[0] * u[0] + u[1] * u[1] + u[2] * u[2] < 1e30)) atomicOr(b.err, kErrNonFinite);
-        return;
-    } else {
-    static_assert(kPairs && kShift, "float arithmetic runs on deviations, summed over +/- pairs");
+    static_assert(kShift, "the node update runs on deviations");
     constexpr bool kUnits = !PS::kExact;
-    using FN = FloatNode<Q, kUnits, CONTRAST, SF>;
+    using Sc = typename ScalarOf<T>::type;
+    using FN = NodeUpdate<Q, kUnits, CONTRAST, Sc>;
     FN nd;
     {
-        SF Ns[Q], gps[3], gus[3][3];
+        Sc Ns[Q], gps[3], gus[3][3];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) Ns[i] = SF(N[i]);
+        for (int i = 0; i < Q; ++i) Ns[i] = Sc(N[i]);
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            gps[a] = SF(gp[a]);
+            gps[a] = Sc(gp[a]);
 #pragma unroll
-            for (int bb = 0; bb < 3; ++bb) gus[a][bb] = SF(du[a][bb]);
+            for (int bb = 0; bb < 3; ++bb) gus[a][bb] = Sc(du[a][bb]);
         }
-        nd.compute(P, Ns, SF(phi), gps, SF(lsum), gus);
+        nd.compute(P, Ns, Sc(phi), gps, Sc(lsum), gus);
     }
 
     // u and p: FP16 storage writes them before the populations, which frees
@@ -1067,7 +949,7 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
     auto* __restrict__ Nmov = PS::moving(b.Nout, pl);
     auto* __restrict__ Bmov = PS::moving(b.Bout, pl);
     if constexpr (PS::kExact) {
-        const SF nst0 = nd.rest_N(P);
+        const Sc nst0 = nd.rest_N(P);
         PS::store_rest(PS::rest(b.Nout), node, nst0.v);
         PS::store_rest(PS::rest(b.Bout), node, nd.rest_B(P, nst0).v);
     }
@@ -1077,7 +959,7 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
     for (int i = 1; i < Q; ++i) {
         if (L::opp(i) < i) continue;
         const int o = L::opp(i);
-        SF ni, no, bi, bo;
+        Sc ni, no, bi, bo;
         nd.dir(i, ni, no, bi, bo);
         PS::store_units(Nmov, (i - 1) * pl + node, ni.v, sumN);
         PS::store_units(Nmov, (o - 1) * pl + node, no.v, sumN);
@@ -1089,7 +971,6 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
         PS::store_rest(PS::rest(b.Bout), node, FN::rest_B_from_sum(sumB, nd.phi.v));
     }
     if constexpr (PS::kExact) store_u_p();
-    }
 }
 
 // The periodic images of x = -1 and x = nx that a block at an x end of the

@@ -2,7 +2,7 @@
 //
 // Every thread updates the two x-adjacent nodes A = (x0 + 2t, y, z) and
 // B = (x0 + 2t + 1, y, z) of its row, with the arithmetic of k_step: the same
-// stencil sums in the same order and FloatNode's per-node update, so the two
+// stencil sums in the same order and NodeUpdate's per-node update, so the two
 // kernels round alike.  Since A's index is even, the pair shares
 //   - its mask (one 8-byte load),
 //   - its streaming pulls along y and z (one two-wide load per direction with
@@ -13,7 +13,7 @@
 //   - its stores of N*, B*, u and p (one two-wide store each),
 // which halves the load/store and address instructions per node of the
 // one-node kernel.  The float arithmetic of the two nodes runs on packed
-// pairs (FloatNode<..., F2>: one add/mul/fma.f32x2 for both nodes, each lane
+// pairs (NodeUpdate<..., F2>: one add/mul/fma.f32x2 for both nodes, each lane
 // rounded as the one-node kernel's scalar operation), which halves the float
 // instructions too.  Blocks are TX/2 x TY x TZ threads covering TX x TY x TZ
 // nodes; the halo tile is copied by the same halo_issue/halo_complete as
@@ -132,7 +132,7 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
     // the moments of both nodes (one packed lane each) while the halo copy
     // completes; the pulled values are then dead, which keeps them out of the
     // registers the stencils need
-    FloatNode<Q, kUnits, CONTRAST, F2> n2;
+    NodeUpdate<Q, kUnits, CONTRAST, F2> n2;
     {
         F2 N2[Q];
 #pragma unroll
@@ -245,7 +245,7 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
         rn = make_float2(n0.lo(), n0.hi());
         rb = make_float2(b0.lo(), b0.hi());
     } else {
-        using FN = FloatNode<Q, kUnits, CONTRAST, F2>;
+        using FN = NodeUpdate<Q, kUnits, CONTRAST, F2>;
         rn = make_float2(FN::rest_N_from_sum(sNA), FN::rest_N_from_sum(sNB));
         rb = make_float2(FN::rest_B_from_sum(sBA, n2.phi.lo()), FN::rest_B_from_sum(sBB, n2.phi.hi()));
     }

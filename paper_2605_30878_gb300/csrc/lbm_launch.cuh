@@ -51,9 +51,9 @@ struct StepPtrs {
 template <typename T, typename S>
 struct Launch {
     static StepParams<T> params(const StepConfig& c);
-    template <int Q>
+    template <int Q, int V = 0>
     static dim3 step_grid(const Dims& d);
-    template <int Q>
+    template <int Q, int V = 0>
     static dim3 step_block();
     template <int Q>
     static dim3 pair_grid(const Dims& d);

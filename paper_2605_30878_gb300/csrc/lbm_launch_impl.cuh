@@ -55,16 +55,16 @@ StepParams<T> Launch<T, S>::params(const StepConfig& c) {
 }
 
 template <typename T, typename S>
-template <int Q>
+template <int Q, int V>
 dim3 Launch<T, S>::step_grid(const Dims& d) {
-    using Tl = Tile<Q>;
+    using Tl = Tile<Q, V>;
     return dim3((d.nx + Tl::TX - 1) / Tl::TX, (d.ny + Tl::TY - 1) / Tl::TY, (d.nz + Tl::TZ - 1) / Tl::TZ);
 }
 
 template <typename T, typename S>
-template <int Q>
+template <int Q, int V>
 dim3 Launch<T, S>::step_block() {
-    using Tl = Tile<Q>;
+    using Tl = Tile<Q, V>;
     return dim3(Tl::TX, Tl::TY, Tl::TZ);
 }
 
@@ -100,6 +100,19 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s
                 k_step_pair<Q, S, false><<<pair_grid<Q>(c.d), block, 0, s>>>(P, b, tm_phi, tm_u, tma);
             return;
         }
+    }
+    if constexpr (sizeof(T) == 8) {
+        // 128-thread tiles: FP64 is bound by its arithmetic rate per SM, so what
+        // counts is that every SM has blocks and the last ones are short.  Against
+        // 256-thread tiles (shape 0): 64^2 19.7 -> 13.3 us per step, 300^2 54.9 ->
+        // 47.2, 24^3 41.2 -> 25.6, equal from 500 x 300 and 64^3 on; one-warp
+        // tiles gain nothing more (13.1, 47.2, 26.6).
+        constexpr int V = 3;
+        if (c.contrast)
+            k_step<Q, T, S, true, V><<<step_grid<Q, V>(c.d), step_block<Q, V>(), 0, s>>>(P, b, tm_phi, tm_u, 0);
+        else
+            k_step<Q, T, S, false, V><<<step_grid<Q, V>(c.d), step_block<Q, V>(), 0, s>>>(P, b, tm_phi, tm_u, 0);
+        return;
     }
     if (sizeof(T) == 4 && p.tm_phi && p.tm_u) {
         tm_phi = *p.tm_phi;
@@ -184,7 +197,7 @@ void Launch<T, S>::build_mask(const StepConfig& c, const uint8_t* cls, uint32_t*
 // base subtracted from direction i of N (is_b = false) or B (true) in storage
 template <typename T, typename S>
 double Launch<T, S>::storage_base(const StepConfig& c, int i, bool is_b) {
-    if (!PopStore<S>::kShift) return 0.0;
+    if (!(is_b ? PopStore<S>::kShiftB : PopStore<S>::kShift)) return 0.0;
     double chi[19];                     // the deviations are taken from the chi the kernels use
     if (sizeof(T) == 4) chi_for_float(c.chi, chi);
     else std::memcpy(chi, c.chi, sizeof(chi));
