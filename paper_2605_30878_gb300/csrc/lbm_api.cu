@@ -46,7 +46,7 @@ struct Layout {
     size_t rest_elem = 0;            // bytes of a stored rest population
     size_t pop_bytes = 0;            // bytes of one population array (Q planes)
     int Q = 0, D = 0, GK = 0;
-    size_t off_N[2], off_B[2], off_phi, off_u[2], off_p, off_cls, off_mask, off_gnode, off_gcorner, off_gwt,
+    size_t off_N[2], off_B, off_flux, off_phi[2], off_phi_lo, off_u[2], off_p, off_cls, off_mask, off_gnode, off_gcorner, off_gwt,
         off_err, off_partial, off_dout, off_stage;
     size_t total = 0;
 };
@@ -81,8 +81,12 @@ bool make_layout(const lbm_params* P, int64_t ng, Layout& L, std::string& err) {
     auto take = [&](size_t bytes) { size_t r = o; o = round_up(o + bytes, ALIGN); return r; };
     const size_t pop = (size_t)L.plane * (L.rest_elem + (size_t)(L.Q - 1) * L.pop_elem);
     L.pop_bytes = pop;
-    for (int k = 0; k < 2; ++k) { L.off_N[k] = take(pop); L.off_B[k] = take(pop); }
-    L.off_phi = take(L.plane * L.elem);
+    for (int k = 0; k < 2; ++k) L.off_N[k] = take(pop);
+    L.off_B = take(pop);                                 // state transfer only
+    L.off_flux = take((size_t)L.D * L.plane * L.elem);
+    L.off_phi[1] = take(L.plane * L.elem);
+    L.off_phi[0] = take(L.plane * L.elem);
+    L.off_phi_lo = take(P->precision == LBM_FP64 ? 0 : L.plane * L.elem);
     for (int k = 0; k < 2; ++k) L.off_u[k] = take((size_t)L.D * L.plane * L.elem);
     L.off_p = take(L.plane * L.elem);
     L.off_cls = take(L.plane);
@@ -128,6 +132,11 @@ cudaMemPool_t workspace_pool(int device) {
 
 }  // namespace
 
+// tiled maps of a domain's halo fields, one box
+struct HaloMaps {
+    CUtensorMap phi[2], u[2], flux;
+};
+
 struct lbm_domain {
     lbm_params prm;
     Layout lay;
@@ -159,21 +168,24 @@ struct lbm_domain {
     cudaGraphExec_t g1[2] = {nullptr, nullptr};
     cudaGraphExec_t g8 = nullptr;
     std::string err;
-    // tiled TMA maps of phi and of both velocity buffers for the step kernel's
-    // halo copies (FP32 arithmetic, rows of a multiple of 16 bytes)
+    // tiled TMA maps of both colors, both velocity buffers and the flux for the
+    // halo copies, with the box of the domain's step kernel
     bool tma = false;
-    CUtensorMap tm_phi{}, tm_u[2]{};
-    bool tma2 = false;                     // the same with the two-node kernel's box
-    CUtensorMap tm2_phi{}, tm2_u[2]{};
+    HaloMaps maps;
+    // true: the buffer B() holds the current B (set by an init or a written B);
+    // false: B follows from the last step's color, N* and flux (rebuild_B)
+    bool b_stored = true;
     // set once a bounded halo-copy wait gave up (LBM_ERR_TIMEOUT): a skipped
     // tile left the state wrong, so the domain takes no further steps
     bool poisoned = false;
 
     template <typename P> P* at(size_t off) const { return reinterpret_cast<P*>(ws + off); }
     void* N(int k) const { return at<void>(lay.off_N[k]); }
-    void* B(int k) const { return at<void>(lay.off_B[k]); }
+    void* B() const { return at<void>(lay.off_B); }
+    void* flux() const { return at<void>(lay.off_flux); }
     void* U(int k) const { return at<void>(lay.off_u[k]); }
-    void* phi() const { return at<void>(lay.off_phi); }
+    void* phi(int k) const { return at<void>(lay.off_phi[k]); }
+    void* phi_lo() const { return at<void>(lay.off_phi_lo); }
     void* p() const { return at<void>(lay.off_p); }
     uint8_t* cls() const { return at<uint8_t>(lay.off_cls); }
     uint32_t* mask() const { return at<uint32_t>(lay.off_mask); }
@@ -588,7 +600,18 @@ lbm_status prepare_ghosts(lbm_domain* d, const lbm_ghost* ghosts) {
     return LBM_OK;
 }
 
-// ev: optional events {before ghost, before step, before phi, after phi}
+// The buffers of a step that starts from buffers cur.
+StepPtrs step_ptrs(const lbm_domain* d, int cur) {
+    StepPtrs sp;
+    sp.Nin = d->N(cur); sp.Nout = d->N(1 - cur);
+    sp.phi = d->phi(cur); sp.phi_out = d->phi(1 - cur); sp.phi_lo = d->phi_lo();
+    sp.u_in = d->U(cur); sp.u_out = d->U(1 - cur); sp.p = d->p(); sp.flux = d->flux();
+    sp.mask = d->mask(); sp.err = d->errflag();
+    if (d->tma) { sp.tm_phi = &d->maps.phi[cur]; sp.tm_u = &d->maps.u[cur]; sp.tm_flux = &d->maps.flux; }
+    return sp;
+}
+
+// ev: optional events {before ghost, before step, before color, after color}
 void launch_one_step(lbm_domain* d, int cur, cudaStream_t s, cudaEvent_t* ev = nullptr) {
     const Layout& L = d->lay;
     if (ev) cudaEventRecord(ev[0], s);
@@ -596,20 +619,15 @@ void launch_one_step(lbm_domain* d, int cur, cudaStream_t s, cudaEvent_t* ev = n
         const void* wt = d->at<void>(L.off_gwt);
         dispatch(d, [&](auto Lx) {
             decltype(Lx)::ghost(L.GK, d->cfg.ghost_rule, d->ng, d->at<int32_t>(L.off_gnode),
-                                d->at<int32_t>(L.off_gcorner), wt, d->cfg.exp_eps, d->cfg.eps, d->phi(), L.plane,
+                                d->at<int32_t>(L.off_gcorner), wt, d->cfg.exp_eps, d->cfg.eps, d->phi(cur), L.plane,
                                 d->errflag(), s);
         });
     }
-    StepPtrs sp;
-    sp.Nin = d->N(cur); sp.Bin = d->B(cur); sp.Nout = d->N(1 - cur); sp.Bout = d->B(1 - cur);
-    sp.phi = d->phi(); sp.u_in = d->U(cur); sp.u_out = d->U(1 - cur); sp.p = d->p();
-    sp.mask = d->mask(); sp.err = d->errflag();
-    if (d->tma) { sp.tm_phi = &d->tm_phi; sp.tm_u = &d->tm_u[cur]; }
-    if (d->tma2) { sp.tm2_phi = &d->tm2_phi; sp.tm2_u = &d->tm2_u[cur]; }
+    const StepPtrs sp = step_ptrs(d, cur);
     if (ev) cudaEventRecord(ev[1], s);
     dispatch(d, [&](auto Lx) { decltype(Lx)::step(d->cfg, sp, s); });
     if (ev) cudaEventRecord(ev[2], s);
-    dispatch(d, [&](auto Lx) { decltype(Lx)::phi(d->cfg, d->B(1 - cur), d->mask(), d->phi(), d->errflag(), s); });
+    dispatch(d, [&](auto Lx) { decltype(Lx)::color(d->cfg, sp, s); });
     if (ev) cudaEventRecord(ev[3], s);
 }
 
@@ -643,59 +661,46 @@ EncodeTiledFn encode_tiled() {
     return fn;
 }
 
-// Tensor maps for the halo copies of the step kernel: phi as (nx, ny, nz) and
-// each velocity buffer as (nx, ny, nz, D) floats, box = the halo tile of
-// Tile<Q, V>; out[0] = phi, out[1 + k] = velocity buffer k.  Only for float
-// fields whose rows are a multiple of 16 bytes (the strides TMA accepts);
-// otherwise, or if the driver refuses, the kernel copies every halo element
-// itself.
+// Tensor maps for the halo copies: each color as (nx, ny, nz), each velocity
+// buffer and the flux as (nx, ny, nz, D) values, box = the halo tile of Tl.
+// Rows are a multiple of 16 bytes (the strides TMA accepts); if the driver
+// refuses, the kernel copies every halo element itself.
 template <class Tl>
-bool encode_halo_maps_tile(const lbm_domain* d, CUtensorMap out[3]) {
+bool encode_halo_maps_tile(const lbm_domain* d, HaloMaps& out) {
     const lbm_params& P = d->prm;
-    if (d->fp64) return false;
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     const int D = Tl::D;
     const cuuint64_t dims[4] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny, (cuuint64_t)P.nz, (cuuint64_t)D};
-    const cuuint64_t strides[3] = {(cuuint64_t)d->lay.px * 4, (cuuint64_t)d->lay.px * P.ny * 4,
-                                   (cuuint64_t)d->lay.plane * 4};
+    const cuuint64_t es = d->lay.elem;
+    const cuuint64_t strides[3] = {d->lay.px * es, d->lay.px * es * P.ny, d->lay.plane * es};
+    const CUtensorMapDataType type = d->fp64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const cuuint32_t box[4] = {(cuuint32_t)Tl::HX, (cuuint32_t)Tl::HY, (cuuint32_t)Tl::HZ, (cuuint32_t)D};
     const cuuint32_t ones[4] = {1, 1, 1, 1};
     auto one = [&](CUtensorMap* m, void* base, cuuint32_t rank) {
-        return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank, base, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        return enc(m, type, rank, base, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    return one(&out[0], d->phi(), 3) && one(&out[1], d->U(0), 4) && one(&out[2], d->U(1), 4);
+    return one(&out.phi[0], d->phi(0), 3) && one(&out.phi[1], d->phi(1), 3) && one(&out.u[0], d->U(0), 4) &&
+           one(&out.u[1], d->U(1), 4) && one(&out.flux, d->flux(), 4);
 }
 
 template <int Q, int V>
-bool encode_halo_maps(const lbm_domain* d, CUtensorMap out[3]) {
+bool encode_halo_maps(const lbm_domain* d, HaloMaps& out) {
     return encode_halo_maps_tile<Tile<Q, V>>(d, out);
 }
 
-template <int Q>
-bool make_pair_maps(lbm_domain* d) {
-    CUtensorMap m[3];
-    if (!encode_halo_maps_tile<PairTile<Q>>(d, m)) return false;
-    d->tm2_phi = m[0];
-    d->tm2_u[0] = m[1];
-    d->tm2_u[1] = m[2];
-    return true;
-}
-
+// The maps of the domain's own kernels.
 template <int Q>
 bool make_halo_maps(lbm_domain* d) {
-    CUtensorMap m[3];
-    if (!encode_halo_maps<Q, 0>(d, m)) return false;
-    d->tm_phi = m[0];
-    d->tm_u[0] = m[1];
-    d->tm_u[1] = m[2];
-    return true;
+    if (d->cfg.pair) return encode_halo_maps_tile<PairTile<Q>>(d, d->maps);
+    return d->fp64 ? encode_halo_maps<Q, kSingleTile<double>>(d, d->maps)
+                   : encode_halo_maps<Q, kSingleTile<float>>(d, d->maps);
 }
 
 // The maps of tile shape V for a domain of lattice Q (the batch's tables).
-bool encode_halo_maps_any(const lbm_domain* d, int V, CUtensorMap out[3]) {
+bool encode_halo_maps_any(const lbm_domain* d, int V, HaloMaps& out) {
     if (d->prm.lattice == 9) {
         switch (V) {
         case 0: return encode_halo_maps<9, 0>(d, out);
@@ -730,6 +735,12 @@ lbm_status check_err_flag(lbm_domain* d) {
     if (h & kErrBounds)
         return fail(d, LBM_ERR_BOUNDS, "a step kernel computed an index outside its array (access skipped)");
     if (h) return fail(d, LBM_ERR_UNSTABLE, "a step produced a non-finite velocity");
+    return LBM_OK;
+}
+
+// The color was set: nothing is left below its last place.
+lbm_status clear_phi_lo(lbm_domain* d) {
+    if (!d->fp64) CUDA_TRY(d, cudaMemsetAsync(d->phi_lo(), 0, (size_t)d->lay.plane * d->lay.elem, d->stream));
     return LBM_OK;
 }
 
@@ -780,19 +791,34 @@ lbm_status init_state(lbm_domain* d, int mode, const double ctr[3], double R0) {
     // (init_pops) and the velocity of the first step's stencil, 0.  Population
     // slots of non-fluid nodes are never read (every pull of a fluid node reads
     // a fluid source or the node's own slots, as the diagnostics and state
-    // transfer do), the second velocity buffer is written at every fluid node
-    // by the first step, and the velocity of non-fluid nodes stays 0 from the
+    // transfer do), the second velocity and color buffers and the flux are written
+    // at every fluid node by the first step, and the velocity of non-fluid nodes stays 0 from the
     // domain's creation (no kernel writes it but as 0).  So of the state only
     // the first velocity buffer and p (state read back as 0 before a step) are
     // cleared.
     CUDA_TRY(d, cudaMemsetAsync(d->errflag(), 0, sizeof(int), d->stream));
     CUDA_TRY(d, cudaMemsetAsync(d->U(0), 0, (size_t)L.D * L.plane * L.elem, d->stream));
     CUDA_TRY(d, cudaMemsetAsync(d->p(), 0, (size_t)L.plane * L.elem, d->stream));
+    lbm_status st = clear_phi_lo(d);
+    if (st != LBM_OK) return st;
     dispatch(d, [&](auto Lx) {
-        decltype(Lx)::init_phi(d->cfg, d->cls(), d->phi(), mode, ctr, R0, ghost_value, d->stream);
-        decltype(Lx)::init_pops(d->cfg, d->cls(), d->phi(), d->N(0), d->B(0), d->stream);
+        decltype(Lx)::init_phi(d->cfg, d->cls(), d->phi(0), mode, ctr, R0, ghost_value, d->stream);
+        decltype(Lx)::init_pops(d->cfg, d->cls(), d->phi(0), d->N(0), d->B(), d->stream);
+    });
+    d->b_stored = true;
+    CUDA_TRY(d, cudaGetLastError());
+    return LBM_OK;
+}
+
+// Makes the buffer B() hold the current B.  After a step it follows from the
+// color that step read (the other color buffer), its N* and its flux.
+lbm_status store_B(lbm_domain* d) {
+    if (d->b_stored) return LBM_OK;
+    dispatch(d, [&](auto Lx) {
+        decltype(Lx)::rebuild_B(d->cfg, d->cls(), d->phi(1 - d->cur), d->N(d->cur), d->flux(), d->B(), d->stream);
     });
     CUDA_TRY(d, cudaGetLastError());
+    d->b_stored = true;
     return LBM_OK;
 }
 
@@ -975,7 +1001,6 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     const char* halo_copy = std::getenv("LBM_HALO_COPY");
     const bool elements_only = halo_copy && std::strcmp(halo_copy, "elements") == 0;
     d->tma = !elements_only && (P.lattice == 9 ? make_halo_maps<9>(d) : make_halo_maps<19>(d));
-    d->tma2 = !elements_only && (P.lattice == 9 ? make_pair_maps<9>(d) : make_pair_maps<19>(d));
     // upload the row bit masks (into the staging planes, 2 W bytes per row
     // against their 8 px) and the ghost table; the node classes and the
     // bounce-back mask are built from them on the device, with the padded row
@@ -985,13 +1010,14 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     uint64_t* dF = d->at<uint64_t>(L.off_stage);
     uint64_t* dG = dF + d->fluid_bits.size();
     if (2 * bits_bytes > 2 * (size_t)L.plane * L.elem) return bail("row bit masks do not fit the staging planes");
-    // zero the fields from phi on (u must stay 0 at non-fluid nodes); the
-    // population buffers are left as they are: lbm_init_* writes every fluid
+    // zero the fields from the first color on (u must stay 0 at non-fluid
+    // nodes); the flux and the second color are written by the first step
+    // before anything reads them, and the population buffers are left as they are: lbm_init_* writes every fluid
     // node's slots of the first ones, the first step those of the second ones,
     // and no pull of a fluid node reads a non-fluid node's slots (the step
     // kernels load them for non-fluid lanes, whose results are never stored
     // as state: u and p get 0 there, the populations values nothing reads)
-    if (cudaMemsetAsync(d->ws + L.off_phi, 0, L.total - L.off_phi, s) != cudaSuccess)
+    if (cudaMemsetAsync(d->ws + L.off_phi[0], 0, L.total - L.off_phi[0], s) != cudaSuccess)
         return bail("cudaMemset failed");
     if (cudaMemcpyAsync(dF, d->fluid_bits.data(), bits_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(dG, d->ghost_bits.data(), bits_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
@@ -1035,7 +1061,7 @@ lbm_status lbm_init_droplet(lbm_domain* d, const double centre[3], double R0) {
 lbm_status lbm_init_phi(lbm_domain* d, const double* phi_host) {
     if (!d || !phi_host) return fail(d, LBM_ERR_ARG, "NULL argument");
     if (d->poisoned) return fail(d, LBM_ERR_TIMEOUT, kPoisonedMsg);
-    lbm_status st = upload(d, d->phi(), phi_host, d->lay.nn_dense);
+    lbm_status st = upload(d, d->phi(0), phi_host, d->lay.nn_dense);
     if (st != LBM_OK) return st;
     const double zero[3] = {0, 0, 0};
     return init_state(d, 1, zero, 1.0);
@@ -1045,6 +1071,7 @@ lbm_status lbm_step(lbm_domain* d, int64_t n) {
     if (!d) return fail(d, LBM_ERR_ARG, "NULL domain");
     if (n < 0) return fail(d, LBM_ERR_ARG, "n must be >= 0");
     if (d->poisoned) return fail(d, LBM_ERR_TIMEOUT, kPoisonedMsg);
+    if (n > 0) d->b_stored = false;
     while (n > 0) {
         if (d->cur == 0 && n >= GRAPH_STEPS) {
             CUDA_TRY(d, cudaGraphLaunch(d->g8, d->stream));
@@ -1067,6 +1094,7 @@ lbm_status lbm_profile_steps(lbm_domain* d, int64_t n, double kernel_ms[3]) {
     cudaEvent_t ev[4];
     for (int k = 0; k < 4; ++k) CUDA_TRY(d, cudaEventCreate(&ev[k]));
     lbm_status st = LBM_OK;
+    d->b_stored = false;
     for (int64_t t = 0; t < n && st == LBM_OK; ++t) {
         launch_one_step(d, d->cur, d->stream, ev);
         cudaError_t e = cudaGetLastError();
@@ -1105,7 +1133,7 @@ lbm_status lbm_diagnostics(lbm_domain* d, const lbm_probe* probe, lbm_diag* out)
     double* partial = d->at<double>(L.off_partial);
     double* dout = d->at<double>(L.off_dout);
     dispatch(d, [&](auto Lx) {
-        decltype(Lx)::diag(d->cfg, d->mask(), d->N(d->cur), d->phi(), d->U(d->cur), d->p(), pr, partial, dout,
+        decltype(Lx)::diag(d->cfg, d->mask(), d->N(d->cur), d->phi(d->cur), d->U(d->cur), d->p(), pr, partial, dout,
                            d->stream);
     });
     CUDA_TRY(d, cudaGetLastError());
@@ -1170,7 +1198,11 @@ lbm_status lbm_read_state(lbm_domain* d, int32_t field, double* host_out) {
     case LBM_FIELD_N:
     case LBM_FIELD_B: {
         const bool is_b = field == LBM_FIELD_B;
-        void* st = is_b ? d->B(d->cur) : d->N(d->cur);
+        if (is_b) {
+            lbm_status r = store_B(d);
+            if (r != LBM_OK) return r;
+        }
+        void* st = is_b ? d->B() : d->N(d->cur);
         void* stage = d->at<void>(L.off_stage);
         for (int i = 0; i < L.Q; ++i) {
             double base = 0.0;
@@ -1188,7 +1220,7 @@ lbm_status lbm_read_state(lbm_domain* d, int32_t field, double* host_out) {
         return LBM_OK;
     }
     case LBM_FIELD_PHI:
-        return download(d, host_out, d->phi(), nn);
+        return download(d, host_out, d->phi(d->cur), nn);
     case LBM_FIELD_U: {
         for (int a = 0; a < 3; ++a) {
             if (a < L.D) {
@@ -1215,7 +1247,13 @@ lbm_status lbm_write_state(lbm_domain* d, int32_t field, const double* host_in) 
     case LBM_FIELD_N:
     case LBM_FIELD_B: {
         const bool is_b = field == LBM_FIELD_B;
-        void* st = is_b ? d->B(d->cur) : d->N(d->cur);
+        if (is_b) {
+            d->b_stored = true;
+        } else {                                   // B follows from the N that is replaced here
+            lbm_status r = store_B(d);
+            if (r != LBM_OK) return r;
+        }
+        void* st = is_b ? d->B() : d->N(d->cur);
         char* stage = d->at<char>(L.off_stage);
         std::vector<double> dev_i((size_t)nn), dev_o((size_t)nn);
         for (int i = 0; i < L.Q; ++i) {
@@ -1239,8 +1277,10 @@ lbm_status lbm_write_state(lbm_domain* d, int32_t field, const double* host_in) 
         CUDA_TRY(d, cudaStreamSynchronize(d->stream));
         return LBM_OK;
     }
-    case LBM_FIELD_PHI:
-        return upload(d, d->phi(), host_in, nn);
+    case LBM_FIELD_PHI: {
+        lbm_status s = clear_phi_lo(d);
+        return s != LBM_OK ? s : upload(d, d->phi(d->cur), host_in, nn);
+    }
     case LBM_FIELD_U: {
         // the velocity of a non-fluid node is 0 whatever the caller passes: the
         // stencils read it there as the wall's velocity
@@ -1348,21 +1388,13 @@ struct lbm_batch {
     std::vector<int> cur0;             // each domain's buffer parity when the batch was made
     int parity = 0;                    // steps taken by the batch, mod 2
     int variant = 0;
-    // tiles of the color kernel, whatever shape the step kernels use (it has
-    // no halo): row chunks of 128 nodes (kPhiRows), which leave only the
-    // padding columns idle.  LBM_BATCH_PHI_SHAPE=step: the step's shape;
-    // =0..5: that shape (shape 3, 32 x 2 x 2, ran a batch of 64 domains of 48^3 to 128^3 at 3.305 ms per
-    // step against 3.331 on the step's 64-wide tiles).
-    int phi_shape = kPhiRows;
-    int4* phi_rows = nullptr;          // {slot, x0, y0, z} row chunks
-    int nphi_rows = 0;
     int ntiles[kTileVariants] = {};
     int ncontrast[kTileVariants] = {};           // tiles of domains with density contrast come first
     int device = 0;
     std::vector<int> slots;            // each domain's slot of the constant table
     char* dev = nullptr;               // one allocation for every device table
     int4* tiles[kTileVariants] = {};             // {slot, x0, y0, z0}
-    CUtensorMap* maps = nullptr;                 // [kTileVariants][kBatchSlots][3] halo maps by shape and slot
+    CUtensorMap* maps = nullptr;                 // [kTileVariants][kBatchSlots][kSlotMaps] halo maps by shape and slot
     void* ghost_tabs = nullptr;
     int64_t* ghost_begin = nullptr;
     int64_t total_ghosts = 0;
@@ -1427,12 +1459,9 @@ void batch_launch_step(lbm_batch* b, int parity, cudaStream_t s) {
     const int V = b->variant;
     bdispatch(b->precision, [&](auto Lx) {
         using L = decltype(Lx);
-        L::ghost_batched(b->GK, b->ghost_tabs, b->ghost_begin, (int)b->doms.size(), b->total_ghosts, s);
-        const int Vp = b->phi_shape < 0 ? V : b->phi_shape;
-        const int4* pt = Vp == kPhiRows ? b->phi_rows : b->tiles[Vp];
-        const int np = Vp == kPhiRows ? b->nphi_rows : b->ntiles[Vp];
-        L::step_phi_batched(b->Q, V, b->tiles[V], b->maps + (size_t)V * kBatchSlots * 3, b->ntiles[V],
-                            b->ncontrast[V], Vp, pt, np, parity, s);
+        L::ghost_batched(b->GK, b->ghost_tabs, b->ghost_begin, (int)b->doms.size(), b->total_ghosts, parity, s);
+        L::step_color_batched(b->Q, V, b->tiles[V], b->maps + (size_t)V * kBatchSlots * kSlotMaps, b->ntiles[V],
+                              b->ncontrast[V], parity, s);
     });
 }
 
@@ -1489,11 +1518,6 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         b->cur0.push_back(doms[i]->cur);
     }
     b->stream = (cudaStream_t)cuda_stream;
-    const char* phi_shape = std::getenv("LBM_BATCH_PHI_SHAPE");
-    if (phi_shape && std::strcmp(phi_shape, "step") == 0) b->phi_shape = -1;
-    else if (phi_shape && std::strcmp(phi_shape, "rows") == 0) b->phi_shape = kPhiRows;
-    else if (phi_shape && phi_shape[0] >= '0' && phi_shape[0] < '0' + kTileVariants && !phi_shape[1])
-        b->phi_shape = phi_shape[0] - '0';
     if (n > kBatchSlots) {
         delete b;
         return bfail(nullptr, LBM_ERR_ARG, "a batch holds at most " + std::to_string(kBatchSlots) + " domains");
@@ -1511,22 +1535,25 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         using L = decltype(Lx);
         esz = L::entry_size(); gsz = L::ghost_table_size();
     });
-    // halo maps by tile shape and slot: phi, then u_in of step parity 0 and 1
-    // (u_in = U(cur0 ^ parity)), each with the box of that shape's halo tile
-    std::vector<CUtensorMap> hm((size_t)kTileVariants * kBatchSlots * 3);
+    // halo maps by tile shape and slot: the color and u_in of step parity 0 and
+    // 1 (buffers cur0 ^ parity), then the flux, each with the box of that
+    // shape's halo tile
+    std::vector<CUtensorMap> hm((size_t)kTileVariants * kBatchSlots * kSlotMaps);
     std::vector<char> slot_tma(kBatchSlots, 0);
     for (int i = 0; i < n; ++i) {
         lbm_domain* d = b->doms[i];
         if (!d->tma) continue;
-        const int sl = b->slots[i];
+        const int sl = b->slots[i], c0 = b->cur0[i];
         bool ok = true;
         for (int V = 0; V < kTileVariants && ok; ++V) {
-            CUtensorMap m[3];
+            HaloMaps m;
             ok = encode_halo_maps_any(d, V, m);
-            CUtensorMap* dst = &hm[((size_t)V * kBatchSlots + sl) * 3];
-            dst[0] = m[0];
-            dst[1] = m[1 + b->cur0[i]];
-            dst[2] = m[1 + (b->cur0[i] ^ 1)];
+            CUtensorMap* dst = &hm[((size_t)V * kBatchSlots + sl) * kSlotMaps];
+            dst[0] = m.phi[c0];
+            dst[1] = m.phi[c0 ^ 1];
+            dst[2] = m.u[c0];
+            dst[3] = m.u[c0 ^ 1];
+            dst[4] = m.flux;
         }
         slot_tma[sl] = ok;                       // a slot uses its maps only if every shape's encoded
     }
@@ -1539,15 +1566,11 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         bdispatch(b->precision, [&](auto Lx) {
             using LL = decltype(Lx);
             StepPtrs sp[2];
-            for (int k = 0; k < 2; ++k) {
-                const int c = b->cur0[i] ^ k;
-                sp[k].Nin = d->N(c); sp[k].Bin = d->B(c); sp[k].Nout = d->N(1 - c); sp[k].Bout = d->B(1 - c);
-                sp[k].phi = d->phi(); sp[k].u_in = d->U(c); sp[k].u_out = d->U(1 - c); sp[k].p = d->p();
-                sp[k].mask = d->mask(); sp[k].err = d->errflag();
-            }
+            for (int k = 0; k < 2; ++k) sp[k] = step_ptrs(d, b->cur0[i] ^ k);
+            void* const phi[2] = {d->phi(b->cur0[i]), d->phi(b->cur0[i] ^ 1)};
             LL::fill_entry(&he[esz * i], d->cfg, sp, slot_tma[b->slots[i]] != 0);
             LL::fill_ghost_table(&hg[gsz * i], d->ng, d->at<int32_t>(L.off_gnode), d->at<int32_t>(L.off_gcorner),
-                                 d->at<void>(L.off_gwt), d->cfg.exp_eps, d->cfg.eps, d->phi(), d->cfg.ghost_rule,
+                                 d->at<void>(L.off_gwt), d->cfg.exp_eps, d->cfg.eps, phi, d->cfg.ghost_rule,
                                  L.plane, d->errflag());
         });
         gbegin[i + 1] = gbegin[i] + d->ng;
@@ -1561,15 +1584,6 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
                 if (pass == 0) b->ncontrast[V] = (int)tiles[V].size();
             }
         }
-    // row chunks of the color kernel, domain by domain, plane by plane
-    std::vector<int4> rows;
-    for (int i = 0; i < n; ++i) {
-        const lbm_params& P = b->doms[i]->prm;
-        const int64_t px = b->doms[i]->lay.px, per_plane = px * P.ny;
-        for (int z = 0; z < P.nz; ++z)
-            for (int64_t o = 0; o < per_plane; o += kPhiChunk)
-                rows.push_back(make_int4(b->slots[i], (int)(o % px), (int)(o / px), z));
-    }
     b->total_ghosts = gbegin[n];
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t r = off; off = round_up(off + bytes, 256); return r; };
@@ -1583,11 +1597,6 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         }
         o_t[V] = take(tiles[V].size() * sizeof(int4));
     }
-    if (rows.size() > (size_t)INT32_MAX) {
-        lbm_batch_destroy(b);
-        return bfail(nullptr, LBM_ERR_ARG, "too many tiles");
-    }
-    const size_t o_r = take(rows.size() * sizeof(int4));
     if (cudaMalloc((void**)&b->dev, off) != cudaSuccess) {
         cudaGetLastError();
         lbm_batch_destroy(b);
@@ -1605,11 +1614,6 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         b->tiles[V] = (int4*)(b->dev + o_t[V]);
         b->ntiles[V] = (int)tiles[V].size();
         e = cudaMemcpy(b->tiles[V], tiles[V].data(), tiles[V].size() * sizeof(int4), cudaMemcpyHostToDevice);
-    }
-    if (e == cudaSuccess) {
-        b->phi_rows = (int4*)(b->dev + o_r);
-        b->nphi_rows = (int)rows.size();
-        e = cudaMemcpy(b->phi_rows, rows.data(), rows.size() * sizeof(int4), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
@@ -1646,6 +1650,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
     for (auto* d : b->doms) {
         d->step += n;
         if (n & 1) d->cur ^= 1;
+        if (n > 0) d->b_stored = false;
     }
     return LBM_OK;
 }
@@ -1696,7 +1701,11 @@ lbm_status lbm_batch_tune(lbm_batch* b, int32_t steps_per_trial, int32_t* chosen
         if (ms_per_step) ms_per_step[V] = per;
         if (per < best) { best = per; best_v = V; }
         const int64_t taken = steps_per_trial + 1;
-        for (auto* d : b->doms) { d->step += taken; if (taken & 1) d->cur ^= 1; }
+        for (auto* d : b->doms) {
+            d->step += taken;
+            d->b_stored = false;
+            if (taken & 1) d->cur ^= 1;
+        }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

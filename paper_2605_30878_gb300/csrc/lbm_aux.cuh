@@ -161,8 +161,40 @@ __global__ void k_init_pops(Dims d, StepParams<T> P, const uint8_t* __restrict__
             // stored one; B_i - chi_i(stored)/2 = phi (that) + (phi - 1/2) chi_i(stored)
             const T e = P.chi_err[i == 0 ? 0 : (L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) + L::cz(i) * L::cz(i) == 1
                                                     ? 1 : 2)];
-            pop_store<S, T>(Nst, i, pl, nd, kShift ? e : P.chi[i], kScaleN);
-            pop_store<S, T>(Bst, i, pl, nd, PopStore<S>::kShiftB ? (ph - T(0.5)) * P.chi[i] + ph * e : ph * P.chi[i], kScaleB);
+            pop_store<Q, S, T>(Nst, i, pl, nd, kShift ? e : P.chi[i], kScaleN);
+            pop_store<Q, S, T>(Bst, i, pl, nd, PopStore<S>::kShiftB ? (ph - T(0.5)) * P.chi[i] + ph * e : ph * P.chi[i], kScaleB);
+        }
+    }
+}
+
+// The populations B* of the last step in storage form, for state transfer: the
+// step keeps only what makes them, B*_i = phi N*_i + w_i c_i . f (phi the color
+// that step read).  With FP16 storage the float rest population takes the node
+// total phi - 1/2 less the rounded moving ones.
+template <int Q, typename T, typename S>
+__global__ void k_rebuild_B(Dims d, StepParams<T> P, const uint8_t* __restrict__ cls, const T* __restrict__ phi,
+                            const S* __restrict__ Nst, const T* __restrict__ flux, S* __restrict__ Bst) {
+    using L = Lattice<Q>;
+    using PS = PopStore<S>;
+    const int nn = (int)padded_nodes(d), pl = (int)d.plane;
+    for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < nn; node += gridDim.x * blockDim.x) {
+        if (cls[node] != CLS_FLUID) continue;
+        const T ph = phi[node], base = PS::kShiftB ? ph - T(0.5) : ph;      // chi_i's factor
+        T sum = T(0);
+#pragma unroll
+        for (int i = Q - 1; i >= 0; --i) {
+            T b = base * P.chi[i] + ph * pop_load<Q, S, T>(Nst, i, pl, node, kScaleN);
+            if (i > 0) {
+                T cf = T(0);
+                if (L::cx(i)) cf += T(L::cx(i)) * flux[node];
+                if (L::cy(i)) cf += T(L::cy(i)) * flux[pl + node];
+                if (L::D == 3 && L::cz(i)) cf += T(L::cz(i)) * flux[2 * pl + node];
+                b += T(L::w(i)) * cf;
+            } else if (!PS::kExact) {
+                b = base - sum;
+            }
+            pop_store<Q, S, T>(Bst, i, pl, node, b, kScaleB);
+            if (!PS::kExact && i > 0) sum += T(__half2float(__float2half_rn(float(b) * kScaleB)) / kScaleB);   // as stored
         }
     }
 }
@@ -181,7 +213,7 @@ __global__ void k_scatter_dir(Dims d, const uint8_t* __restrict__ cls, int i, co
         node_xyz(node, d, x, y, z);
         const int64_t dn = shifted(d, x, y, z, L::cx(i), L::cy(i), L::cz(i));
         const T v = (cls[dn] == CLS_FLUID) ? post_i[dn] : post_opp[node];
-        pop_store<S, T>(st, i, (int)d.plane, (int)node, v - base, scale);
+        pop_store<Q, S, T>(st, i, (int)d.plane, (int)node, v - base, scale);
     }
 }
 
@@ -199,7 +231,7 @@ __global__ void k_gather_dir(Dims d, const uint8_t* __restrict__ cls, int i, con
             node_xyz(node, d, x, y, z);
             const int64_t sn = shifted(d, x, y, z, -L::cx(i), -L::cy(i), -L::cz(i));
             const bool from_fluid = cls[sn] == CLS_FLUID;
-            v = base + pop_load<S, T>(st, from_fluid ? i : L::opp(i), (int)d.plane, (int)(from_fluid ? sn : node),
+            v = base + pop_load<Q, S, T>(st, from_fluid ? i : L::opp(i), (int)d.plane, (int)(from_fluid ? sn : node),
                                       scale);
         }
         post[node] = v;
@@ -275,7 +307,7 @@ __global__ void __launch_bounds__(DIAG_THREADS) k_diag_partial(Dims d, double rh
         for (int i = 0; i < Q; ++i) {
             const bool from_fluid = i == 0 || !((m >> i) & 1u);
             const int src = from_fluid ? node + W.off(-L::cx(i), -L::cy(i), -L::cz(i)) : node;
-            ps += pop_load<S, T>(Nst, from_fluid ? i : L::opp(i), pl, src, kScaleN);
+            ps += pop_load<Q, S, T>(Nst, from_fluid ? i : L::opp(i), pl, src, kScaleN);
         }
         acc[DG_POP] += PopStore<S>::kShift ? (double)ps + chi_total : (double)ps;
         T u2 = T(0);
