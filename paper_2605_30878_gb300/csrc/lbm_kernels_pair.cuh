@@ -254,11 +254,12 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
     constexpr bool kUnits = !PopStore<S>::kExact;
     int* const err = b.err;
     const bool interior = tm_phi != nullptr;
+    const PairNode pn(P, b.mask, x0, y0, z0, err);
+    pdl_wait();
     HaloFix<Tl, float, CONTRAST> fx;
     if (!halo_issue<Tl, float, CONTRAST>(P, b.phi, b.u_in, err, s_phi, s_u, x0, y0, z0, tm_phi, tm_u, bar, fx)) return;
 
     // the pair's populations, pulled while the halo is in flight
-    const PairNode pn(P, b.mask, x0, y0, z0, err);
     const bool fluidA = pn.fluidA, fluidB = pn.fluidB;
     const int nodeA = pn.nodeA, xa = pn.xa, y = pn.y, z = pn.z;
     float NA[Q], NB[Q];
@@ -298,9 +299,11 @@ __device__ __forceinline__ void color_pair_tile(const StepParams<float>& P, cons
     using PS = PopStore<S>;
     constexpr int D = L::D;
     int* const err = b.err;
+    const PairNode pn(P, b.mask, x0, y0, z0, err);
+    pdl_wait();
+    pdl_trigger();
     HaloFix<Tl, float, true> fx;
     if (!halo_issue<Tl, float, true>(P, b.phi, b.flux, err, s_phi, s_f, x0, y0, z0, tm_phi, tm_f, bar, fx)) return;
-    const PairNode pn(P, b.mask, x0, y0, z0, err);
     float NA[Q], NB[Q];
     pull_pair<Q, S>(P, b.Nout, pn, NA, NB, err);
     const S* const Ncst = b.Nout;
@@ -411,8 +414,10 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
     const BatchEntry<float, S>& e = c_batch<float, S>[idx_checked(t.x, kBatchSlots, c_batch<float, S>[0].b[0].err)];
     const int y0 = t.z, z0 = t.w;
     if (kDebugBounds && !(idx_ok(t.y, e.P.nx, e.b[0].err) && idx_ok(y0, e.P.ny, e.b[0].err) &&
-                          idx_ok(z0, e.P.nz, e.b[0].err)))
+                          idx_ok(z0, e.P.nz, e.b[0].err))) {
+        pdl_wait();
         return;                                         // a tile outside its domain
+    }
     const bool tma = maps != nullptr && e.tma && y0 >= 1 && y0 + Tl::TY + 1 <= e.P.ny &&
                      (D == 2 || (z0 >= 1 && z0 + Tl::TZ + 1 <= e.P.nz));
     if (tma) {
@@ -436,8 +441,10 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, (ColorBlocks<P
     const BatchEntry<float, S>& e = c_batch<float, S>[idx_checked(t.x, kBatchSlots, c_batch<float, S>[0].b[0].err)];
     const int y0 = t.z, z0 = t.w;
     if (kDebugBounds && !(idx_ok(t.y, e.P.nx, e.b[0].err) && idx_ok(y0, e.P.ny, e.b[0].err) &&
-                          idx_ok(z0, e.P.nz, e.b[0].err)))
+                          idx_ok(z0, e.P.nz, e.b[0].err))) {
+        pdl_wait();
         return;                                         // a tile outside its domain
+    }
     const bool tma = maps != nullptr && e.tma && y0 >= 1 && y0 + Tl::TY + 1 <= e.P.ny &&
                      (D == 2 || (z0 >= 1 && z0 + Tl::TZ + 1 <= e.P.nz));
     if (tma) {

@@ -26,6 +26,23 @@ inline void chi_for_float(const double* chi, double* out) {
     out[0] = rest;
 }
 
+// Launches a kernel of the step chain with programmatic stream serialization:
+// it may start before the work in front of it on the stream has finished, and
+// waits for it in pdl_wait().
+template <typename... Params, typename... Args>
+void launch_pdl(void (*kernel)(Params...), dim3 grid, dim3 block, cudaStream_t s, Args&&... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 template <typename T, typename S>
 StepParams<T> Launch<T, S>::params(const StepConfig& c) {
     StepParams<T> P;
@@ -102,17 +119,17 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s
             using Tl = PairTile<Q>;
             const dim3 block(Tl::BX, Tl::TY, Tl::TZ);
             if (c.contrast)
-                k_step_pair<Q, S, true><<<pair_grid<Q>(c.d), block, 0, s>>>(P, b, tm_phi, tm_u, tma);
+                launch_pdl(k_step_pair<Q, S, true>, pair_grid<Q>(c.d), block, s, P, b, tm_phi, tm_u, tma);
             else
-                k_step_pair<Q, S, false><<<pair_grid<Q>(c.d), block, 0, s>>>(P, b, tm_phi, tm_u, tma);
+                launch_pdl(k_step_pair<Q, S, false>, pair_grid<Q>(c.d), block, s, P, b, tm_phi, tm_u, tma);
             return;
         }
     }
     constexpr int V = kSingleTile<T>;
     if (c.contrast)
-        k_step<Q, T, S, true, V><<<step_grid<Q, V>(c.d), step_block<Q, V>(), 0, s>>>(P, b, tm_phi, tm_u, tma);
+        launch_pdl(k_step<Q, T, S, true, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma);
     else
-        k_step<Q, T, S, false, V><<<step_grid<Q, V>(c.d), step_block<Q, V>(), 0, s>>>(P, b, tm_phi, tm_u, tma);
+        launch_pdl(k_step<Q, T, S, false, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma);
 }
 
 template <typename T, typename S>
@@ -134,12 +151,12 @@ void Launch<T, S>::color_q(const StepConfig& c, const StepPtrs& p, cudaStream_t 
     if constexpr (sizeof(T) == 4) {
         if (c.pair) {
             using Tl = PairTile<Q>;
-            k_color_pair<Q, S><<<pair_grid<Q>(c.d), dim3(Tl::BX, Tl::TY, Tl::TZ), 0, s>>>(P, b, tm_phi, tm_f, tma);
+            launch_pdl(k_color_pair<Q, S>, pair_grid<Q>(c.d), dim3(Tl::BX, Tl::TY, Tl::TZ), s, P, b, tm_phi, tm_f, tma);
             return;
         }
     }
     constexpr int V = kSingleTile<T>;
-    k_color<Q, T, S, V><<<step_grid<Q, V>(c.d), step_block<Q, V>(), 0, s>>>(P, b, tm_phi, tm_f, tma);
+    launch_pdl(k_color<Q, T, S, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_f, tma);
 }
 
 template <typename T, typename S>
@@ -154,10 +171,10 @@ void Launch<T, S>::ghost(int GK, int rule, int64_t ng, const int32_t* node, cons
     const unsigned blocks = (unsigned)((ng + 255) / 256);
     const T* w = (const T*)wt;
     T* f = (T*)phi;
-    if (GK == 4 && rule == 0) k_ghost<4, T, 0><<<blocks, 256, 0, s>>>(ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
-    if (GK == 4 && rule == 1) k_ghost<4, T, 1><<<blocks, 256, 0, s>>>(ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
-    if (GK == 8 && rule == 0) k_ghost<8, T, 0><<<blocks, 256, 0, s>>>(ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
-    if (GK == 8 && rule == 1) k_ghost<8, T, 1><<<blocks, 256, 0, s>>>(ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
+    if (GK == 4 && rule == 0) launch_pdl(k_ghost<4, T, 0>, blocks, 256, s, ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
+    if (GK == 4 && rule == 1) launch_pdl(k_ghost<4, T, 1>, blocks, 256, s, ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
+    if (GK == 8 && rule == 0) launch_pdl(k_ghost<8, T, 0>, blocks, 256, s, ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
+    if (GK == 8 && rule == 1) launch_pdl(k_ghost<8, T, 1>, blocks, 256, s, ng, node, corner, w, (T)exp_eps, (T)eps, f, plane, err);
 }
 
 template <typename T, typename S>
@@ -264,15 +281,15 @@ void Launch<T, S>::step_batched_v(const int4* tiles, const CUtensorMap* maps, in
         static_assert(Pt::TX == Tl::TX && Pt::TY == Tl::TY && Pt::TZ == Tl::TZ, "the pair tile covers the shape's tile");
         const dim3 pblock(Pt::BX, Pt::TY, Pt::TZ);
         if (ncontrast > 0)
-            k_step_pair_batched<Qc, S, true, TXn, TYn><<<ncontrast, pblock, 0, s>>>(tiles, maps, parity);
+            launch_pdl(k_step_pair_batched<Qc, S, true, TXn, TYn>, ncontrast, pblock, s, tiles, maps, parity);
         if (ntiles > ncontrast)
-            k_step_pair_batched<Qc, S, false, TXn, TYn><<<ntiles - ncontrast, pblock, 0, s>>>(tiles + ncontrast,
+            launch_pdl(k_step_pair_batched<Qc, S, false, TXn, TYn>, ntiles - ncontrast, pblock, s, tiles + ncontrast,
                                                                                              maps, parity);
     } else {
         if (ncontrast > 0)
-            k_step_batched<Qc, T, S, V, true><<<ncontrast, block, 0, s>>>(tiles, maps, parity);
+            launch_pdl(k_step_batched<Qc, T, S, V, true>, ncontrast, block, s, tiles, maps, parity);
         if (ntiles > ncontrast)
-            k_step_batched<Qc, T, S, V, false><<<ntiles - ncontrast, block, 0, s>>>(tiles + ncontrast, maps,
+            launch_pdl(k_step_batched<Qc, T, S, V, false>, ntiles - ncontrast, block, s, tiles + ncontrast, maps,
                                                                                     parity);
     }
 }
@@ -284,9 +301,9 @@ void Launch<T, S>::color_batched_v(const int4* tiles, const CUtensorMap* maps, i
     if constexpr ((V == 5 || V == 3 || V == 0) && sizeof(T) == 4) {
         constexpr int TXn = Tl::TX, TYn = Tl::TY;
         using Pt = PairTile<Qc, TXn, TYn>;
-        k_color_pair_batched<Qc, S, TXn, TYn><<<ntiles, dim3(Pt::BX, Pt::TY, Pt::TZ), 0, s>>>(tiles, maps, parity);
+        launch_pdl(k_color_pair_batched<Qc, S, TXn, TYn>, ntiles, dim3(Pt::BX, Pt::TY, Pt::TZ), s, tiles, maps, parity);
     } else {
-        k_color_batched<Qc, T, S, V><<<ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), 0, s>>>(tiles, maps, parity);
+        launch_pdl(k_color_batched<Qc, T, S, V>, ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), s, tiles, maps, parity);
     }
 }
 
@@ -333,8 +350,8 @@ void Launch<T, S>::ghost_batched(int GK, const void* tabs, const int64_t* begin,
                                  cudaStream_t s) {
     if (total == 0) return;
     const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (GK == 4) k_ghost_batched<4, T><<<blocks, 256, 0, s>>>((const GhostTable<T>*)tabs, begin, ndom, total, parity);
-    else k_ghost_batched<8, T><<<blocks, 256, 0, s>>>((const GhostTable<T>*)tabs, begin, ndom, total, parity);
+    if (GK == 4) launch_pdl(k_ghost_batched<4, T>, blocks, 256, s, (const GhostTable<T>*)tabs, begin, ndom, total, parity);
+    else launch_pdl(k_ghost_batched<8, T>, blocks, 256, s, (const GhostTable<T>*)tabs, begin, ndom, total, parity);
 }
 
 template <typename T, typename S>
