@@ -759,15 +759,111 @@ lbm_status upload_as(lbm_domain* d, void* dst, const double* src) {
     return LBM_OK;
 }
 
+// Pinned memory that fields are read back through, two halves of kHalf bytes
+// per device, made on first use and kept: a copy into it runs at the link's
+// rate and beside the conversion of the half before, and neither pages of a
+// fresh buffer nor the driver's own staging cost anything.  One read uses it at
+// a time; lbm_release_cached_memory gives it back.
+struct ReadStage {
+    static constexpr size_t kHalf = (size_t)4 << 20;
+    std::mutex use;
+    char* half[2] = {nullptr, nullptr};
+    cudaEvent_t landed[2] = {nullptr, nullptr};
+    bool ready() {
+        if (half[0]) return true;
+        void* p = nullptr;
+        if (cudaHostAlloc(&p, 2 * kHalf, cudaHostAllocPortable) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        for (auto& e : landed)
+            if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
+                cudaGetLastError();
+                release_events();
+                cudaFreeHost(p);
+                return false;
+            }
+        half[0] = (char*)p;
+        half[1] = half[0] + kHalf;
+        return true;
+    }
+    void release_events() {
+        for (auto& e : landed) {
+            if (e) cudaEventDestroy(e);
+            e = nullptr;
+        }
+    }
+    void release() {
+        std::lock_guard<std::mutex> lk(use);
+        if (!half[0]) return;
+        release_events();
+        cudaFreeHost(half[0]);
+        half[0] = half[1] = nullptr;
+    }
+};
+std::mutex g_stage_mutex;
+std::map<int, std::unique_ptr<ReadStage>> g_stages;
+ReadStage& read_stage() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(g_stage_mutex);
+    auto& s = g_stages[dev];
+    if (!s) s.reset(new ReadStage());
+    return *s;
+}
+
+// `planes` whole fields, src_step elements apart on the device (rows padded to
+// px), into dense host arrays of doubles one after the other.
 template <typename V>
-lbm_status download_as(lbm_domain* d, double* dst, const void* src) {
+lbm_status download_as(lbm_domain* d, double* dst, const V* src, int planes, int64_t src_step) {
     const Layout& L = d->lay;
-    const int64_t nx = d->prm.nx, rows = L.nn_dense / nx;
-    std::vector<V> tmp((size_t)L.nn);
-    CUDA_TRY(d, cudaMemcpyAsync(tmp.data(), src, tmp.size() * sizeof(V), cudaMemcpyDeviceToHost, d->stream));
-    CUDA_TRY(d, cudaStreamSynchronize(d->stream));
-    for (int64_t r = 0; r < rows; ++r)
-        for (int64_t x = 0; x < nx; ++x) dst[r * nx + x] = (double)tmp[(size_t)(r * L.px + x)];
+    const int64_t nx = d->prm.nx, px = L.px, rows = L.nn_dense / nx;
+    const int64_t row_bytes = px * (int64_t)sizeof(V);
+    ReadStage& st = read_stage();
+    std::lock_guard<std::mutex> one_read(st.use);
+    if (row_bytes > (int64_t)ReadStage::kHalf || !st.ready()) {
+        std::vector<V> tmp((size_t)L.nn);
+        for (int a = 0; a < planes; ++a) {
+            CUDA_TRY(d, cudaMemcpyAsync(tmp.data(), src + a * src_step, tmp.size() * sizeof(V), cudaMemcpyDeviceToHost,
+                                        d->stream));
+            CUDA_TRY(d, cudaStreamSynchronize(d->stream));
+            for (int64_t r = 0; r < rows; ++r)
+                for (int64_t x = 0; x < nx; ++x) dst[a * L.nn_dense + r * nx + x] = (double)tmp[(size_t)(r * px + x)];
+        }
+        return LBM_OK;
+    }
+    // pieces of whole rows, one plane after the other
+    const int64_t piece = std::min<int64_t>(rows, (int64_t)ReadStage::kHalf / row_bytes);
+    const int64_t per_plane = (rows + piece - 1) / piece, n = per_plane * planes;
+    auto first_row = [&](int64_t k) { return (k % per_plane) * piece; };
+    auto row_count = [&](int64_t k) { return std::min(piece, rows - first_row(k)); };
+    auto copy = [&](int64_t k) {
+        cudaError_t e = cudaMemcpyAsync(st.half[k & 1], src + (k / per_plane) * src_step + first_row(k) * px,
+                                        (size_t)(row_count(k) * row_bytes), cudaMemcpyDeviceToHost, d->stream);
+        return e == cudaSuccess ? cudaEventRecord(st.landed[k & 1], d->stream) : e;
+    };
+    cudaError_t e = copy(0);
+    for (int64_t k = 0; k < n && e == cudaSuccess; ++k) {
+        if (k + 1 < n) e = copy(k + 1);
+        if (e == cudaSuccess) e = cudaEventSynchronize(st.landed[k & 1]);
+        if (e != cudaSuccess) break;
+        const V* const from = (const V*)st.half[k & 1];
+        double* const to = dst + (k / per_plane) * L.nn_dense + first_row(k) * nx;
+        // rows over host threads, 32k nodes each at least (waking them costs ~10 us)
+        parallel_chunks(row_count(k), std::max<int64_t>(1, ((int64_t)1 << 15) / nx), [&](int64_t r0, int64_t r1, int) {
+            if (px == nx) {
+                if (sizeof(V) == sizeof(double)) std::memcpy(to + r0 * nx, from + r0 * nx, (size_t)((r1 - r0) * nx) * sizeof(V));
+                else for (int64_t k = r0 * nx; k < r1 * nx; ++k) to[k] = (double)from[k];
+                return;
+            }
+            for (int64_t r = r0; r < r1; ++r)
+                for (int64_t x = 0; x < nx; ++x) to[r * nx + x] = (double)from[r * px + x];
+        });
+    }
+    if (e != cudaSuccess) {
+        cudaStreamSynchronize(d->stream);            // no copy is left on its way into the stage
+        return fail(d, LBM_ERR_CUDA, std::string("reading a field: ") + cudaGetErrorString(e));
+    }
     return LBM_OK;
 }
 
@@ -777,9 +873,10 @@ lbm_status upload(lbm_domain* d, void* dst, const double* src, size_t count) {
     return d->fp64 ? upload_as<double>(d, dst, src) : upload_as<float>(d, dst, src);
 }
 
-lbm_status download(lbm_domain* d, double* dst, const void* src, size_t count) {
-    if ((int64_t)count != d->lay.nn_dense) return fail(d, LBM_ERR_ARG, "field size mismatch");
-    return d->fp64 ? download_as<double>(d, dst, src) : download_as<float>(d, dst, src);
+lbm_status download(lbm_domain* d, double* dst, const void* src, int planes = 1) {
+    const int64_t step = d->lay.plane;
+    return d->fp64 ? download_as(d, dst, (const double*)src, planes, step)
+                   : download_as(d, dst, (const float*)src, planes, step);
 }
 
 lbm_status init_state(lbm_domain* d, int mode, const double ctr[3], double R0) {
@@ -1212,7 +1309,7 @@ lbm_status lbm_read_state(lbm_domain* d, int32_t field, double* host_out) {
             });
             CUDA_TRY(d, cudaGetLastError());
             double* out = host_out + (size_t)i * nn;
-            lbm_status s = download(d, out, stage, nn);
+            lbm_status s = download(d, out, stage);
             if (s != LBM_OK) return s;
             if (base != 0.0)                       // deviations from the storage reference -> values, in double
                 for_fluid_nodes(d, [&](int64_t k) { out[k] += base; });
@@ -1220,20 +1317,13 @@ lbm_status lbm_read_state(lbm_domain* d, int32_t field, double* host_out) {
         return LBM_OK;
     }
     case LBM_FIELD_PHI:
-        return download(d, host_out, d->phi(d->cur), nn);
+        return download(d, host_out, d->phi(d->cur));
     case LBM_FIELD_U: {
-        for (int a = 0; a < 3; ++a) {
-            if (a < L.D) {
-                lbm_status s = download(d, host_out + (size_t)a * nn, (const char*)d->U(d->cur) + (size_t)a * L.plane * L.elem, nn);
-                if (s != LBM_OK) return s;
-            } else {
-                std::fill(host_out + (size_t)a * nn, host_out + (size_t)(a + 1) * nn, 0.0);
-            }
-        }
-        return LBM_OK;
+        if (L.D == 2) std::fill(host_out + 2 * nn, host_out + 3 * nn, 0.0);
+        return download(d, host_out, d->U(d->cur), L.D);
     }
     case LBM_FIELD_P:
-        return download(d, host_out, d->p(), nn);
+        return download(d, host_out, d->p());
     }
     return fail(d, LBM_ERR_ARG, "unknown field");
 }
@@ -1370,6 +1460,13 @@ lbm_status lbm_release_cached_memory(void) {
             cudaGetLastError();
             cudaSetDevice(cur);
             return LBM_ERR_CUDA;
+        }
+    }
+    {
+        std::lock_guard<std::mutex> ls(g_stage_mutex);
+        for (auto& kv : g_stages) {
+            cudaSetDevice(kv.first);
+            kv.second->release();
         }
     }
     cudaSetDevice(cur);

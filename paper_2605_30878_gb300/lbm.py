@@ -333,7 +333,7 @@ class Domain:
         return {"N": self.Q * self.nn, "B": self.Q * self.nn, "phi": self.nn, "u": 3 * self.nn, "p": self.nn}[field]
 
     def read(self, field):
-        out = np.zeros(self._count(field))
+        out = np.empty(self._count(field))                # every value is written
         _check(load().lbm_read_state(self.h, FIELDS[field], out.ctypes.data_as(_dp)), self.h)
         if field in ("N", "B"):
             return out.reshape(self.Q, self.nn)

@@ -79,3 +79,23 @@ def test_one_step_at_tile_edges(shape, ratio, precision):
             got = {f: mate.read(f) for f in want}
             for f in got:
                 assert np.array_equal(got[f], alone.read(f)), (v, f)
+
+
+@pytest.mark.parametrize("precision", [lbm.FP64, lbm.FP32])
+@pytest.mark.parametrize("shape", [(1, 1500, 1021), (3, 700, 1024), (1, 5, 1200001), (1, 1, 1)])
+def test_fields_read_back_whole(shape, precision):
+    """Fields of several read-back pieces (4 MiB each), ragged and dense rows, a
+    row longer than a piece (FP64), and one value: the values as written, in the
+    domain's precision."""
+    nz, ny, nx = shape
+    params = dict(lattice=9 if nz == 1 else 19, nx=nx, ny=ny, nz=nz, periodic=7, rho_l=1.0, rho_g=1.0, mu_l=0.1,
+                  mu_g=0.1, sigma=0.01, W=4.0, M_phi=0.02, theta=1.0, g=(0, 0, 0), precision=precision)
+    d = lbm.Domain(params, np.zeros(shape, np.uint8), (np.zeros(0, np.int64), np.zeros((0, 3))))
+    rng = np.random.default_rng(nx)
+    kind = np.float64 if precision == lbm.FP64 else np.float32
+    for f, n in (("phi", 1), ("u", 3), ("p", 1)):
+        v = rng.uniform(0, 1, n * nx * ny * nz)
+        if f == "u" and nz == 1:
+            v[2 * nx * ny:] = 0.0
+        d.write(f, v)
+        assert np.array_equal(d.read(f).reshape(-1), v.astype(kind).astype(np.float64)), f
