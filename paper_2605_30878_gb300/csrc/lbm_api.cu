@@ -694,7 +694,9 @@ bool encode_halo_maps(const lbm_domain* d, HaloMaps& out) {
 // The maps of the domain's own kernels.
 template <int Q>
 bool make_halo_maps(lbm_domain* d) {
-    if (d->cfg.pair) return encode_halo_maps_tile<PairTile<Q>>(d, d->maps);
+    if (d->cfg.pair)
+        return d->cfg.pair_width == 64 ? encode_halo_maps_tile<PairTile<Q>>(d, d->maps)
+                                       : encode_halo_maps_tile<NarrowTile<Q>>(d, d->maps);
     return d->fp64 ? encode_halo_maps<Q, kSingleTile<double>>(d, d->maps)
                    : encode_halo_maps<Q, kSingleTile<float>>(d, d->maps);
 }
@@ -1007,6 +1009,13 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     const char* step_kernel = std::getenv("LBM_STEP_KERNEL");
     c.pair = P.precision != LBM_FP64 && (step_kernel == nullptr || std::strcmp(step_kernel, "pair") == 0);
 
+    // 64-node tiles hold fewer idle lanes at row ends per block and cost less
+    // per lane; a 3D grid whose rows 32-wide tiles cover with 1/6 fewer lanes
+    // (nx = 65..96, 129..160) runs faster on those.  us per step, 64 against 32
+    // wide, FP32: 70^3 28.9 / 27.1, 96^3 51.5 / 49.6, 65 x 120 x 40 28.2 / 26.1;
+    // 100^3 60.0 / 63.0, 128^3 102 / 105, 192^3 316 / 323, 2D 600^2 12.0 / 12.3.
+    auto covered = [&](int w) { return (P.nx + w - 1) / w * w; };
+    c.pair_width = L.D == 3 && 6 * covered(32) <= 5 * covered(64) ? 32 : 64;
     // node classes, as row bit masks on the host (the device expands them)
     const int64_t nn = L.nn_dense;
     const int64_t nx = P.nx, ny = P.ny, nz = P.nz;
@@ -1485,6 +1494,12 @@ struct lbm_batch {
     std::vector<int> cur0;             // each domain's buffer parity when the batch was made
     int parity = 0;                    // steps taken by the batch, mod 2
     int variant = 0;
+    // tile shape of the color kernel, -1: the step kernels'.  Float: shape 0 or
+    // 5, the two-node kernel's 32- or 64-wide tiles, whichever covers the
+    // domains' rows with fewer lanes (shape 5 if they are within 10%: it costs
+    // 3% less per lane).  Twelve ragged domains of 50^3 to 93^3: 304 us per step
+    // on shape 0 against 319 on shape 5 with the step on shape 5.
+    int color_shape = -1;
     int ntiles[kTileVariants] = {};
     int ncontrast[kTileVariants] = {};           // tiles of domains with density contrast come first
     int device = 0;
@@ -1556,9 +1571,11 @@ void batch_launch_step(lbm_batch* b, int parity, cudaStream_t s) {
     const int V = b->variant;
     bdispatch(b->precision, [&](auto Lx) {
         using L = decltype(Lx);
+        const int Vc = b->color_shape < 0 ? V : b->color_shape;
+        const size_t per_shape = (size_t)kBatchSlots * kSlotMaps;
         L::ghost_batched(b->GK, b->ghost_tabs, b->ghost_begin, (int)b->doms.size(), b->total_ghosts, parity, s);
-        L::step_color_batched(b->Q, V, b->tiles[V], b->maps + (size_t)V * kBatchSlots * kSlotMaps, b->ntiles[V],
-                              b->ncontrast[V], parity, s);
+        L::step_batched(b->Q, V, b->tiles[V], b->maps + V * per_shape, b->ntiles[V], b->ncontrast[V], parity, s);
+        L::color_batched(b->Q, Vc, b->tiles[Vc], b->maps + Vc * per_shape, b->ntiles[Vc], parity, s);
     });
 }
 
@@ -1681,6 +1698,13 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
                 if (pass == 0) b->ncontrast[V] = (int)tiles[V].size();
             }
         }
+    if (b->precision != LBM_FP64) {
+        const int64_t lanes0 = (int64_t)tiles[0].size() * tile_extent(b->Q, 0, 0) * tile_extent(b->Q, 0, 1) *
+                               tile_extent(b->Q, 0, 2);
+        const int64_t lanes5 = (int64_t)tiles[5].size() * tile_extent(b->Q, 5, 0) * tile_extent(b->Q, 5, 1) *
+                               tile_extent(b->Q, 5, 2);
+        b->color_shape = 10 * lanes0 <= 9 * lanes5 ? 0 : 5;
+    }
     b->total_ghosts = gbegin[n];
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t r = off; off = round_up(off + bytes, 256); return r; };

@@ -46,6 +46,9 @@ struct PairTile {
     __host__ __device__ static constexpr int off(int cx, int cy, int cz) { return cx + HX * (cy + HY * cz); }
 };
 
+// 32 nodes wide, as batch shape 0.
+template <int Q> using NarrowTile = PairTile<Q, 32, Q == 9 ? 8 : 4>;
+
 // Resident blocks per SM the pair kernel is compiled for (registers per
 // thread <= 65536 / (THREADS * blocks)), measured at 192^3 with the packed
 // node update: 6 (80 registers, no spills) for FP32 and FP16 storage; 7 (72
@@ -354,11 +357,11 @@ __device__ __forceinline__ void color_pair_tile(const StepParams<float>& P, cons
     *reinterpret_cast<float2*>(b.phi_out + pn.nodeA) = out;
 }
 
-template <int Q, typename S, bool CONTRAST>
-__global__ void __launch_bounds__(PairTile<Q>::THREADS, PairBlocks<S>::value)
+template <int Q, typename S, bool CONTRAST, int TXn, int TYn>
+__global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, PairBlocks<S>::value)
     k_step_pair(StepParams<float> P, StepBuffers<float, S> b, const __grid_constant__ CUtensorMap tm_phi,
                 const __grid_constant__ CUtensorMap tm_u, int tma) {
-    using Tl = PairTile<Q>;
+    using Tl = PairTile<Q, TXn, TYn>;
     constexpr int D = Tl::D;
     __shared__ __align__(128) float s_phi[Tl::HN];
     __shared__ __align__(128) float s_u[CONTRAST ? D * Tl::HN : 2];
@@ -371,17 +374,17 @@ __global__ void __launch_bounds__(PairTile<Q>::THREADS, PairBlocks<S>::value)
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();                                      // the barrier exists before anyone waits on it
     }
-    step_pair_tile<Q, S, CONTRAST>(P, b, s_phi, s_u, x0, y0, z0, interior ? &tm_phi : nullptr, &tm_u, &s_bar);
+    step_pair_tile<Q, S, CONTRAST, TXn, TYn>(P, b, s_phi, s_u, x0, y0, z0, interior ? &tm_phi : nullptr, &tm_u, &s_bar);
 }
 
 // Resident blocks per SM of the color kernel.
 template <int THREADS = 128> struct ColorBlocks { static constexpr int value = 8 * 128 / THREADS; };
 
-template <int Q, typename S>
-__global__ void __launch_bounds__(PairTile<Q>::THREADS, ColorBlocks<>::value)
+template <int Q, typename S, int TXn, int TYn>
+__global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, ColorBlocks<>::value)
     k_color_pair(StepParams<float> P, StepBuffers<float, S> b, const __grid_constant__ CUtensorMap tm_phi,
                  const __grid_constant__ CUtensorMap tm_f, int tma) {
-    using Tl = PairTile<Q>;
+    using Tl = PairTile<Q, TXn, TYn>;
     constexpr int D = Tl::D;
     __shared__ __align__(128) float s_phi[Tl::HN];
     __shared__ __align__(128) float s_f[D * Tl::HN];
@@ -395,7 +398,7 @@ __global__ void __launch_bounds__(PairTile<Q>::THREADS, ColorBlocks<>::value)
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();
     }
-    color_pair_tile<Q, S>(P, b, s_phi, s_f, x0, y0, z0, interior ? &tm_phi : nullptr, &tm_f, &s_bar);
+    color_pair_tile<Q, S, TXn, TYn>(P, b, s_phi, s_f, x0, y0, z0, interior ? &tm_phi : nullptr, &tm_f, &s_bar);
 }
 
 // Batched form: one pair tile of one domain per block, the domain's

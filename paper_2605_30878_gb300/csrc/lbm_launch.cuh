@@ -28,7 +28,8 @@ struct StepConfig {
     double exp_eps;
     double eps;                    // -(4/W) cos(theta)
     int ghost_rule;                // lbm_ghost_rule
-    bool pair = false;             // float arithmetic: the two-node step kernel (k_step_pair)
+    bool pair = false;             // float arithmetic: the two-node kernels (k_step_pair, k_color_pair)
+    int pair_width = 32;           // nodes along x of their tiles, 32 or 64
 };
 
 struct StepPtrs {
@@ -65,7 +66,7 @@ struct Launch {
     static dim3 step_grid(const Dims& d);
     template <int Q, int V = 0>
     static dim3 step_block();
-    template <int Q>
+    template <class Tl>
     static dim3 pair_grid(const Dims& d);
     template <int Q>
     static void step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
@@ -99,12 +100,15 @@ struct Launch {
     template <int Qc, int V>
     static void step_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast, int parity,
                                cudaStream_t s);
+    // the step kernels of every domain (the ghost update precedes them) on tile
+    // shape V; tiles[0, ncontrast) belong to domains with density contrast
+    static void step_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
+                             int parity, cudaStream_t s);
     template <int Qc, int V>
     static void color_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int parity, cudaStream_t s);
-    // step kernels then color kernel of every domain (the ghost update precedes them);
-    // tiles[0, ncontrast) belong to domains with density contrast
-    static void step_color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
-                                   int parity, cudaStream_t s);
+    // the color kernel of every domain on tile shape V
+    static void color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int parity,
+                              cudaStream_t s);
     // Slot tables: entry_size() bytes per domain, filled by fill_entry, copied
     // to slots [slot0, slot0 + n) of the constant table by upload_entries.
     static size_t entry_size() { return sizeof(BatchEntry<T, S>); }

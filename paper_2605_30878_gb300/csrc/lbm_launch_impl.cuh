@@ -87,9 +87,8 @@ dim3 Launch<T, S>::step_block() {
 }
 
 template <typename T, typename S>
-template <int Q>
+template <class Tl>
 dim3 Launch<T, S>::pair_grid(const Dims& d) {
-    using Tl = PairTile<Q>;
     return dim3((d.nx + Tl::TX - 1) / Tl::TX, (d.ny + Tl::TY - 1) / Tl::TY, (d.nz + Tl::TZ - 1) / Tl::TZ);
 }
 
@@ -116,12 +115,15 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s
     }
     if constexpr (sizeof(T) == 4) {
         if (c.pair) {
-            using Tl = PairTile<Q>;
-            const dim3 block(Tl::BX, Tl::TY, Tl::TZ);
-            if (c.contrast)
-                launch_pdl(k_step_pair<Q, S, true>, pair_grid<Q>(c.d), block, s, P, b, tm_phi, tm_u, tma);
-            else
-                launch_pdl(k_step_pair<Q, S, false>, pair_grid<Q>(c.d), block, s, P, b, tm_phi, tm_u, tma);
+            auto run = [&](auto tile) {
+                using Tl = decltype(tile);
+                const dim3 block(Tl::BX, Tl::TY, Tl::TZ), grid = pair_grid<Tl>(c.d);
+                if (c.contrast)
+                    launch_pdl(k_step_pair<Q, S, true, Tl::TX, Tl::TY>, grid, block, s, P, b, tm_phi, tm_u, tma);
+                else
+                    launch_pdl(k_step_pair<Q, S, false, Tl::TX, Tl::TY>, grid, block, s, P, b, tm_phi, tm_u, tma);
+            };
+            if (c.pair_width == 64) run(PairTile<Q>{}); else run(NarrowTile<Q>{});
             return;
         }
     }
@@ -150,8 +152,12 @@ void Launch<T, S>::color_q(const StepConfig& c, const StepPtrs& p, cudaStream_t 
     }
     if constexpr (sizeof(T) == 4) {
         if (c.pair) {
-            using Tl = PairTile<Q>;
-            launch_pdl(k_color_pair<Q, S>, pair_grid<Q>(c.d), dim3(Tl::BX, Tl::TY, Tl::TZ), s, P, b, tm_phi, tm_f, tma);
+            auto run = [&](auto tile) {
+                using Tl = decltype(tile);
+                launch_pdl(k_color_pair<Q, S, Tl::TX, Tl::TY>, pair_grid<Tl>(c.d), dim3(Tl::BX, Tl::TY, Tl::TZ), s, P, b,
+                           tm_phi, tm_f, tma);
+            };
+            if (c.pair_width == 64) run(PairTile<Q>{}); else run(NarrowTile<Q>{});
             return;
         }
     }
@@ -307,27 +313,39 @@ void Launch<T, S>::color_batched_v(const int4* tiles, const CUtensorMap* maps, i
     }
 }
 
-// step kernels then color kernel of every domain (the ghost update precedes them);
-// tiles[0, ncontrast) belong to domains with density contrast
-template <typename T, typename S>
-void Launch<T, S>::step_color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles,
-                                      int ncontrast, int parity, cudaStream_t s) {
-    if (ntiles == 0) return;
-    auto run = [&](auto q, auto v) {
-        constexpr int Qc = decltype(q)::value, Vc = decltype(v)::value;
-        step_batched_v<Qc, Vc>(tiles, maps, ntiles, ncontrast, parity, s);
-        color_batched_v<Qc, Vc>(tiles, maps, ntiles, parity, s);
-    };
+// f(lattice, shape) with both as compile-time constants
+template <class F>
+void with_shape(int Q, int V, F&& f) {
     auto shapes = [&](auto q) {
-        if (V == 0) run(q, std::integral_constant<int, 0>{});
-        if (V == 1) run(q, std::integral_constant<int, 1>{});
-        if (V == 2) run(q, std::integral_constant<int, 2>{});
-        if (V == 3) run(q, std::integral_constant<int, 3>{});
-        if (V == 4) run(q, std::integral_constant<int, 4>{});
-        if (V == 5) run(q, std::integral_constant<int, 5>{});
+        switch (V) {
+        case 0: f(q, std::integral_constant<int, 0>{}); break;
+        case 1: f(q, std::integral_constant<int, 1>{}); break;
+        case 2: f(q, std::integral_constant<int, 2>{}); break;
+        case 3: f(q, std::integral_constant<int, 3>{}); break;
+        case 4: f(q, std::integral_constant<int, 4>{}); break;
+        default: f(q, std::integral_constant<int, 5>{}); break;
+        }
     };
     if (Q == 9) shapes(std::integral_constant<int, 9>{});
     else shapes(std::integral_constant<int, 19>{});
+}
+
+template <typename T, typename S>
+void Launch<T, S>::step_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
+                                int parity, cudaStream_t s) {
+    if (ntiles == 0) return;
+    with_shape(Q, V, [&](auto q, auto v) {
+        step_batched_v<decltype(q)::value, decltype(v)::value>(tiles, maps, ntiles, ncontrast, parity, s);
+    });
+}
+
+template <typename T, typename S>
+void Launch<T, S>::color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int parity,
+                                 cudaStream_t s) {
+    if (ntiles == 0) return;
+    with_shape(Q, V, [&](auto q, auto v) {
+        color_batched_v<decltype(q)::value, decltype(v)::value>(tiles, maps, ntiles, parity, s);
+    });
 }
 
 template <typename T, typename S>
