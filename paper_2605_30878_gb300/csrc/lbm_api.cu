@@ -627,7 +627,7 @@ void launch_one_step(lbm_domain* d, int cur, cudaStream_t s, cudaEvent_t* ev = n
     if (ev) cudaEventRecord(ev[1], s);
     dispatch(d, [&](auto Lx) { decltype(Lx)::step(d->cfg, sp, s); });
     if (ev) cudaEventRecord(ev[2], s);
-    dispatch(d, [&](auto Lx) { decltype(Lx)::color(d->cfg, sp, s); });
+    dispatch(d, [&](auto Lx) { decltype(Lx)::color(d->cfg, sp, d->ng > 0, s); });
     if (ev) cudaEventRecord(ev[3], s);
 }
 
@@ -1575,7 +1575,8 @@ void batch_launch_step(lbm_batch* b, int parity, cudaStream_t s) {
         const size_t per_shape = (size_t)kBatchSlots * kSlotMaps;
         L::ghost_batched(b->GK, b->ghost_tabs, b->ghost_begin, (int)b->doms.size(), b->total_ghosts, parity, s);
         L::step_batched(b->Q, V, b->tiles[V], b->maps + V * per_shape, b->ntiles[V], b->ncontrast[V], parity, s);
-        L::color_batched(b->Q, Vc, b->tiles[Vc], b->maps + Vc * per_shape, b->ntiles[Vc], parity, s);
+        L::color_batched(b->Q, Vc, b->tiles[Vc], b->maps + Vc * per_shape, b->ntiles[Vc], parity,
+                         b->total_ghosts > 0, s);
     });
 }
 

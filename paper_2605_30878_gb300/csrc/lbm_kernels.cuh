@@ -305,11 +305,14 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // tables, parameters).  pdl_wait() returns when the kernel before has finished
 // and its writes are visible; every thread of every kernel in the chain passes
 // it, so "the kernel before" covers all earlier ones.  The next kernel may start
-// from pdl_trigger() on, or as this one's blocks end.  The ghost and color
-// kernels trigger at once, the step kernels do not: their successor's blocks
-// would only hold room beside them (us per step, all three triggering against
-// this: 49 x 52 x 47 15.2 and 13.1, 64^3 FP64 260 and 248; without programmatic
-// launches 14.9 and 251, 401^2 9.4 against 7.9, 16 batched 2D domains 48 against 45).
+// from pdl_trigger() on, or as this one's blocks end.  Only a kernel that the
+// ghost kernel follows (the color kernel of a domain with ghost nodes) and the
+// ghost kernel itself trigger at once: the blocks of a large successor would
+// hold room beside a running kernel (us per step: step kernels triggering too,
+// 49 x 52 x 47 15.2 against 13.1, 64^3 FP64 260 against 248; a color kernel that
+// the step kernel follows, 192^3 without ghost nodes 436 against 316).  Without
+// programmatic launches: 49 x 52 x 47 14.9, 401^2 9.4 against 7.9, 128^3 packing
+// 112 against 108, 16 batched 2D domains 48 against 45.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -1166,12 +1169,13 @@ __device__ __forceinline__ V color_update(const StepParams<typename V::Real>& P,
     return s;
 }
 
-// The color tile at (x0, y0, z0), one node per thread: halo of the color and
+// The color tile at (x0, y0, z0), one node per thread (early: the ghost kernel
+// follows and may start at once): halo of the color and
 // the flux, the pull of N* while it is in flight.  A node that is not fluid
 // keeps its value (ghost nodes their ghost color, read back as it was used).
 template <int Q, int V, typename T, typename S>
 __device__ __forceinline__ void color_tile(const StepParams<T>& P, const StepBuffers<T, S>& b, T* s_phi, T* s_f, int x0,
-                                           int y0, int z0, const CUtensorMap* tm_phi = nullptr,
+                                           int y0, int z0, int early, const CUtensorMap* tm_phi = nullptr,
                                            const CUtensorMap* tm_f = nullptr, uint64_t* bar = nullptr) {
     using Tl = Tile<Q, V>;
     using L = Lattice<Q>;
@@ -1183,7 +1187,7 @@ __device__ __forceinline__ void color_tile(const StepParams<T>& P, const StepBuf
     const int node = in_grid ? idx_checked(x + P.px * (y + P.ny * z), P.plane, b.err) : 0;
     const uint32_t m = in_grid ? __ldg(b.mask + node) : MASK_NOT_FLUID;
     pdl_wait();
-    pdl_trigger();
+    if (early) pdl_trigger();
     HaloFix<Tl, T, true> fx;
     if (!halo_issue<Tl, T, true>(P, b.phi, b.flux, b.err, s_phi, s_f, x0, y0, z0, tm_phi, tm_f, bar, fx)) return;
     T N[Q], n0 = T(0);
@@ -1229,7 +1233,7 @@ __device__ __forceinline__ void color_tile(const StepParams<T>& P, const StepBuf
 template <int Q, typename T, typename S, int V = 0>
 __global__ void __launch_bounds__(Tile<Q, V>::THREADS)
     k_color(StepParams<T> P, StepBuffers<T, S> b, const __grid_constant__ CUtensorMap tm_phi,
-            const __grid_constant__ CUtensorMap tm_f, int tma) {
+            const __grid_constant__ CUtensorMap tm_f, int tma, int early) {
     using Tl = Tile<Q, V>;
     __shared__ __align__(128) T s_phi[Tl::HN];
     __shared__ __align__(128) T s_f[Tl::D * Tl::HN];
@@ -1243,9 +1247,9 @@ __global__ void __launch_bounds__(Tile<Q, V>::THREADS)
     if (interior) {
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();
-        color_tile<Q, V, T, S>(P, b, s_phi, s_f, x0, y0, z0, &tm_phi, &tm_f, &s_bar);
+        color_tile<Q, V, T, S>(P, b, s_phi, s_f, x0, y0, z0, early, &tm_phi, &tm_f, &s_bar);
     } else {
-        color_tile<Q, V, T, S>(P, b, s_phi, s_f, x0, y0, z0);
+        color_tile<Q, V, T, S>(P, b, s_phi, s_f, x0, y0, z0, early);
     }
 }
 
@@ -1353,7 +1357,7 @@ __global__ void __launch_bounds__(Tile<Q, V>::THREADS, (step_min_blocks<T, S, Ti
 
 template <int Q, typename T, typename S, int V>
 __global__ void __launch_bounds__(Tile<Q, V>::THREADS)
-    k_color_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity) {
+    k_color_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity, int early) {
     using Tl = Tile<Q, V>;
     __shared__ __align__(128) T s_phi[Tl::HN];
     __shared__ __align__(128) T s_f[Tl::D * Tl::HN];
@@ -1371,10 +1375,10 @@ __global__ void __launch_bounds__(Tile<Q, V>::THREADS)
     if (tma) {
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();
-        color_tile<Q, V, T, S>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0, slot_phi_map(maps, t.x, parity),
+        color_tile<Q, V, T, S>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0, early, slot_phi_map(maps, t.x, parity),
                                slot_flux_map(maps, t.x), &s_bar);
     } else {
-        color_tile<Q, V, T, S>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0);
+        color_tile<Q, V, T, S>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0, early);
     }
 }
 

@@ -295,7 +295,7 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
 // arithmetic.  Warps without a bounce-back direction skip its selects.
 template <int Q, typename S, int TXn = 64, int TYn = 0>
 __device__ __forceinline__ void color_pair_tile(const StepParams<float>& P, const StepBuffers<float, S>& b,
-                                                float* s_phi, float* s_f, int x0, int y0, int z0,
+                                                float* s_phi, float* s_f, int x0, int y0, int z0, int early,
                                                 const CUtensorMap* tm_phi, const CUtensorMap* tm_f, uint64_t* bar) {
     using Tl = PairTile<Q, TXn, TYn>;
     using L = Lattice<Q>;
@@ -304,7 +304,7 @@ __device__ __forceinline__ void color_pair_tile(const StepParams<float>& P, cons
     int* const err = b.err;
     const PairNode pn(P, b.mask, x0, y0, z0, err);
     pdl_wait();
-    pdl_trigger();
+    if (early) pdl_trigger();
     HaloFix<Tl, float, true> fx;
     if (!halo_issue<Tl, float, true>(P, b.phi, b.flux, err, s_phi, s_f, x0, y0, z0, tm_phi, tm_f, bar, fx)) return;
     float NA[Q], NB[Q];
@@ -383,7 +383,7 @@ template <int THREADS = 128> struct ColorBlocks { static constexpr int value = 8
 template <int Q, typename S, int TXn, int TYn>
 __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, ColorBlocks<>::value)
     k_color_pair(StepParams<float> P, StepBuffers<float, S> b, const __grid_constant__ CUtensorMap tm_phi,
-                 const __grid_constant__ CUtensorMap tm_f, int tma) {
+                 const __grid_constant__ CUtensorMap tm_f, int tma, int early) {
     using Tl = PairTile<Q, TXn, TYn>;
     constexpr int D = Tl::D;
     __shared__ __align__(128) float s_phi[Tl::HN];
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, ColorBlocks<>:
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();
     }
-    color_pair_tile<Q, S, TXn, TYn>(P, b, s_phi, s_f, x0, y0, z0, interior ? &tm_phi : nullptr, &tm_f, &s_bar);
+    color_pair_tile<Q, S, TXn, TYn>(P, b, s_phi, s_f, x0, y0, z0, early, interior ? &tm_phi : nullptr, &tm_f, &s_bar);
 }
 
 // Batched form: one pair tile of one domain per block, the domain's
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
 
 template <int Q, typename S, int TXn = 64, int TYn = 0>
 __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, (ColorBlocks<PairTile<Q, TXn, TYn>::THREADS>::value))
-    k_color_pair_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity) {
+    k_color_pair_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity, int early) {
     using Tl = PairTile<Q, TXn, TYn>;
     constexpr int D = Tl::D;
     __shared__ __align__(128) float s_phi[Tl::HN];
@@ -454,7 +454,7 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, (ColorBlocks<P
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();
     }
-    color_pair_tile<Q, S, TXn, TYn>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0,
+    color_pair_tile<Q, S, TXn, TYn>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0, early,
                                     tma ? slot_phi_map(maps, t.x, parity) : nullptr, slot_flux_map(maps, t.x), &s_bar);
 }
 

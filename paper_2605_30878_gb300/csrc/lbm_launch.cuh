@@ -72,8 +72,9 @@ struct Launch {
     static void step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
     static void step(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
     template <int Q>
-    static void color_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
-    static void color(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
+    static void color_q(const StepConfig& c, const StepPtrs& p, int early, cudaStream_t s);
+    // ghosts_follow: the next kernel on the stream is the ghost kernel
+    static void color(const StepConfig& c, const StepPtrs& p, bool ghosts_follow, cudaStream_t s);
     static StepBuffers<T, S> buffers(const StepPtrs& p);
     static void ghost(int GK, int rule, int64_t ng, const int32_t* node, const int32_t* corner, const void* wt,
                       double exp_eps, double eps, void* phi, int64_t plane, int* err, cudaStream_t s);
@@ -105,10 +106,11 @@ struct Launch {
     static void step_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
                              int parity, cudaStream_t s);
     template <int Qc, int V>
-    static void color_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int parity, cudaStream_t s);
+    static void color_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int parity, int early,
+                                cudaStream_t s);
     // the color kernel of every domain on tile shape V
     static void color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int parity,
-                              cudaStream_t s);
+                              bool ghosts_follow, cudaStream_t s);
     // Slot tables: entry_size() bytes per domain, filled by fill_entry, copied
     // to slots [slot0, slot0 + n) of the constant table by upload_entries.
     static size_t entry_size() { return sizeof(BatchEntry<T, S>); }

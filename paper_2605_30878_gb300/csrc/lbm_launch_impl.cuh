@@ -141,7 +141,7 @@ void Launch<T, S>::step(const StepConfig& c, const StepPtrs& p, cudaStream_t s) 
 
 template <typename T, typename S>
 template <int Q>
-void Launch<T, S>::color_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s) {
+void Launch<T, S>::color_q(const StepConfig& c, const StepPtrs& p, int early, cudaStream_t s) {
     const StepParams<T> P = params(c);
     const StepBuffers<T, S> b = buffers(p);
     CUtensorMap tm_phi{}, tm_f{};
@@ -155,19 +155,19 @@ void Launch<T, S>::color_q(const StepConfig& c, const StepPtrs& p, cudaStream_t 
             auto run = [&](auto tile) {
                 using Tl = decltype(tile);
                 launch_pdl(k_color_pair<Q, S, Tl::TX, Tl::TY>, pair_grid<Tl>(c.d), dim3(Tl::BX, Tl::TY, Tl::TZ), s, P, b,
-                           tm_phi, tm_f, tma);
+                           tm_phi, tm_f, tma, early);
             };
             if (c.pair_width == 64) run(PairTile<Q>{}); else run(NarrowTile<Q>{});
             return;
         }
     }
     constexpr int V = kSingleTile<T>;
-    launch_pdl(k_color<Q, T, S, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_f, tma);
+    launch_pdl(k_color<Q, T, S, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_f, tma, early);
 }
 
 template <typename T, typename S>
-void Launch<T, S>::color(const StepConfig& c, const StepPtrs& p, cudaStream_t s) {
-    if (c.Q == 9) color_q<9>(c, p, s); else color_q<19>(c, p, s);
+void Launch<T, S>::color(const StepConfig& c, const StepPtrs& p, bool ghosts_follow, cudaStream_t s) {
+    if (c.Q == 9) color_q<9>(c, p, ghosts_follow, s); else color_q<19>(c, p, ghosts_follow, s);
 }
 
 template <typename T, typename S>
@@ -302,14 +302,16 @@ void Launch<T, S>::step_batched_v(const int4* tiles, const CUtensorMap* maps, in
 
 template <typename T, typename S>
 template <int Qc, int V>
-void Launch<T, S>::color_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int parity, cudaStream_t s) {
+void Launch<T, S>::color_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int parity, int early,
+                                   cudaStream_t s) {
     using Tl = Tile<Qc, V>;
     if constexpr ((V == 5 || V == 3 || V == 0) && sizeof(T) == 4) {
         constexpr int TXn = Tl::TX, TYn = Tl::TY;
         using Pt = PairTile<Qc, TXn, TYn>;
-        launch_pdl(k_color_pair_batched<Qc, S, TXn, TYn>, ntiles, dim3(Pt::BX, Pt::TY, Pt::TZ), s, tiles, maps, parity);
+        launch_pdl(k_color_pair_batched<Qc, S, TXn, TYn>, ntiles, dim3(Pt::BX, Pt::TY, Pt::TZ), s, tiles, maps, parity,
+                   early);
     } else {
-        launch_pdl(k_color_batched<Qc, T, S, V>, ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), s, tiles, maps, parity);
+        launch_pdl(k_color_batched<Qc, T, S, V>, ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), s, tiles, maps, parity, early);
     }
 }
 
@@ -341,10 +343,10 @@ void Launch<T, S>::step_batched(int Q, int V, const int4* tiles, const CUtensorM
 
 template <typename T, typename S>
 void Launch<T, S>::color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int parity,
-                                 cudaStream_t s) {
+                                 bool ghosts_follow, cudaStream_t s) {
     if (ntiles == 0) return;
     with_shape(Q, V, [&](auto q, auto v) {
-        color_batched_v<decltype(q)::value, decltype(v)::value>(tiles, maps, ntiles, parity, s);
+        color_batched_v<decltype(q)::value, decltype(v)::value>(tiles, maps, ntiles, parity, ghosts_follow, s);
     });
 }
 
