@@ -49,12 +49,14 @@ struct PairTile {
 // 32 nodes wide, as batch shape 0.
 template <int Q> using NarrowTile = PairTile<Q, 32, Q == 9 ? 8 : 4>;
 
-// Resident blocks per SM the pair kernel is compiled for (registers per
-// thread <= 65536 / (THREADS * blocks)), measured at 192^3 with the packed
-// node update: 6 (80 registers, no spills) for FP32 and FP16 storage; 7 (72
-// registers) spills 50 bytes with FP16 storage and runs 9% slower; 4 is 20%
-// slower; 8 spills 76 bytes or more.
-template <typename S, int THREADS = 128> struct PairBlocks { static constexpr int value = 6 * 128 / THREADS; };
+// Resident blocks per SM the pair kernel is compiled for (registers per thread
+// <= 65536 / (THREADS * blocks)): 7 with density contrast (72 registers), 8
+// without (64).  us per step with 6, 7 and 8: 192^3 FP16 storage 255, 250, 255
+// and FP32 316, 317, 317, twelve 3D domains, both kinds, 304, 294, 291, 128^3
+// packing (no contrast) 107.9, 108.0, 106.7.
+template <bool CONTRAST, int THREADS = 128> struct PairBlocks {
+    static constexpr int value = (CONTRAST ? 7 : 8) * 128 / THREADS;
+};
 
 // The values at halo slots hc + o and hc + o + 1 (hc even): one aligned
 // two-wide load for even o, else the odd half of the pair below and the even
@@ -358,7 +360,7 @@ __device__ __forceinline__ void color_pair_tile(const StepParams<float>& P, cons
 }
 
 template <int Q, typename S, bool CONTRAST, int TXn, int TYn>
-__global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, PairBlocks<S>::value)
+__global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, PairBlocks<CONTRAST>::value)
     k_step_pair(StepParams<float> P, StepBuffers<float, S> b, const __grid_constant__ CUtensorMap tm_phi,
                 const __grid_constant__ CUtensorMap tm_u, int tma) {
     using Tl = PairTile<Q, TXn, TYn>;
@@ -377,7 +379,8 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, PairBlocks<S>:
     step_pair_tile<Q, S, CONTRAST, TXn, TYn>(P, b, s_phi, s_u, x0, y0, z0, interior ? &tm_phi : nullptr, &tm_u, &s_bar);
 }
 
-// Resident blocks per SM of the color kernel.
+// Resident blocks per SM of the color kernel: 8 (64 registers).  With 6, 7, 8:
+// 192^3 FP32 130, 122, 119 us per launch, FP16 storage 103, 101, 97.
 template <int THREADS = 128> struct ColorBlocks { static constexpr int value = 8 * 128 / THREADS; };
 
 template <int Q, typename S, int TXn, int TYn>
@@ -406,7 +409,7 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS, ColorBlocks<>:
 // for tile shape 5, 32 for tile shapes 0 and 3.
 template <int Q, typename S, bool CONTRAST, int TXn = 64, int TYn = 0>
 __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
-                                  (PairBlocks<S, PairTile<Q, TXn, TYn>::THREADS>::value))
+                                  (PairBlocks<CONTRAST, PairTile<Q, TXn, TYn>::THREADS>::value))
     k_step_pair_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity) {
     using Tl = PairTile<Q, TXn, TYn>;
     constexpr int D = Tl::D;
