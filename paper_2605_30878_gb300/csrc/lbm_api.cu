@@ -1001,11 +1001,10 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     c.eps = -(4.0 / P.W) * std::cos(P.theta);
     c.exp_eps = std::exp(c.eps);
     c.ghost_rule = P.ghost_rule;
-    // Float arithmetic: the two-node step kernel (half the load/store and
-    // address instructions per node of the one-node kernel; at 192^3 0.967
-    // against 0.919 of the measured copy peak with FP32 storage, 0.667 against
-    // 0.658 of its roofline with FP16 storage).  LBM_STEP_KERNEL=pair|single
-    // overrides; both kernels give the same results to the bit.
+    // Float arithmetic: the two-node kernels (half the load and store
+    // instructions per node of the one-node kernels; 192^3 319 us per step
+    // against 349 with FP32 and 252 against 313 with FP16 storage).
+    // LBM_STEP_KERNEL=pair|single overrides; both give the same results to the bit.
     const char* step_kernel = std::getenv("LBM_STEP_KERNEL");
     c.pair = P.precision != LBM_FP64 && (step_kernel == nullptr || std::strcmp(step_kernel, "pair") == 0);
 
@@ -1421,13 +1420,14 @@ double lbm_bytes_per_fluid_node(const lbm_domain* d) {
     const double s = (double)d->lay.elem;
     const double moving = (d->lay.Q - 1) * (double)d->lay.pop_elem;
     const double pop = (double)d->lay.rest_elem + moving;   // per node and array
-    // k_step pulls N: the FP64 update follows the literal collision and reads the
-    // rest population, the float updates take every moment from the moving ones
+    // the two-population scheme's count, not the kernels' (which make B from N*,
+    // phi and the flux: 304 bytes in D3Q19 FP32 with density contrast against
+    // 344 here): N pulled, N* and B* written, B* pulled; in FP64 with the rest
+    // population's pull
     const double pull = d->lay.elem == 8 ? pop : moving;
     const int D = d->lay.D;
-    // N* and B* written, B* pulled by k_phi; phi written (k_phi) and read (k_step);
-    // u written, and read when the density contrast makes F_visc active; p written; the 4-byte
-    // bounce-back mask read by k_step and k_phi
+    // phi written and read; u written, and read when the density contrast makes
+    // F_visc active; p written; the 4-byte bounce-back mask read twice
     return pull + 3.0 * pop + 2.0 * s + (d->contrast ? 2.0 : 1.0) * D * s + s + 8.0;
 }
 

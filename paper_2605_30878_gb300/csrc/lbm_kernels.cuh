@@ -77,8 +77,7 @@ struct StepParams {
 // ratio 1000) representable.  B, kept for state transfer only: full values in
 // S = double (FP64 mode), B_i - chi_i/2 in S = float (FP32 mode).  S = __half: the same deviations, the rest
 // populations (i = 0, whose B deviation reaches chi_0/2 ~ 0.46) as float in the
-// first plane, the moving ones times 2^16 (N) and 2^7 (B) as FP16 in the
-// following Q-1 planes.
+// first plane, the moving ones times 2^16 (N) and 2^7 (B) as FP16 after it.
 constexpr float kScaleN = 65536.0f;
 constexpr float kScaleB = 128.0f;
 
@@ -899,7 +898,7 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
     const int hc = (threadIdx.x + Tl::XO) + Tl::HX * ((threadIdx.y + 1) + Tl::HY * (D == 2 ? 0 : threadIdx.z + 1));
     const int pl = (int)P.plane;
     int* const err = b.err;
-    // every store index below is a direction's plane offset plus this node
+    // every store index below follows from this node
     if (!idx_ok(node, P.plane, err)) return;
     using PS = PopStore<S>;
     constexpr bool kShift = PS::kShift;

@@ -1,15 +1,21 @@
-// Two-node step kernel (float arithmetic, FP32 or FP16 population storage).
+// Two-node step and color kernels (float arithmetic, FP32 or FP16 population
+// storage).
 //
 // Every thread updates the two x-adjacent nodes A = (x0 + 2t, y, z) and
-// B = (x0 + 2t + 1, y, z) of its row, with the arithmetic of k_step: the same
-// stencil sums in the same order and NodeUpdate's per-node update, so the two
-// kernels round alike.  Since A's index is even, the pair shares
+// B = (x0 + 2t + 1, y, z) of its row, with the arithmetic of k_step and k_color:
+// the same sums in the same order and NodeUpdate's per-node update, so the
+// kernels round alike.  What bounds them on 192^3 (D3Q19, one GB300): with FP32
+// the DRAM (step 196 bytes per fluid node in 192 us, 7.1 TB/s; color 108 bytes
+// in 120 us, 6.3 TB/s), with FP16 storage instruction issue and latency (step
+// 124 bytes in 145 us, color 72 bytes in 102 us; ~1000 and ~620 instructions per
+// warp of 64 nodes).  Since A's index is even, the pair shares
 //   - its mask (one 8-byte load),
 //   - its streaming pulls along y and z (one two-wide load per direction with
 //     c_x = 0; directions with c_x != 0 pull from odd offsets, two loads),
 //   - its shared-memory stencil values (two-wide loads; the rows a +/- x
 //     direction needs come from three aligned two-wide loads, shared by the
-//     directions of that row),
+//     directions of that row; values at odd offsets enter by scalar operations,
+//     see H2),
 //   - its stores of N*, f, u and p (one two-wide store each),
 // which halves the load/store and address instructions per node of the
 // one-node kernel.  The float arithmetic of the two nodes runs on packed
