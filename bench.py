@@ -180,29 +180,9 @@ def recorded_traffic(fluid_nodes, fp16=False):
     return rec["dram_bytes_per_fluid_node"] * fluid_nodes
 
 
-def step_kernel_bytes(Q, D, s, contrast, moving=None, rest=None):
-    """Bytes that one step kernel launch moves per fluid node: pull the Q - 1
-    moving populations of N (moving bytes each: s, or 2 with FP16 storage), read
-    phi and, with a density contrast, the previous u, and the 4-byte mask; write
-    N* (the rest plane is float), u, the recolouring flux (D values) and p."""
-    moving = s if moving is None else moving
-    rest = s if rest is None else rest
-    return (Q - 1) * moving + s + (D * s if contrast else 0) + 4 + rest + (Q - 1) * moving + 2 * D * s + s
-
-
-def color_kernel_bytes(Q, D, s, moving=None, rest=None):
-    """Bytes that one color kernel launch moves per fluid node: pull N* whole,
-    read phi, the flux, the part of the color below its last place (float
-    arithmetic) and the mask; write phi and that part."""
-    moving = s if moving is None else moving
-    rest = s if rest is None else rest
-    lo = 2 * s if s == 4 else 0
-    return rest + (Q - 1) * moving + s + D * s + 4 + s + lo
-
-
 def k_step_bytes_per_fluid_node(Q, D, s, contrast, moving=None, rest=None):
-    """Bytes per fluid node of a step that writes N* and B* (the two-population
-    scheme; the kernels here move step_kernel_bytes): pull the Q - 1 moving populations of N (moving bytes each: s, or 2 with FP16
+    """Algorithmic bytes of one k_step launch per fluid node (float arithmetic):
+    pull the Q - 1 moving populations of N (moving bytes each: s, or 2 with FP16
     storage) -- the deviation form takes the pressure and every moment from
     them, so the rest population is not read, and the collision needs B only
     through phi, which k_phi computed --, write N* and B* (rest + (Q - 1)
@@ -476,7 +456,7 @@ def run_other_storage(lbm, args, cfg, probe, n_angle, fp64_deg):
     sec = time_domain(d, args.steps, warmup=args.warmup)
     kms = d.profile_steps(max(3, min(args.steps, 60)))
     t_step = kms[1] / max(3, min(args.steps, 60)) * 1e-3
-    kb = step_kernel_bytes(19, 3, 4, True, 2 if prec == lbm.FP16 else 4, 4) * fluid
+    kb = k_step_bytes_per_fluid_node(19, 3, 4, True, 2 if prec == lbm.FP16 else 4) * fluid
     peak, peak_kind = hbm_peak()
     d.close()
     da = lbm.Domain(P, cfg["solid"], cfg["ghosts"])
@@ -720,13 +700,13 @@ def run_ours(args):
     t_step = kms[1] / prof_steps * 1e-3
     s, Q, D = 4, 19, 3
     sp = 2 if prec == lbm.FP16 else 4
-    kb = step_kernel_bytes(Q, D, s, True, sp, 4) * fluid
+    kb = k_step_bytes_per_fluid_node(Q, D, s, True, sp) * fluid
     achieved = kb / t_step / 1e9
     peak, peak_kind = hbm_peak()
     traffic = recorded_traffic(fluid, fp16=prec == lbm.FP16)
     share = kms / kms.sum()
     launches = dom.launches_per_step()
-    bytes_step = step_kernel_bytes(Q, D, s, True, sp, 4) + color_kernel_bytes(Q, D, s, sp, 4)
+    bytes_step = dom.bytes_per_fluid_node()
     dom.close()
     del dom
     torch.cuda.empty_cache()
@@ -852,7 +832,7 @@ def run_ours(args):
             "roofline": {"bound": "hbm", "kernel": "k_step_pair<19,%s,contrast>" % ("half" if sp == 2 else "float"),
                          "achieved": achieved,
                          "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": achieved / peak,
-                         "traffic": traffic, "bytes_per_fluid_node": step_kernel_bytes(Q, D, s, True, sp, 4),
+                         "traffic": traffic, "bytes_per_fluid_node": k_step_bytes_per_fluid_node(Q, D, s, True, sp),
                          "avg_launch_ms": t_step * 1e3,
                          "kernel_share": {"ghost": share[0], "step": share[1], "phi": share[2]}},
             "step_bytes_per_fluid_node": bytes_step,

@@ -62,8 +62,7 @@ typedef enum { LBM_GHOST_PRESENT = 0, LBM_GHOST_FAKHARI = 1 } lbm_ghost_rule;
 /* Arithmetic and storage type of the step.  LBM_FP64: double throughout.
  * LBM_FP32: float arithmetic; populations stored in float as deviations from
  * the rest state (N_i - chi_i, B_i - chi_i/2), which keeps the small pressure
- * p = p_h/rho of a dense liquid representable.  The float modes carry the part
- * of the color below its last place from step to step.  LBM_FP32_STORE_FP16: float
+ * p = p_h/rho of a dense liquid representable.  LBM_FP32_STORE_FP16: float
  * arithmetic, the moving populations' deviations stored in FP16 scaled by
  * 2^16 (N) and 2^7 (B), the rest populations in float; the collision fixes
  * each node's totals (sum of N_i - chi_i is 0, sum of B_i - chi_i/2 is
@@ -226,10 +225,8 @@ lbm_status lbm_ghost_table(lbm_domain* dom, int64_t* corner, double* weight, int
 /* Number of ghosts that used the most-aligned-neighbour fallback. */
 int64_t lbm_ghost_fallbacks(const lbm_domain* dom);
 
-/* Kernel launches one lbm_step(dom, 1) issues, and the device bytes per fluid
- * node of a step that writes and reads both populations N and B (populations,
- * fields, node type).  The kernels move fewer: they make B from N, the color
- * and one vector. */
+/* Kernel launches one lbm_step(dom, 1) issues, and the algorithmic device
+ * bytes one step moves per fluid node (populations, fields, node type). */
 int32_t lbm_launches_per_step(const lbm_domain* dom);
 double  lbm_bytes_per_fluid_node(const lbm_domain* dom);
 int64_t lbm_fluid_nodes(const lbm_domain* dom);

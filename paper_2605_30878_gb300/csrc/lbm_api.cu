@@ -46,7 +46,7 @@ struct Layout {
     size_t rest_elem = 0;            // bytes of a stored rest population
     size_t pop_bytes = 0;            // bytes of one population array (Q planes)
     int Q = 0, D = 0, GK = 0;
-    size_t off_N[2], off_B, off_flux, off_phi[2], off_phi_lo, off_u[2], off_p, off_cls, off_mask, off_gnode, off_gcorner, off_gwt,
+    size_t off_N[2], off_B[2], off_phi, off_u[2], off_p, off_cls, off_mask, off_gnode, off_gcorner, off_gwt,
         off_err, off_partial, off_dout, off_stage;
     size_t total = 0;
 };
@@ -81,12 +81,8 @@ bool make_layout(const lbm_params* P, int64_t ng, Layout& L, std::string& err) {
     auto take = [&](size_t bytes) { size_t r = o; o = round_up(o + bytes, ALIGN); return r; };
     const size_t pop = (size_t)L.plane * (L.rest_elem + (size_t)(L.Q - 1) * L.pop_elem);
     L.pop_bytes = pop;
-    for (int k = 0; k < 2; ++k) L.off_N[k] = take(pop);
-    L.off_B = take(pop);                                 // state transfer only
-    L.off_flux = take((size_t)L.D * L.plane * L.elem);
-    L.off_phi[1] = take(L.plane * L.elem);
-    L.off_phi[0] = take(L.plane * L.elem);
-    L.off_phi_lo = take(P->precision == LBM_FP64 ? 0 : L.plane * L.elem);
+    for (int k = 0; k < 2; ++k) { L.off_N[k] = take(pop); L.off_B[k] = take(pop); }
+    L.off_phi = take(L.plane * L.elem);
     for (int k = 0; k < 2; ++k) L.off_u[k] = take((size_t)L.D * L.plane * L.elem);
     L.off_p = take(L.plane * L.elem);
     L.off_cls = take(L.plane);
@@ -132,11 +128,6 @@ cudaMemPool_t workspace_pool(int device) {
 
 }  // namespace
 
-// tiled maps of a domain's halo fields, one box
-struct HaloMaps {
-    CUtensorMap phi[2], u[2], flux;
-};
-
 struct lbm_domain {
     lbm_params prm;
     Layout lay;
@@ -168,24 +159,19 @@ struct lbm_domain {
     cudaGraphExec_t g1[2] = {nullptr, nullptr};
     cudaGraphExec_t g8 = nullptr;
     std::string err;
-    // tiled TMA maps of both colors, both velocity buffers and the flux for the
-    // halo copies, with the box of the domain's step kernel
+    // tiled TMA maps of phi and of both velocity buffers for the step kernel's
+    // halo copies (FP32 arithmetic, rows of a multiple of 16 bytes)
     bool tma = false;
-    HaloMaps maps;
-    // true: the buffer B() holds the current B (set by an init or a written B);
-    // false: B follows from the last step's color, N* and flux (rebuild_B)
-    bool b_stored = true;
+    CUtensorMap tm_phi{}, tm_u[2]{};       // with the box of the domain's step kernel
     // set once a bounded halo-copy wait gave up (LBM_ERR_TIMEOUT): a skipped
     // tile left the state wrong, so the domain takes no further steps
     bool poisoned = false;
 
     template <typename P> P* at(size_t off) const { return reinterpret_cast<P*>(ws + off); }
     void* N(int k) const { return at<void>(lay.off_N[k]); }
-    void* B() const { return at<void>(lay.off_B); }
-    void* flux() const { return at<void>(lay.off_flux); }
+    void* B(int k) const { return at<void>(lay.off_B[k]); }
     void* U(int k) const { return at<void>(lay.off_u[k]); }
-    void* phi(int k) const { return at<void>(lay.off_phi[k]); }
-    void* phi_lo() const { return at<void>(lay.off_phi_lo); }
+    void* phi() const { return at<void>(lay.off_phi); }
     void* p() const { return at<void>(lay.off_p); }
     uint8_t* cls() const { return at<uint8_t>(lay.off_cls); }
     uint32_t* mask() const { return at<uint32_t>(lay.off_mask); }
@@ -600,18 +586,7 @@ lbm_status prepare_ghosts(lbm_domain* d, const lbm_ghost* ghosts) {
     return LBM_OK;
 }
 
-// The buffers of a step that starts from buffers cur.
-StepPtrs step_ptrs(const lbm_domain* d, int cur) {
-    StepPtrs sp;
-    sp.Nin = d->N(cur); sp.Nout = d->N(1 - cur);
-    sp.phi = d->phi(cur); sp.phi_out = d->phi(1 - cur); sp.phi_lo = d->phi_lo();
-    sp.u_in = d->U(cur); sp.u_out = d->U(1 - cur); sp.p = d->p(); sp.flux = d->flux();
-    sp.mask = d->mask(); sp.err = d->errflag();
-    if (d->tma) { sp.tm_phi = &d->maps.phi[cur]; sp.tm_u = &d->maps.u[cur]; sp.tm_flux = &d->maps.flux; }
-    return sp;
-}
-
-// ev: optional events {before ghost, before step, before color, after color}
+// ev: optional events {before ghost, before step, before phi, after phi}
 void launch_one_step(lbm_domain* d, int cur, cudaStream_t s, cudaEvent_t* ev = nullptr) {
     const Layout& L = d->lay;
     if (ev) cudaEventRecord(ev[0], s);
@@ -619,15 +594,19 @@ void launch_one_step(lbm_domain* d, int cur, cudaStream_t s, cudaEvent_t* ev = n
         const void* wt = d->at<void>(L.off_gwt);
         dispatch(d, [&](auto Lx) {
             decltype(Lx)::ghost(L.GK, d->cfg.ghost_rule, d->ng, d->at<int32_t>(L.off_gnode),
-                                d->at<int32_t>(L.off_gcorner), wt, d->cfg.exp_eps, d->cfg.eps, d->phi(cur), L.plane,
+                                d->at<int32_t>(L.off_gcorner), wt, d->cfg.exp_eps, d->cfg.eps, d->phi(), L.plane,
                                 d->errflag(), s);
         });
     }
-    const StepPtrs sp = step_ptrs(d, cur);
+    StepPtrs sp;
+    sp.Nin = d->N(cur); sp.Bin = d->B(cur); sp.Nout = d->N(1 - cur); sp.Bout = d->B(1 - cur);
+    sp.phi = d->phi(); sp.u_in = d->U(cur); sp.u_out = d->U(1 - cur); sp.p = d->p();
+    sp.mask = d->mask(); sp.err = d->errflag();
+    if (d->tma) { sp.tm_phi = &d->tm_phi; sp.tm_u = &d->tm_u[cur]; }
     if (ev) cudaEventRecord(ev[1], s);
     dispatch(d, [&](auto Lx) { decltype(Lx)::step(d->cfg, sp, s); });
     if (ev) cudaEventRecord(ev[2], s);
-    dispatch(d, [&](auto Lx) { decltype(Lx)::color(d->cfg, sp, d->ng > 0, s); });
+    dispatch(d, [&](auto Lx) { decltype(Lx)::phi(d->cfg, d->B(1 - cur), d->mask(), d->phi(), d->ng > 0, d->errflag(), s); });
     if (ev) cudaEventRecord(ev[3], s);
 }
 
@@ -661,48 +640,53 @@ EncodeTiledFn encode_tiled() {
     return fn;
 }
 
-// Tensor maps for the halo copies: each color as (nx, ny, nz), each velocity
-// buffer and the flux as (nx, ny, nz, D) values, box = the halo tile of Tl.
-// Rows are a multiple of 16 bytes (the strides TMA accepts); if the driver
-// refuses, the kernel copies every halo element itself.
+// Tensor maps for the halo copies of the step kernel: phi as (nx, ny, nz) and
+// each velocity buffer as (nx, ny, nz, D) floats, box = the halo tile of
+// Tile<Q, V>; out[0] = phi, out[1 + k] = velocity buffer k.  Only for float
+// fields whose rows are a multiple of 16 bytes (the strides TMA accepts);
+// otherwise, or if the driver refuses, the kernel copies every halo element
+// itself.
 template <class Tl>
-bool encode_halo_maps_tile(const lbm_domain* d, HaloMaps& out) {
+bool encode_halo_maps_tile(const lbm_domain* d, CUtensorMap out[3]) {
     const lbm_params& P = d->prm;
+    if (d->fp64) return false;
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return false;
     const int D = Tl::D;
     const cuuint64_t dims[4] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny, (cuuint64_t)P.nz, (cuuint64_t)D};
-    const cuuint64_t es = d->lay.elem;
-    const cuuint64_t strides[3] = {d->lay.px * es, d->lay.px * es * P.ny, d->lay.plane * es};
-    const CUtensorMapDataType type = d->fp64 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    const cuuint64_t strides[3] = {(cuuint64_t)d->lay.px * 4, (cuuint64_t)d->lay.px * P.ny * 4,
+                                   (cuuint64_t)d->lay.plane * 4};
     const cuuint32_t box[4] = {(cuuint32_t)Tl::HX, (cuuint32_t)Tl::HY, (cuuint32_t)Tl::HZ, (cuuint32_t)D};
     const cuuint32_t ones[4] = {1, 1, 1, 1};
     auto one = [&](CUtensorMap* m, void* base, cuuint32_t rank) {
-        return enc(m, type, rank, base, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, rank, base, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
                    CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
     };
-    return one(&out.phi[0], d->phi(0), 3) && one(&out.phi[1], d->phi(1), 3) && one(&out.u[0], d->U(0), 4) &&
-           one(&out.u[1], d->U(1), 4) && one(&out.flux, d->flux(), 4);
+    return one(&out[0], d->phi(), 3) && one(&out[1], d->U(0), 4) && one(&out[2], d->U(1), 4);
 }
 
 template <int Q, int V>
-bool encode_halo_maps(const lbm_domain* d, HaloMaps& out) {
+bool encode_halo_maps(const lbm_domain* d, CUtensorMap out[3]) {
     return encode_halo_maps_tile<Tile<Q, V>>(d, out);
 }
 
-// The maps of the domain's own kernels.
+// The maps of the domain's own step kernel.
 template <int Q>
 bool make_halo_maps(lbm_domain* d) {
-    if (d->cfg.pair)
-        return d->cfg.pair_width == 64 ? encode_halo_maps_tile<PairTile<Q>>(d, d->maps)
-                                       : encode_halo_maps_tile<NarrowTile<Q>>(d, d->maps);
-    return d->fp64 ? encode_halo_maps<Q, kSingleTile<double>>(d, d->maps)
-                   : encode_halo_maps<Q, kSingleTile<float>>(d, d->maps);
+    CUtensorMap m[3];
+    if (!(!d->cfg.pair ? encode_halo_maps<Q, 0>(d, m)
+          : d->cfg.pair_width == 64 ? encode_halo_maps_tile<PairTile<Q>>(d, m)
+                                    : encode_halo_maps_tile<NarrowTile<Q>>(d, m)))
+        return false;
+    d->tm_phi = m[0];
+    d->tm_u[0] = m[1];
+    d->tm_u[1] = m[2];
+    return true;
 }
 
 // The maps of tile shape V for a domain of lattice Q (the batch's tables).
-bool encode_halo_maps_any(const lbm_domain* d, int V, HaloMaps& out) {
+bool encode_halo_maps_any(const lbm_domain* d, int V, CUtensorMap out[3]) {
     if (d->prm.lattice == 9) {
         switch (V) {
         case 0: return encode_halo_maps<9, 0>(d, out);
@@ -737,12 +721,6 @@ lbm_status check_err_flag(lbm_domain* d) {
     if (h & kErrBounds)
         return fail(d, LBM_ERR_BOUNDS, "a step kernel computed an index outside its array (access skipped)");
     if (h) return fail(d, LBM_ERR_UNSTABLE, "a step produced a non-finite velocity");
-    return LBM_OK;
-}
-
-// The color was set: nothing is left below its last place.
-lbm_status clear_phi_lo(lbm_domain* d) {
-    if (!d->fp64) CUDA_TRY(d, cudaMemsetAsync(d->phi_lo(), 0, (size_t)d->lay.plane * d->lay.elem, d->stream));
     return LBM_OK;
 }
 
@@ -890,34 +868,19 @@ lbm_status init_state(lbm_domain* d, int mode, const double ctr[3], double R0) {
     // (init_pops) and the velocity of the first step's stencil, 0.  Population
     // slots of non-fluid nodes are never read (every pull of a fluid node reads
     // a fluid source or the node's own slots, as the diagnostics and state
-    // transfer do), the second velocity and color buffers and the flux are written
-    // at every fluid node by the first step, and the velocity of non-fluid nodes stays 0 from the
+    // transfer do), the second velocity buffer is written at every fluid node
+    // by the first step, and the velocity of non-fluid nodes stays 0 from the
     // domain's creation (no kernel writes it but as 0).  So of the state only
     // the first velocity buffer and p (state read back as 0 before a step) are
     // cleared.
     CUDA_TRY(d, cudaMemsetAsync(d->errflag(), 0, sizeof(int), d->stream));
     CUDA_TRY(d, cudaMemsetAsync(d->U(0), 0, (size_t)L.D * L.plane * L.elem, d->stream));
     CUDA_TRY(d, cudaMemsetAsync(d->p(), 0, (size_t)L.plane * L.elem, d->stream));
-    lbm_status st = clear_phi_lo(d);
-    if (st != LBM_OK) return st;
     dispatch(d, [&](auto Lx) {
-        decltype(Lx)::init_phi(d->cfg, d->cls(), d->phi(0), mode, ctr, R0, ghost_value, d->stream);
-        decltype(Lx)::init_pops(d->cfg, d->cls(), d->phi(0), d->N(0), d->B(), d->stream);
-    });
-    d->b_stored = true;
-    CUDA_TRY(d, cudaGetLastError());
-    return LBM_OK;
-}
-
-// Makes the buffer B() hold the current B.  After a step it follows from the
-// color that step read (the other color buffer), its N* and its flux.
-lbm_status store_B(lbm_domain* d) {
-    if (d->b_stored) return LBM_OK;
-    dispatch(d, [&](auto Lx) {
-        decltype(Lx)::rebuild_B(d->cfg, d->cls(), d->phi(1 - d->cur), d->N(d->cur), d->flux(), d->B(), d->stream);
+        decltype(Lx)::init_phi(d->cfg, d->cls(), d->phi(), mode, ctr, R0, ghost_value, d->stream);
+        decltype(Lx)::init_pops(d->cfg, d->cls(), d->phi(), d->N(0), d->B(0), d->stream);
     });
     CUDA_TRY(d, cudaGetLastError());
-    d->b_stored = true;
     return LBM_OK;
 }
 
@@ -1001,20 +964,24 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     c.eps = -(4.0 / P.W) * std::cos(P.theta);
     c.exp_eps = std::exp(c.eps);
     c.ghost_rule = P.ghost_rule;
-    // Float arithmetic: the two-node kernels (half the load and store
-    // instructions per node of the one-node kernels; 192^3 319 us per step
-    // against 349 with FP32 and 252 against 313 with FP16 storage).
-    // LBM_STEP_KERNEL=pair|single overrides; both give the same results to the bit.
+    // Float arithmetic: the two-node step kernel (half the load/store and
+    // address instructions per node of the one-node kernel; at 192^3 0.967
+    // against 0.919 of the measured copy peak with FP32 storage, 0.667 against
+    // 0.658 of its roofline with FP16 storage).  LBM_STEP_KERNEL=pair|single
+    // overrides; both kernels give the same results to the bit.
     const char* step_kernel = std::getenv("LBM_STEP_KERNEL");
     c.pair = P.precision != LBM_FP64 && (step_kernel == nullptr || std::strcmp(step_kernel, "pair") == 0);
 
     // 64-node tiles hold fewer idle lanes at row ends per block and cost less
     // per lane; a 3D grid whose rows 32-wide tiles cover with 1/6 fewer lanes
     // (nx = 65..96, 129..160) runs faster on those.  us per step, 64 against 32
-    // wide, FP32: 70^3 28.9 / 27.1, 96^3 51.5 / 49.6, 65 x 120 x 40 28.2 / 26.1;
-    // 100^3 60.0 / 63.0, 128^3 102 / 105, 192^3 316 / 323, 2D 600^2 12.0 / 12.3.
+    // wide, FP16 storage: 70^3 23.4 / 20.9, 96^3 41.3 / 37.4, 65 x 120 x 40 22.5 /
+    // 20.4, 160 x 90 x 90 54.2 / 51.4 (FP32: 26.9 / 26.4, 51.9 / 50.5, 25.6 / 25.8,
+    // 72.2 / 71.8); 100^3 46.7 / 51.6, 128^3 78.0 / 80.9, 192^3 234 / 243, 2D
+    // 1000 x 600 FP32 16.0 / 16.8.
     auto covered = [&](int w) { return (P.nx + w - 1) / w * w; };
     c.pair_width = L.D == 3 && 6 * covered(32) <= 5 * covered(64) ? 32 : 64;
+
     // node classes, as row bit masks on the host (the device expands them)
     const int64_t nn = L.nn_dense;
     const int64_t nx = P.nx, ny = P.ny, nz = P.nz;
@@ -1115,14 +1082,13 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     uint64_t* dF = d->at<uint64_t>(L.off_stage);
     uint64_t* dG = dF + d->fluid_bits.size();
     if (2 * bits_bytes > 2 * (size_t)L.plane * L.elem) return bail("row bit masks do not fit the staging planes");
-    // zero the fields from the first color on (u must stay 0 at non-fluid
-    // nodes); the flux and the second color are written by the first step
-    // before anything reads them, and the population buffers are left as they are: lbm_init_* writes every fluid
+    // zero the fields from phi on (u must stay 0 at non-fluid nodes); the
+    // population buffers are left as they are: lbm_init_* writes every fluid
     // node's slots of the first ones, the first step those of the second ones,
     // and no pull of a fluid node reads a non-fluid node's slots (the step
     // kernels load them for non-fluid lanes, whose results are never stored
     // as state: u and p get 0 there, the populations values nothing reads)
-    if (cudaMemsetAsync(d->ws + L.off_phi[0], 0, L.total - L.off_phi[0], s) != cudaSuccess)
+    if (cudaMemsetAsync(d->ws + L.off_phi, 0, L.total - L.off_phi, s) != cudaSuccess)
         return bail("cudaMemset failed");
     if (cudaMemcpyAsync(dF, d->fluid_bits.data(), bits_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess ||
         cudaMemcpyAsync(dG, d->ghost_bits.data(), bits_bytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
@@ -1166,7 +1132,7 @@ lbm_status lbm_init_droplet(lbm_domain* d, const double centre[3], double R0) {
 lbm_status lbm_init_phi(lbm_domain* d, const double* phi_host) {
     if (!d || !phi_host) return fail(d, LBM_ERR_ARG, "NULL argument");
     if (d->poisoned) return fail(d, LBM_ERR_TIMEOUT, kPoisonedMsg);
-    lbm_status st = upload(d, d->phi(0), phi_host, d->lay.nn_dense);
+    lbm_status st = upload(d, d->phi(), phi_host, d->lay.nn_dense);
     if (st != LBM_OK) return st;
     const double zero[3] = {0, 0, 0};
     return init_state(d, 1, zero, 1.0);
@@ -1176,7 +1142,6 @@ lbm_status lbm_step(lbm_domain* d, int64_t n) {
     if (!d) return fail(d, LBM_ERR_ARG, "NULL domain");
     if (n < 0) return fail(d, LBM_ERR_ARG, "n must be >= 0");
     if (d->poisoned) return fail(d, LBM_ERR_TIMEOUT, kPoisonedMsg);
-    if (n > 0) d->b_stored = false;
     while (n > 0) {
         if (d->cur == 0 && n >= GRAPH_STEPS) {
             CUDA_TRY(d, cudaGraphLaunch(d->g8, d->stream));
@@ -1199,7 +1164,6 @@ lbm_status lbm_profile_steps(lbm_domain* d, int64_t n, double kernel_ms[3]) {
     cudaEvent_t ev[4];
     for (int k = 0; k < 4; ++k) CUDA_TRY(d, cudaEventCreate(&ev[k]));
     lbm_status st = LBM_OK;
-    d->b_stored = false;
     for (int64_t t = 0; t < n && st == LBM_OK; ++t) {
         launch_one_step(d, d->cur, d->stream, ev);
         cudaError_t e = cudaGetLastError();
@@ -1238,7 +1202,7 @@ lbm_status lbm_diagnostics(lbm_domain* d, const lbm_probe* probe, lbm_diag* out)
     double* partial = d->at<double>(L.off_partial);
     double* dout = d->at<double>(L.off_dout);
     dispatch(d, [&](auto Lx) {
-        decltype(Lx)::diag(d->cfg, d->mask(), d->N(d->cur), d->phi(d->cur), d->U(d->cur), d->p(), pr, partial, dout,
+        decltype(Lx)::diag(d->cfg, d->mask(), d->N(d->cur), d->phi(), d->U(d->cur), d->p(), pr, partial, dout,
                            d->stream);
     });
     CUDA_TRY(d, cudaGetLastError());
@@ -1303,11 +1267,7 @@ lbm_status lbm_read_state(lbm_domain* d, int32_t field, double* host_out) {
     case LBM_FIELD_N:
     case LBM_FIELD_B: {
         const bool is_b = field == LBM_FIELD_B;
-        if (is_b) {
-            lbm_status r = store_B(d);
-            if (r != LBM_OK) return r;
-        }
-        void* st = is_b ? d->B() : d->N(d->cur);
+        void* st = is_b ? d->B(d->cur) : d->N(d->cur);
         void* stage = d->at<void>(L.off_stage);
         for (int i = 0; i < L.Q; ++i) {
             double base = 0.0;
@@ -1325,7 +1285,7 @@ lbm_status lbm_read_state(lbm_domain* d, int32_t field, double* host_out) {
         return LBM_OK;
     }
     case LBM_FIELD_PHI:
-        return download(d, host_out, d->phi(d->cur));
+        return download(d, host_out, d->phi());
     case LBM_FIELD_U: {
         if (L.D == 2) std::fill(host_out + 2 * nn, host_out + 3 * nn, 0.0);
         return download(d, host_out, d->U(d->cur), L.D);
@@ -1345,13 +1305,7 @@ lbm_status lbm_write_state(lbm_domain* d, int32_t field, const double* host_in) 
     case LBM_FIELD_N:
     case LBM_FIELD_B: {
         const bool is_b = field == LBM_FIELD_B;
-        if (is_b) {
-            d->b_stored = true;
-        } else {                                   // B follows from the N that is replaced here
-            lbm_status r = store_B(d);
-            if (r != LBM_OK) return r;
-        }
-        void* st = is_b ? d->B() : d->N(d->cur);
+        void* st = is_b ? d->B(d->cur) : d->N(d->cur);
         char* stage = d->at<char>(L.off_stage);
         std::vector<double> dev_i((size_t)nn), dev_o((size_t)nn);
         for (int i = 0; i < L.Q; ++i) {
@@ -1375,10 +1329,8 @@ lbm_status lbm_write_state(lbm_domain* d, int32_t field, const double* host_in) 
         CUDA_TRY(d, cudaStreamSynchronize(d->stream));
         return LBM_OK;
     }
-    case LBM_FIELD_PHI: {
-        lbm_status s = clear_phi_lo(d);
-        return s != LBM_OK ? s : upload(d, d->phi(d->cur), host_in, nn);
-    }
+    case LBM_FIELD_PHI:
+        return upload(d, d->phi(), host_in, nn);
     case LBM_FIELD_U: {
         // the velocity of a non-fluid node is 0 whatever the caller passes: the
         // stencils read it there as the wall's velocity
@@ -1420,14 +1372,13 @@ double lbm_bytes_per_fluid_node(const lbm_domain* d) {
     const double s = (double)d->lay.elem;
     const double moving = (d->lay.Q - 1) * (double)d->lay.pop_elem;
     const double pop = (double)d->lay.rest_elem + moving;   // per node and array
-    // the two-population scheme's count, not the kernels' (which make B from N*,
-    // phi and the flux: 304 bytes in D3Q19 FP32 with density contrast against
-    // 344 here): N pulled, N* and B* written, B* pulled; in FP64 with the rest
-    // population's pull
+    // k_step pulls N: the FP64 update follows the literal collision and reads the
+    // rest population, the float updates take every moment from the moving ones
     const double pull = d->lay.elem == 8 ? pop : moving;
     const int D = d->lay.D;
-    // phi written and read; u written, and read when the density contrast makes
-    // F_visc active; p written; the 4-byte bounce-back mask read twice
+    // N* and B* written, B* pulled by k_phi; phi written (k_phi) and read (k_step);
+    // u written, and read when the density contrast makes F_visc active; p written; the 4-byte
+    // bounce-back mask read by k_step and k_phi
     return pull + 3.0 * pop + 2.0 * s + (d->contrast ? 2.0 : 1.0) * D * s + s + 8.0;
 }
 
@@ -1494,19 +1445,21 @@ struct lbm_batch {
     std::vector<int> cur0;             // each domain's buffer parity when the batch was made
     int parity = 0;                    // steps taken by the batch, mod 2
     int variant = 0;
-    // tile shape of the color kernel, -1: the step kernels'.  Float: shape 0 or
-    // 5, the two-node kernel's 32- or 64-wide tiles, whichever covers the
-    // domains' rows with fewer lanes (shape 5 if they are within 10%: it costs
-    // 3% less per lane).  Twelve ragged domains of 50^3 to 93^3: 304 us per step
-    // on shape 0 against 319 on shape 5 with the step on shape 5.
-    int color_shape = -1;
+    // tiles of the color kernel, whatever shape the step kernels use (it has
+    // no halo): row chunks of 128 nodes (kPhiRows), which leave only the
+    // padding columns idle.  LBM_BATCH_PHI_SHAPE=step: the step's shape;
+    // =0..5: that shape (shape 3, 32 x 2 x 2, ran a batch of 64 domains of 48^3 to 128^3 at 3.305 ms per
+    // step against 3.331 on the step's 64-wide tiles).
+    int phi_shape = kPhiRows;
+    int4* phi_rows = nullptr;          // {slot, x0, y0, z} row chunks
+    int nphi_rows = 0;
     int ntiles[kTileVariants] = {};
     int ncontrast[kTileVariants] = {};           // tiles of domains with density contrast come first
     int device = 0;
     std::vector<int> slots;            // each domain's slot of the constant table
     char* dev = nullptr;               // one allocation for every device table
     int4* tiles[kTileVariants] = {};             // {slot, x0, y0, z0}
-    CUtensorMap* maps = nullptr;                 // [kTileVariants][kBatchSlots][kSlotMaps] halo maps by shape and slot
+    CUtensorMap* maps = nullptr;                 // [kTileVariants][kBatchSlots][3] halo maps by shape and slot
     void* ghost_tabs = nullptr;
     int64_t* ghost_begin = nullptr;
     int64_t total_ghosts = 0;
@@ -1571,12 +1524,12 @@ void batch_launch_step(lbm_batch* b, int parity, cudaStream_t s) {
     const int V = b->variant;
     bdispatch(b->precision, [&](auto Lx) {
         using L = decltype(Lx);
-        const int Vc = b->color_shape < 0 ? V : b->color_shape;
-        const size_t per_shape = (size_t)kBatchSlots * kSlotMaps;
-        L::ghost_batched(b->GK, b->ghost_tabs, b->ghost_begin, (int)b->doms.size(), b->total_ghosts, parity, s);
-        L::step_batched(b->Q, V, b->tiles[V], b->maps + V * per_shape, b->ntiles[V], b->ncontrast[V], parity, s);
-        L::color_batched(b->Q, Vc, b->tiles[Vc], b->maps + Vc * per_shape, b->ntiles[Vc], parity,
-                         b->total_ghosts > 0, s);
+        L::ghost_batched(b->GK, b->ghost_tabs, b->ghost_begin, (int)b->doms.size(), b->total_ghosts, s);
+        const int Vp = b->phi_shape < 0 ? V : b->phi_shape;
+        const int4* pt = Vp == kPhiRows ? b->phi_rows : b->tiles[Vp];
+        const int np = Vp == kPhiRows ? b->nphi_rows : b->ntiles[Vp];
+        L::step_phi_batched(b->Q, V, b->tiles[V], b->maps + (size_t)V * kBatchSlots * 3, b->ntiles[V],
+                            b->ncontrast[V], Vp, pt, np, parity, b->total_ghosts > 0, s);
     });
 }
 
@@ -1633,6 +1586,11 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         b->cur0.push_back(doms[i]->cur);
     }
     b->stream = (cudaStream_t)cuda_stream;
+    const char* phi_shape = std::getenv("LBM_BATCH_PHI_SHAPE");
+    if (phi_shape && std::strcmp(phi_shape, "step") == 0) b->phi_shape = -1;
+    else if (phi_shape && std::strcmp(phi_shape, "rows") == 0) b->phi_shape = kPhiRows;
+    else if (phi_shape && phi_shape[0] >= '0' && phi_shape[0] < '0' + kTileVariants && !phi_shape[1])
+        b->phi_shape = phi_shape[0] - '0';
     if (n > kBatchSlots) {
         delete b;
         return bfail(nullptr, LBM_ERR_ARG, "a batch holds at most " + std::to_string(kBatchSlots) + " domains");
@@ -1650,25 +1608,22 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         using L = decltype(Lx);
         esz = L::entry_size(); gsz = L::ghost_table_size();
     });
-    // halo maps by tile shape and slot: the color and u_in of step parity 0 and
-    // 1 (buffers cur0 ^ parity), then the flux, each with the box of that
-    // shape's halo tile
-    std::vector<CUtensorMap> hm((size_t)kTileVariants * kBatchSlots * kSlotMaps);
+    // halo maps by tile shape and slot: phi, then u_in of step parity 0 and 1
+    // (u_in = U(cur0 ^ parity)), each with the box of that shape's halo tile
+    std::vector<CUtensorMap> hm((size_t)kTileVariants * kBatchSlots * 3);
     std::vector<char> slot_tma(kBatchSlots, 0);
     for (int i = 0; i < n; ++i) {
         lbm_domain* d = b->doms[i];
         if (!d->tma) continue;
-        const int sl = b->slots[i], c0 = b->cur0[i];
+        const int sl = b->slots[i];
         bool ok = true;
         for (int V = 0; V < kTileVariants && ok; ++V) {
-            HaloMaps m;
+            CUtensorMap m[3];
             ok = encode_halo_maps_any(d, V, m);
-            CUtensorMap* dst = &hm[((size_t)V * kBatchSlots + sl) * kSlotMaps];
-            dst[0] = m.phi[c0];
-            dst[1] = m.phi[c0 ^ 1];
-            dst[2] = m.u[c0];
-            dst[3] = m.u[c0 ^ 1];
-            dst[4] = m.flux;
+            CUtensorMap* dst = &hm[((size_t)V * kBatchSlots + sl) * 3];
+            dst[0] = m[0];
+            dst[1] = m[1 + b->cur0[i]];
+            dst[2] = m[1 + (b->cur0[i] ^ 1)];
         }
         slot_tma[sl] = ok;                       // a slot uses its maps only if every shape's encoded
     }
@@ -1681,11 +1636,15 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         bdispatch(b->precision, [&](auto Lx) {
             using LL = decltype(Lx);
             StepPtrs sp[2];
-            for (int k = 0; k < 2; ++k) sp[k] = step_ptrs(d, b->cur0[i] ^ k);
-            void* const phi[2] = {d->phi(b->cur0[i]), d->phi(b->cur0[i] ^ 1)};
+            for (int k = 0; k < 2; ++k) {
+                const int c = b->cur0[i] ^ k;
+                sp[k].Nin = d->N(c); sp[k].Bin = d->B(c); sp[k].Nout = d->N(1 - c); sp[k].Bout = d->B(1 - c);
+                sp[k].phi = d->phi(); sp[k].u_in = d->U(c); sp[k].u_out = d->U(1 - c); sp[k].p = d->p();
+                sp[k].mask = d->mask(); sp[k].err = d->errflag();
+            }
             LL::fill_entry(&he[esz * i], d->cfg, sp, slot_tma[b->slots[i]] != 0);
             LL::fill_ghost_table(&hg[gsz * i], d->ng, d->at<int32_t>(L.off_gnode), d->at<int32_t>(L.off_gcorner),
-                                 d->at<void>(L.off_gwt), d->cfg.exp_eps, d->cfg.eps, phi, d->cfg.ghost_rule,
+                                 d->at<void>(L.off_gwt), d->cfg.exp_eps, d->cfg.eps, d->phi(), d->cfg.ghost_rule,
                                  L.plane, d->errflag());
         });
         gbegin[i + 1] = gbegin[i] + d->ng;
@@ -1699,12 +1658,14 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
                 if (pass == 0) b->ncontrast[V] = (int)tiles[V].size();
             }
         }
-    if (b->precision != LBM_FP64) {
-        const int64_t lanes0 = (int64_t)tiles[0].size() * tile_extent(b->Q, 0, 0) * tile_extent(b->Q, 0, 1) *
-                               tile_extent(b->Q, 0, 2);
-        const int64_t lanes5 = (int64_t)tiles[5].size() * tile_extent(b->Q, 5, 0) * tile_extent(b->Q, 5, 1) *
-                               tile_extent(b->Q, 5, 2);
-        b->color_shape = 10 * lanes0 <= 9 * lanes5 ? 0 : 5;
+    // row chunks of the color kernel, domain by domain, plane by plane
+    std::vector<int4> rows;
+    for (int i = 0; i < n; ++i) {
+        const lbm_params& P = b->doms[i]->prm;
+        const int64_t px = b->doms[i]->lay.px, per_plane = px * P.ny;
+        for (int z = 0; z < P.nz; ++z)
+            for (int64_t o = 0; o < per_plane; o += kPhiChunk)
+                rows.push_back(make_int4(b->slots[i], (int)(o % px), (int)(o / px), z));
     }
     b->total_ghosts = gbegin[n];
     size_t off = 0;
@@ -1719,6 +1680,11 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         }
         o_t[V] = take(tiles[V].size() * sizeof(int4));
     }
+    if (rows.size() > (size_t)INT32_MAX) {
+        lbm_batch_destroy(b);
+        return bfail(nullptr, LBM_ERR_ARG, "too many tiles");
+    }
+    const size_t o_r = take(rows.size() * sizeof(int4));
     if (cudaMalloc((void**)&b->dev, off) != cudaSuccess) {
         cudaGetLastError();
         lbm_batch_destroy(b);
@@ -1736,6 +1702,11 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         b->tiles[V] = (int4*)(b->dev + o_t[V]);
         b->ntiles[V] = (int)tiles[V].size();
         e = cudaMemcpy(b->tiles[V], tiles[V].data(), tiles[V].size() * sizeof(int4), cudaMemcpyHostToDevice);
+    }
+    if (e == cudaSuccess) {
+        b->phi_rows = (int4*)(b->dev + o_r);
+        b->nphi_rows = (int)rows.size();
+        e = cudaMemcpy(b->phi_rows, rows.data(), rows.size() * sizeof(int4), cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
@@ -1772,7 +1743,6 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
     for (auto* d : b->doms) {
         d->step += n;
         if (n & 1) d->cur ^= 1;
-        if (n > 0) d->b_stored = false;
     }
     return LBM_OK;
 }
@@ -1823,11 +1793,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int32_t steps_per_trial, int32_t* chosen
         if (ms_per_step) ms_per_step[V] = per;
         if (per < best) { best = per; best_v = V; }
         const int64_t taken = steps_per_trial + 1;
-        for (auto* d : b->doms) {
-            d->step += taken;
-            d->b_stored = false;
-            if (taken & 1) d->cur ^= 1;
-        }
+        for (auto* d : b->doms) { d->step += taken; if (taken & 1) d->cur ^= 1; }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

@@ -167,38 +167,6 @@ __global__ void k_init_pops(Dims d, StepParams<T> P, const uint8_t* __restrict__
     }
 }
 
-// The populations B* of the last step in storage form, for state transfer: the
-// step keeps only what makes them, B*_i = phi N*_i + w_i c_i . f (phi the color
-// that step read).  With FP16 storage the float rest population takes the node
-// total phi - 1/2 less the rounded moving ones.
-template <int Q, typename T, typename S>
-__global__ void k_rebuild_B(Dims d, StepParams<T> P, const uint8_t* __restrict__ cls, const T* __restrict__ phi,
-                            const S* __restrict__ Nst, const T* __restrict__ flux, S* __restrict__ Bst) {
-    using L = Lattice<Q>;
-    using PS = PopStore<S>;
-    const int nn = (int)padded_nodes(d), pl = (int)d.plane;
-    for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < nn; node += gridDim.x * blockDim.x) {
-        if (cls[node] != CLS_FLUID) continue;
-        const T ph = phi[node], base = PS::kShiftB ? ph - T(0.5) : ph;      // chi_i's factor
-        T sum = T(0);
-#pragma unroll
-        for (int i = Q - 1; i >= 0; --i) {
-            T b = base * P.chi[i] + ph * pop_load<Q, S, T>(Nst, i, pl, node, kScaleN);
-            if (i > 0) {
-                T cf = T(0);
-                if (L::cx(i)) cf += T(L::cx(i)) * flux[node];
-                if (L::cy(i)) cf += T(L::cy(i)) * flux[pl + node];
-                if (L::D == 3 && L::cz(i)) cf += T(L::cz(i)) * flux[2 * pl + node];
-                b += T(L::w(i)) * cf;
-            } else if (!PS::kExact) {
-                b = base - sum;
-            }
-            pop_store<Q, S, T>(Bst, i, pl, node, b, kScaleB);
-            if (!PS::kExact && i > 0) sum += T(__half2float(__float2half_rn(float(b) * kScaleB)) / kScaleB);   // as stored
-        }
-    }
-}
-
 // One direction i of post-streaming values -> pull layout: st_i[y] = post_i[y + c_i]
 // if y + c_i is fluid, else post_opp[y]; stored as value - base (base = 0, chi_i or chi_i/2).
 template <int Q, typename T, typename S>

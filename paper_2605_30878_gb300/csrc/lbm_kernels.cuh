@@ -8,14 +8,6 @@
 //     N_i(x) = N*_opp(i)(x)         otherwise (halfway bounce-back, walls at rest),
 // which is Eqs. (propTotal)/(propBlue) with bounce-back on the staircase solid.
 //
-// B is not stored.  The segregation step makes it from values that the step
-// stores anyway and one vector: with w_i the lattice weights and kappa =
-// chi_i / w_i (the same for every moving direction),
-//     B*_i(y) = phi(y) N*_i(y) + w_i c_i . f(y),
-//     f = (2/W) phi (1 - phi) (kappa + 3 p) grad phi / max(|grad phi|, 1e-6),
-// so the step stores the recolouring flux f (D values) in the place of the Q
-// values of B*, and the color kernel sums the pulled B* from N*, phi and f.
-//
 // One time step is three launches on one stream:
 //   k_ghost  Eq. (ghost-nodePrescription) at every ghost node, from the color
 //            of the fluid corners of x_F (weights precomputed on the host)
@@ -23,11 +15,9 @@
 //            the previous velocity) from a shared-memory halo tile; forces of
 //            Eqs. (surfaceTensionForce), (pressCorrection), (viscCorrection),
 //            (totalForce); u, p of Eqs. (velUpdate), (pressureUpdate);
-//            collision of Eq. (MRTCOLL) in closed form; the recolouring flux
-//            of Eq. (segragationStepBlue); write N*, f, u, p at the node
-//   k_color  Eq. (phiUpdate): sum the pulled B*_i = phi N*_i + w_i c_i . f at
-//            every fluid node, phi and f from a shared-memory halo tile; the
-//            new color goes to a second buffer
+//            collision of Eq. (MRTCOLL) in closed form; segregation of Eq.
+//            (segragationStepBlue); write N*, B*, u, p at the node
+//   k_phi    Eq. (phiUpdate): pull B* and sum it at every fluid node
 //
 // Fields are structure-of-arrays with a plane stride `plane` (a multiple of 64
 // elements): field[a * plane + node]; populations are grouped (pop_at).
@@ -66,7 +56,6 @@ struct StepParams {
     // pressure's zero are taken at the exact chi through these corrections
     T chi_err[3];
     T c2chi;                 // sum_i chi_i c_ix^2 = (1-alpha) c_s^2/(1-w_0)
-    T kappa;                 // chi_i / w_i of the moving directions, (1-alpha)/(1-w_0)
     T exp_eps;               // exp(eps), eps = -(4/W) cos(theta)
 };
 
@@ -74,8 +63,8 @@ struct StepParams {
 // N_i - chi_i, in every mode; the step computes directly in these deviations,
 // an exact rewrite because sum chi = 1, sum c chi = 0 and chi is isotropic, and
 // it keeps the small pressure of a dense liquid (p = p_h/rho ~ 1e-8 at density
-// ratio 1000) representable.  B, kept for state transfer only: full values in
-// S = double (FP64 mode), B_i - chi_i/2 in S = float (FP32 mode).  S = __half: the same deviations, the rest
+// ratio 1000) representable.  B: full values in S = double (FP64 mode),
+// B_i - chi_i/2 in S = float (FP32 mode).  S = __half: the same deviations, the rest
 // populations (i = 0, whose B deviation reaches chi_0/2 ~ 0.46) as float in the
 // first plane, the moving ones times 2^16 (N) and 2^7 (B) as FP16 after it.
 constexpr float kScaleN = 65536.0f;
@@ -95,9 +84,12 @@ __device__ __forceinline__ float add_f16_f32(__half h, float c) {
 // parts.  Moving populations lie in groups of 64 nodes, the Q - 1 directions of
 // a group one after the other: direction d >= 1 of a node is element
 // pop_at<Q>(node) + pop_dir(d).  A thread's 18 values of a node then share one
-// address but for a constant (planes of their own, millions of bytes apart,
-// cost every load and store a 64-bit address of its own), rows still load and
-// store as 256-byte runs, and a node's 19 values share a DRAM page.
+// address but for a constant, where planes of their own, millions of bytes
+// apart, cost every load and store a 64-bit address of its own; rows still load
+// and store as 256-byte runs, and a node's 19 values share a DRAM page.  192^3
+// with FP16 storage, whose step is bound by its instructions: 269 us per step
+// with planes, 234 so, together with H2's halo values and the two-node color
+// kernel.
 constexpr int kGroup = 64;
 template <int Q> __host__ __device__ constexpr unsigned pop_at(int node) {
     return (unsigned)node + ((unsigned)node / kGroup) * (kGroup * (Q - 2));
@@ -119,6 +111,7 @@ template <typename V> struct PlainStore {
     __device__ static void store_moving(V* m, int idx, V v, float) { m[idx] = v; }
     // in storage units: the value itself
     __device__ static V load_units(const V* m, int idx) { return __ldg(m + idx); }
+    __device__ static void accumulate(const V* m, int idx, V& acc) { acc += __ldg(m + idx); }
     // stores v; exact storage leaves nothing to account for, acc is untouched
     __device__ static void store_units(V* m, int idx, V v, V&) { m[idx] = v; }
 };
@@ -134,15 +127,11 @@ template <> struct PopStore<float> : PlainStore<float> {
     __device__ static void store_units2(float* m, int idx, float va, float vb, float&, float&) {
         *reinterpret_cast<float2*>(m + idx) = make_float2(va, vb);
     }
-    __device__ static float2 load_rest2(const float* r, int idx) {
-        return __ldg(reinterpret_cast<const float2*>(r + idx));
-    }
     __device__ static void store_zero2(float* m) { *reinterpret_cast<float2*>(m) = make_float2(0.f, 0.f); }
 };
 template <> struct PopStore<__half> {
     static constexpr bool kShift = true, kShiftB = true, kExact = false;     // moving populations are rounded on store
     static constexpr int kRestBytes = 4, kMovingBytes = 2;
-    using Moving = __half;
     __device__ static const float* rest(const __half* p) { return reinterpret_cast<const float*>(p); }
     __device__ static float* rest(__half* p) { return reinterpret_cast<float*>(p); }
     __device__ static const __half* moving(const __half* p, int plane) { return p + 2 * plane; }
@@ -158,6 +147,7 @@ template <> struct PopStore<__half> {
     // in storage units (value x scale): the step kernels fold the power-of-two
     // scales into their arithmetic instead of scaling every population
     __device__ static float load_units(const __half* m, int idx) { return __half2float(__ldg(m + idx)); }
+    __device__ static void accumulate(const __half* m, int idx, float& acc) { acc = add_f16_f32(__ldg(m + idx), acc); }
     // stores v (already scaled) and adds the value stored to acc
     __device__ static void store_units(__half* m, int idx, float v, float& acc) {
         const __half h = __float2half_rn(v);
@@ -166,9 +156,6 @@ template <> struct PopStore<__half> {
     }
     // two adjacent nodes (idx even, so 4-byte aligned): one 32-bit load or
     // store for both, each value rounded as store_units rounds it
-    __device__ static float2 load_rest2(const float* r, int idx) {
-        return __ldg(reinterpret_cast<const float2*>(r + idx));
-    }
     __device__ static float2 load_units2(const __half* m, int idx) {
         return __half22float2(__ldg(reinterpret_cast<const __half2*>(m + idx)));
     }
@@ -197,14 +184,13 @@ __device__ __forceinline__ void pop_store(S* p, int d, int plane, int node, V v,
 template <typename T, typename S>
 struct StepBuffers {
     const S* Nin;
+    const S* Bin;
     S* Nout;
-    const T* phi;            // color the step reads, ghost nodes included
-    T* phi_out;              // color after the step
-    T* phi_lo;               // float: the part of the color below its last place, see color_update
+    S* Bout;
+    T* phi;
     const T* u_in;           // velocity of the previous step (F_visc stencil)
     T* u_out;
     T* p;
-    T* flux;                 // recolouring flux f of the step
     const uint32_t* mask;    // per-node bounce-back mask, see MASK_NOT_FLUID
     int* err;                // bit 0: non-finite value seen
 };
@@ -212,7 +198,6 @@ struct StepBuffers {
 // Per-node mask: bit i (1 <= i < Q) is set when x - c_i is not a fluid node,
 // so the pull in direction i bounces back; MASK_NOT_FLUID marks non-fluid x.
 constexpr uint32_t MASK_NOT_FLUID = 0x80000000u;
-constexpr uint32_t MASK_DIRS = 0x0007fffeu;
 
 // Block tiles of the step kernels in the shapes the batch autotuner chooses
 // between (V = 0 is the float one-node single-domain kernel's tile, V = 3 that
@@ -226,6 +211,8 @@ constexpr uint32_t MASK_DIRS = 0x0007fffeu;
 // (k_step_pair_batched, PairTile: two x-adjacent nodes per thread); shape 5 is
 // also the tile of the single-domain two-node kernel (k_step_pair).
 constexpr int kTileVariants = 6;
+constexpr int kPhiRows = kTileVariants;     // the batch color kernel on row chunks (k_phi_rows_batched)
+constexpr int kPhiChunk = 128;              // nodes per block of the color kernels over row chunks
 __host__ __device__ constexpr int tile_extent(int Q, int V, int axis) {
     return V == 5 ? (axis == 0 ? 64 : axis == 1 ? (Q == 9 ? 4 : 2) : (Q == 9 ? 1 : 2))
          : Q == 9 ? (axis == 0 ? (V == 1 ? 64 : (V == 2 ? 128 : 32))
@@ -306,12 +293,9 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // it, so "the kernel before" covers all earlier ones.  The next kernel may start
 // from pdl_trigger() on, or as this one's blocks end.  Only a kernel that the
 // ghost kernel follows (the color kernel of a domain with ghost nodes) and the
-// ghost kernel itself trigger at once: the blocks of a large successor would
-// hold room beside a running kernel (us per step: step kernels triggering too,
-// 49 x 52 x 47 15.2 against 13.1, 64^3 FP64 260 against 248; a color kernel that
-// the step kernel follows, 192^3 without ghost nodes 436 against 316).  Without
-// programmatic launches: 49 x 52 x 47 14.9, 401^2 9.4 against 7.9, 128^3 packing
-// 112 against 108, 16 batched 2D domains 48 against 45.
+// ghost kernel itself trigger at once: the blocks of a large successor hold
+// room beside a running kernel (64^3 FP64 260 us per step against 248 with step
+// kernels that trigger too).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -432,6 +416,56 @@ __device__ __forceinline__ void load_halo(const StepParams<T>& P, const T* __res
 }
 
 // ---------------------------------------------------------------------------
+// k_phi: Eq. (phiUpdate) on pulled B* (early: the ghost kernel follows and may
+// start at once).  Bound by DRAM: it reads B* and little else (two nodes per
+// thread in float, k_phi_pair).
+// ---------------------------------------------------------------------------
+template <int Q, typename T, typename S>
+__device__ __forceinline__ void phi_node(const StepParams<T>& P, const S* __restrict__ Bst,
+                                         const uint32_t* __restrict__ mask, T* __restrict__ phi, int x, int y, int z,
+                                         int early, int* err) {
+    using L = Lattice<Q>;
+    const bool in_grid = x < P.nx && y < P.ny && z < P.nz;
+    const int node = in_grid ? idx_checked(x + P.px * (y + P.ny * z), P.plane, err) : 0;
+    const uint32_t m = in_grid ? __ldg(mask + node) : MASK_NOT_FLUID;
+    pdl_wait();
+    if (early) pdl_trigger();
+    if (m & MASK_NOT_FLUID) return;
+    const Wrap W(x, y, z, P.nx, P.ny, P.nz, P.px);
+    const int pl = (int)P.plane;
+    using PS = PopStore<S>;
+    const auto* mv = PS::moving(Bst, pl);
+    // FP64 sums in lattice order, as Eq. (phiUpdate) is written.  The
+    // deviation forms sum the moving populations first, in storage units, and
+    // add the rest population last: with FP16 storage the moving values lie on
+    // a grid coarse enough for their float sum to be exact, so the node's color
+    // comes back as k_step wrote it.
+    const T rest = (T)PS::load_rest(PS::rest(Bst), node);
+    T s = PS::kShiftB ? T(0) : rest;
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        const bool back = (m >> i) & 1u;
+        const int from = idx_checked(back ? node : node + W.off(-L::cx(i), -L::cy(i), -L::cz(i)), P.plane, err);
+        PS::accumulate(mv + pop_at<Q>(from), back ? pop_dir(L::opp(i)) : pop_dir(i), s);
+    }
+    if (PS::kShiftB) s = rest + (PS::kExact ? s : s * T(1.0 / kScaleB));
+    // stored deviations B_i - chi_i/2 sum to phi - 1/2
+    phi[node] = PS::kShiftB ? T(0.5) + s : s;
+}
+
+template <int Q, typename T, typename S>
+__global__ void __launch_bounds__(Tile<Q>::THREADS) k_phi(StepParams<T> P, const S* __restrict__ Bst,
+                                                          const uint32_t* __restrict__ mask, T* __restrict__ phi,
+                                                          int early, int* err) {
+    using Tl = Tile<Q>;
+    // tiles in the reverse of k_step's order: the B* that k_step wrote last is
+    // still in L2 when this kernel starts
+    const int bx = gridDim.x - 1 - blockIdx.x, by = gridDim.y - 1 - blockIdx.y, bz = gridDim.z - 1 - blockIdx.z;
+    phi_node<Q, T, S>(P, Bst, mask, phi, bx * Tl::TX + threadIdx.x, by * Tl::TY + threadIdx.y, bz * Tl::TZ + threadIdx.z,
+                      early, err);
+}
+
+// ---------------------------------------------------------------------------
 // k_ghost: Eq. (ghost-nodePrescription)
 // ---------------------------------------------------------------------------
 // RULE 0: the paper's rule; RULE 1: Eq. (ghostNodeFakhari) multiplied through by
@@ -497,7 +531,7 @@ __device__ __forceinline__ float inv_norm_floor(float g2, float floor) {
 // before the node's mask is known: every direction by streaming (x - c_i
 // always lies in the grid), then the directions whose neighbour is not fluid
 // are read again from the node's own opposite slot.  B enters the collision
-// only through phi = sum B, which k_color computed.  Values come in storage
+// only through phi = sum B, which k_phi computed.  Values come in storage
 // units (times kScaleN with FP16 storage).  In the deviation form the pressure
 // and every moment come from the moving populations (Eq. pressureUpdate), so
 // N[0] is not read.
@@ -651,13 +685,12 @@ template <typename V>
 struct Acc {
     V v = V(typename V::Real(0));
     bool set = false;
-    template <typename T>
-    __device__ __forceinline__ void add(int k, T t) {
+    __device__ __forceinline__ void add(int k, V t) {
         if (k == 0) return;
         if (!set) {
-            v = k == 1 ? V(t) : (k == -1 ? -V(t) : V(typename V::Real(k)) * V(t));
+            v = k == 1 ? t : (k == -1 ? -t : V(typename V::Real(k)) * t);
         } else {
-            v = k == 1 ? v + t : (k == -1 ? v - t : fma(V(typename V::Real(k)), V(t), v));
+            v = k == 1 ? v + t : (k == -1 ? v - t : fma(V(typename V::Real(k)), t, v));
         }
         set = true;
     }
@@ -689,16 +722,20 @@ struct NodeUpdate {
     using R = typename V::Real;
     static constexpr int D = L::D;
     static constexpr double w0 = L::w(0);
-    // storage units: times sN, 2^16 with FP16 storage, else 1.  Being a power of
-    // two, the scale folds into the per-node factors (the stress projections,
-    // the weights) and the scaled values round exactly as the unscaled ones would.
-    static constexpr R sN = UNITS ? kScaleN : 1;
+    // storage units: times sN (N) and sB (B), 2^16 and 2^7 with FP16 storage,
+    // else 1.  Being powers of two, the scales fold into the per-node factors
+    // (the stress projections, the weights, phi, kseg) and the scaled values
+    // round exactly as the unscaled ones would.
+    static constexpr R sN = UNITS ? kScaleN : 1, sB = UNITS ? kScaleB : 1;
+    // B is stored in full in FP64, as its deviation from chi/2 in float
+    static constexpr bool kFullB = sizeof(R) == 8;
     V phi, u[3], uu, p;
     V F[3], gp[3];
     V A0, A1, Axy, Axz, Ayz;                   // stress projections of N - Neq, times (1 - 1/tau)
     V base0, base1, base2, three_p, halfF;
-    V common1, common2;                        // per direction class (1 axis, 2 diagonal/edge)
-    V kflux;                                   // f = kflux grad phi
+    V common1, common2, krc1, krc2;            // per direction class (1 axis, 2 diagonal/edge)
+    V shb1, shb2;                              // (phi - 1/2) chi_i per class, in B's units (FP64: phi chi_i)
+    V phiB;
 
     // raw moments of the pulled N (storage units): sum, first and second moments
     V m_sum, m_u0[3], m_xx, m_yy, m_zz, m_xy, m_xz, m_yz;
@@ -831,26 +868,34 @@ struct NodeUpdate {
         const V g2 = D == 2 ? fma(gp[0], gp[0], gp[1] * gp[1]) : fma(gp[0], gp[0], fma(gp[1], gp[1], gp[2] * gp[2]));
         const V inv_gn = inv_norm_floor(g2, R(1e-6));
         const V kseg = V(P.two_over_W) * phi * (V(R(1.0)) - phi) * inv_gn;
+        const V ksegB = UNITS ? kseg * V(sB) : kseg;                        // recoloring in B's units
+        phiB = UNITS ? phi * V(sB / sN) : phi;                              // phi N*, from N's units to B's
+        const V phmB = kFullB ? phi : (UNITS ? (phi - V(R(0.5))) * V(sB) : phi - V(R(0.5)));
+        shb1 = phmB * V(P.chi[1]);
+        shb2 = phmB * V(P.chi[D == 2 ? 5 : 7]);
         three_p = V(R(3.0)) * p;
         halfF = V(R(1.5)) * inv_rho;   // (1/2) F_i = (3/2) w_i (c_i . F)/rho
         const V common = fma(V(R(-1.5)), uu, three_p);
         // per direction class (1 axis, 2 diagonal/edge): the equilibrium's constant
-        // part w_i (3p - 3u^2/2) + (chi_i - stored chi_i), divided by w_i
+        // part w_i (3p - 3u^2/2) + (chi_i - stored chi_i), divided by w_i, and the
+        // recolouring weight ksegB (chi_i + w_i 3p) with the exact chi_i
         constexpr double kW1 = L::w(1), kW2 = L::w(D == 2 ? 5 : 7);
         common1 = fma(V(P.chi_err[1]), V(R(1.0 / kW1)), common);
         common2 = fma(V(P.chi_err[2]), V(R(1.0 / kW2)), common);
-        kflux = kseg * (V(P.kappa) + three_p);
+        krc1 = ksegB * fma(V(R(kW1)), three_p, V(P.chi[1] + P.chi_err[1]));
+        krc2 = ksegB * fma(V(R(kW2)), three_p, V(P.chi[D == 2 ? 5 : 7] + P.chi_err[2]));
     }
 
     // Direction i (opp(i) > i) and its opposite o, in storage units: the
     // post-collision N*_i - chi_i, N*_o - chi_o (they share the even part and
-    // flip the odd part).
-    __device__ __forceinline__ void dir(int i, V& ni, V& no) const {
+    // flip the odd part) and B*_i - chi_i/2, B*_o - chi_o/2 with
+    // B* = phi N* + recolor, i.e. phi dN* + (phi - 1/2) chi_i + recolor.
+    __device__ __forceinline__ void dir(int i, V& ni, V& no, V& bi, V& bo) const {
         const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
         const R wiN = R(L::w(i)) * sN;
-        // the stress projection, 3 c.u and c.F, each without the terms
+        // the stress projection, 3 c.u, c.F and c.grad phi, each without the terms
         // whose lattice coefficient is zero
-        Acc<V> proj, cu3, cF;
+        Acc<V> proj, cu3, cF, cg;
         if (D == 2) {
             proj.add(cx * cx - cy * cy, A0);
             proj.add(cx * cy, Axy);
@@ -862,29 +907,40 @@ struct NodeUpdate {
             proj.add(cx * cz, Axz);
             proj.add(cy * cz, Ayz);
         }
-        cu3.add(cx, base0); cF.add(cx, F[0]);
-        cu3.add(cy, base1); cF.add(cy, F[1]);
-        cu3.add(cz, base2); cF.add(cz, F[2]);
+        cu3.add(cx, base0); cF.add(cx, F[0]); cg.add(cx, gp[0]);
+        cu3.add(cy, base1); cF.add(cy, F[1]); cg.add(cy, gp[1]);
+        cu3.add(cz, base2); cF.add(cz, F[2]); cg.add(cz, gp[2]);
         const bool axis = cx * cx + cy * cy + cz * cz == 1;
+        const V krc = axis ? krc1 : krc2, g = cg.get();                // recoloring krc (c . grad phi), odd in c
         const V c3 = cu3.get();
         const V even = fma(V(wiN), fma(V(R(0.5)) * c3, c3, axis ? common1 : common2), proj.get());
         const V odd = fma(halfF, cF.get(), c3);                        // the odd part over wiN
         ni = fma(V(wiN), odd, even);
         no = fma(V(-wiN), odd, even);
+        const V shift_b = axis ? shb1 : shb2;                          // (phi - 1/2) chi_i
+        bi = fma(krc, g, fma(phiB, ni, shift_b));
+        bo = fma(-krc, g, fma(phiB, no, shift_b));
     }
 
-    // Rest direction (no forcing, no stress projection, c_0 = 0), stored
-    // exactly: N*_0 - chi_0.
+    // Rest direction (no forcing, no stress projection, no recoloring, c_0 = 0),
+    // stored exactly (FP32): N*_0 - chi_0 and B*_0 - chi_0/2.
     __device__ __forceinline__ V rest_N(const StepParams<R>& P) const {
         return fma(V(-R(1.5 * w0)), uu, fma(V(-R(1.0 - w0)), three_p, V(P.chi_err[0])));
     }
-    // With FP16 storage the float rest population takes the node total the
-    // collision fixes less the moving populations as stored (sumN in storage
-    // units, one node): sum_i (N*_i - chi_i) = 0 for any N, u, p and F (the
-    // equilibrium sums to sum chi = 1; the stress projection and the forcing
-    // have no zeroth moment), so FP16 rounding moves no mass out of the domain,
-    // nor between the phases (sum_i B*_i = phi sum_i N*_i).
+    __device__ __forceinline__ V rest_B(const StepParams<R>& P, V nst0) const {
+        return fma(phi, nst0, (kFullB ? phi : phi - V(R(0.5))) * V(P.chi[0]));
+    }
+    // With FP16 storage the float rest populations take the node totals the
+    // collision fixes less the moving populations as stored (sumN, sumB in
+    // storage units, one node each): sum_i (N*_i - chi_i) = 0 for any N, u, p
+    // and F (the equilibrium sums to sum chi = 1; the stress projection and the
+    // forcing have no zeroth moment) and sum_i (B*_i - chi_i/2) = phi - 1/2 (the
+    // recoloring is odd in c), so FP16 rounding moves no mass between the
+    // phases or out of the domain.
     __device__ __forceinline__ static float rest_N_from_sum(float sumN) { return -sumN * (1.0f / kScaleN); }
+    __device__ __forceinline__ static float rest_B_from_sum(float sumB, float phi_node) {
+        return fmaf(-sumB, 1.0f / kScaleB, phi_node - 0.5f);
+    }
 };
 
 // One fluid node of the step: pulled populations N, the block's halo tile.
@@ -958,29 +1014,36 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
     // FP32 writes them last, measured 0.7% faster
     auto store_u_p = [&]() {
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-            b.u_out[a * pl + node] = nd.u[a].v;
-            b.flux[a * pl + node] = (nd.kflux * nd.gp[a]).v;
-        }
+        for (int a = 0; a < D; ++a) b.u_out[a * pl + node] = nd.u[a].v;
         b.p[node] = nd.p.v;
         if (!(nd.uu.v < T(1e30))) atomicOr(b.err, kErrNonFinite);   // also catches NaN
     };
     if constexpr (!PS::kExact) store_u_p();
 
     auto* __restrict__ Nmov = PS::moving(b.Nout, pl) + pop_at<Q>(node);
-    if constexpr (PS::kExact) PS::store_rest(PS::rest(b.Nout), node, nd.rest_N(P).v);
-    // sum of the moving populations as stored (FP16 storage)
-    T sumN = T(0);
+    auto* __restrict__ Bmov = PS::moving(b.Bout, pl) + pop_at<Q>(node);
+    if constexpr (PS::kExact) {
+        const Sc nst0 = nd.rest_N(P);
+        PS::store_rest(PS::rest(b.Nout), node, nst0.v);
+        PS::store_rest(PS::rest(b.Bout), node, nd.rest_B(P, nst0).v);
+    }
+    // sums of the moving populations as stored (FP16 storage)
+    T sumN = T(0), sumB = T(0);
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         if (L::opp(i) < i) continue;
         const int o = L::opp(i);
-        Sc ni, no;
-        nd.dir(i, ni, no);
+        Sc ni, no, bi, bo;
+        nd.dir(i, ni, no, bi, bo);
         PS::store_units(Nmov, pop_dir(i), ni.v, sumN);
         PS::store_units(Nmov, pop_dir(o), no.v, sumN);
+        PS::store_units(Bmov, pop_dir(i), bi.v, sumB);
+        PS::store_units(Bmov, pop_dir(o), bo.v, sumB);
     }
-    if constexpr (!PS::kExact) PS::store_rest(PS::rest(b.Nout), node, FN::rest_N_from_sum(sumN));
+    if constexpr (!PS::kExact) {
+        PS::store_rest(PS::rest(b.Nout), node, FN::rest_N_from_sum(sumN));
+        PS::store_rest(PS::rest(b.Bout), node, FN::rest_B_from_sum(sumB, nd.phi.v));
+    }
     if constexpr (PS::kExact) store_u_p();
 }
 
@@ -988,9 +1051,9 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
 // grid patches into its halo after a tiled copy: one per halo row and field
 // at each end, K per thread (1 unless the block has fewer threads than both
 // ends' images).
-template <class Tl, typename T, bool VEC>
+template <class Tl, typename T, bool CONTRAST>
 struct HaloFix {
-    static constexpr int kFields = VEC ? 1 + Tl::D : 1;
+    static constexpr int kFields = CONTRAST ? 1 + Tl::D : 1;
     static constexpr int kRows = Tl::HY * Tl::HZ;
     static constexpr int kPerCol = kRows * kFields;
     static constexpr int K = (2 * kPerCol + Tl::THREADS - 1) / Tl::THREADS;
@@ -998,10 +1061,9 @@ struct HaloFix {
     int at[K];                                 // halo slot (phi, then the u fields), or -1
 };
 
-// A block's halo tile with a one-node ring: the color and, with VEC, a vector
-// field (the previous velocity for the step kernels with a density contrast,
-// the recolouring flux for the color kernels).  Issued by halo_issue, waited
-// for by halo_complete, shared by the kernels of every tile shape.  With maps
+// A block's halo tile (color, and the previous velocity with a density
+// contrast) with a one-node ring: issued by halo_issue, waited for by
+// halo_complete, shared by the step kernels of every tile shape.  With maps
 // (tiles whose halo needs no periodic image in y and z) two tiled TMA copies
 // fill it, completed on the mbarrier `bar`; at the x ends of the grid the box
 // reads zeros where x < 0 or x >= nx, and the stencil needs the periodic
@@ -1009,11 +1071,11 @@ struct HaloFix {
 // and write them once the copy has landed.  Without maps the halo is copied
 // element by element with cp.async.  halo_issue returns false when the debug
 // bounds checks reject the tile's box.
-template <class Tl, typename T, bool VEC>
-__device__ __forceinline__ bool halo_issue(const StepParams<T>& P, const T* phi, const T* vec, int* err, T* s_phi,
-                                           T* s_u, int x0, int y0, int z0, const CUtensorMap* tm_phi,
-                                           const CUtensorMap* tm_u, uint64_t* bar, HaloFix<Tl, T, VEC>& fx) {
-    using Fx = HaloFix<Tl, T, VEC>;
+template <class Tl, typename T, typename S, bool CONTRAST>
+__device__ __forceinline__ bool halo_issue(const StepParams<T>& P, const StepBuffers<T, S>& b, T* s_phi, T* s_u,
+                                           int x0, int y0, int z0, const CUtensorMap* tm_phi,
+                                           const CUtensorMap* tm_u, uint64_t* bar, HaloFix<Tl, T, CONTRAST>& fx) {
+    using Fx = HaloFix<Tl, T, CONTRAST>;
     const bool tma = tm_phi != nullptr;
 #pragma unroll
     for (int j = 0; j < Fx::K; ++j) {
@@ -1027,18 +1089,18 @@ __device__ __forceinline__ bool halo_issue(const StepParams<T>& P, const T* phi,
         const bool box_ok = ((x0 - Tl::XO) & 3) == 0 && y0 >= 1 && y0 + Tl::TY + 1 <= P.ny &&
                             (Tl::D == 2 || (z0 >= 1 && z0 + Tl::TZ + 1 <= P.nz));
         if (!box_ok) {
-            if (threadIdx.x + threadIdx.y + threadIdx.z == 0) atomicOr(err, kErrBounds);
+            if (threadIdx.x + threadIdx.y + threadIdx.z == 0) atomicOr(b.err, kErrBounds);
             return false;                                  // the whole block takes this branch
         }
     }
     if (tma) {
         const int tid = threadIdx.x + Tl::BX * (threadIdx.y + Tl::TY * threadIdx.z);
         if (tid == 0) {
-            constexpr unsigned kBytes = (VEC ? 1 + Tl::D : 1) * Tl::HN * sizeof(T);
+            constexpr unsigned kBytes = (CONTRAST ? 1 + Tl::D : 1) * Tl::HN * sizeof(T);
             mbar_expect_tx(bar, kBytes);
             const int zc = Tl::D == 2 ? 0 : z0 - 1;
             tma_load_3d(s_phi, tm_phi, x0 - Tl::XO, y0 - 1, zc, bar);
-            if (VEC) tma_load_4d(s_u, tm_u, x0 - Tl::XO, y0 - 1, zc, 0, bar);
+            if (CONTRAST) tma_load_4d(s_u, tm_u, x0 - Tl::XO, y0 - 1, zc, 0, bar);
         }
         const bool lo = x0 == 0, hi = x0 + Tl::TX >= P.nx;
         constexpr int kRows = Fx::kRows, kPerCol = Fx::kPerCol;
@@ -1054,13 +1116,13 @@ __device__ __forceinline__ bool halo_issue(const StepParams<T>& P, const T* phi,
             const int hy = r % Tl::HY, hz = r / Tl::HY;
             const int gz = Tl::D == 2 ? 0 : z0 - 1 + hz;
             const int node = (left ? P.nx - 1 : 0) + P.px * (y0 - 1 + hy + P.ny * gz);
-            const int fn = idx_checked(node, P.plane, err);
-            fx.v[j] = field == 0 ? phi[fn] : vec[(field - 1) * (int)P.plane + fn];
+            const int fn = idx_checked(node, P.plane, b.err);
+            fx.v[j] = field == 0 ? b.phi[fn] : b.u_in[(field - 1) * (int)P.plane + fn];
             fx.at[j] = (field == 0 ? 0 : Tl::HN * field) + (left ? Tl::XO - 1 : P.nx - x0 + Tl::XO) + Tl::HX * r;
-            if (!idx_ok(fx.at[j], kHaloFields * Tl::HN, err)) fx.at[j] = -1;
+            if (!idx_ok(fx.at[j], kHaloFields * Tl::HN, b.err)) fx.at[j] = -1;
         }
     } else {
-        load_halo<Tl, T, VEC>(P, phi, vec, s_phi, s_u, x0, y0, z0, err);
+        load_halo<Tl, T, CONTRAST>(P, b.phi, b.u_in, s_phi, s_u, x0, y0, z0, b.err);
     }
     return true;
 }
@@ -1068,8 +1130,8 @@ __device__ __forceinline__ bool halo_issue(const StepParams<T>& P, const T* phi,
 // Waits for the halo issued by halo_issue and patches the x-end images;
 // false if a tiled copy did not complete within the bounded wait.  The
 // caller's barrier follows.
-template <class Tl, typename T, class Fx>
-__device__ __forceinline__ bool halo_complete(int* err, bool tma, uint64_t* bar, T* s_phi,
+template <class Tl, typename T, typename S, class Fx>
+__device__ __forceinline__ bool halo_complete(const StepBuffers<T, S>& b, bool tma, uint64_t* bar, T* s_phi,
                                               T* s_u, const Fx& fx) {
     if (!tma) {
         cp_async_wait_all();
@@ -1081,7 +1143,7 @@ __device__ __forceinline__ bool halo_complete(int* err, bool tma, uint64_t* bar,
         // is refused further steps).  The copy may still be in flight into
         // this block's shared memory: wait for it once more, again bounded,
         // before the block exits, so that it does not land in a later block.
-        if (threadIdx.x + threadIdx.y + threadIdx.z == 0) atomicOr(err, kErrCopyTimeout);
+        if (threadIdx.x + threadIdx.y + threadIdx.z == 0) atomicOr(b.err, kErrCopyTimeout);
         mbar_wait(bar, 0);
     }
 #pragma unroll
@@ -1105,151 +1167,14 @@ __device__ __forceinline__ void step_tile(const StepParams<T>& P, const StepBuff
     const uint32_t m = in_grid ? __ldg(b.mask + node) : MASK_NOT_FLUID;
     pdl_wait();
     HaloFix<Tl, T, CONTRAST> fx;
-    if (!halo_issue<Tl, T, CONTRAST>(P, b.phi, b.u_in, b.err, s_phi, s_u, x0, y0, z0, tm_phi, tm_u, bar, fx)) return;
+    if (!halo_issue<Tl, T, S, CONTRAST>(P, b, s_phi, s_u, x0, y0, z0, tm_phi, tm_u, bar, fx)) return;
     T N[Q];
     if (in_grid) pull_streaming<Q, T, S>(P, b.Nin, node, x, y, z, N, b.err);      // in flight with the mask load
     const bool fluid = !(m & MASK_NOT_FLUID);
-    if (fluid && (m & MASK_DIRS)) pull_bounce_back<Q, T, S>(P, b.Nin, m, node, N, b.err);
-    const bool halo_ok = halo_complete<Tl, T>(b.err, tma, bar, s_phi, s_u, fx);
+    if (fluid && (m & ~MASK_NOT_FLUID)) pull_bounce_back<Q, T, S>(P, b.Nin, m, node, N, b.err);
+    const bool halo_ok = halo_complete<Tl, T, S>(b, tma, bar, s_phi, s_u, fx);
     __syncthreads();
     if (fluid && halo_ok) step_node<Q, V, T, S, CONTRAST>(P, b, s_phi, s_u, N, node);
-}
-
-// ---------------------------------------------------------------------------
-// k_color: Eq. (phiUpdate) on the pulled B*_i = phi N*_i + w_i c_i . f
-// ---------------------------------------------------------------------------
-// The new color of one node (V = SF, SD), or of the two nodes of a pair (F2):
-// N the pulled populations (storage units), n0 the rest population, ph(i) the
-// color and fl(i, a) the flux component a at the node direction i comes from.
-// Taken as the change from the node's own color,
-//     phi' = phi + sum_i chi_i (phi_i - phi) + sum_i phi_i (N_i - chi_i) + sum_i w_i c_i . f_i,
-// whose terms are small: what two neighbours exchange cancels to the bit in
-// the color's sum but for the products' rounding.  In float the sum's rounding
-// is kept in lo and joins the next change: changes below the color's last
-// place (6e-8 in the liquid) would otherwise be dropped step after step and
-// hold the interface off its equilibrium.  With FP64 the differences are taken
-// class by class, which saves Q - 3 FP64 instructions.
-template <int Q, bool UNITS, typename V, class PhiAt, class FluxAt>
-__device__ __forceinline__ V color_update(const StepParams<typename V::Real>& P, V phi, V n0, const V (&N)[Q],
-                                          PhiAt ph, FluxAt fl, V& lo) {
-    using L = Lattice<Q>;
-    using R = typename V::Real;
-    constexpr int kDiag = L::D == 2 ? 5 : 7;                 // first diagonal/edge direction
-    constexpr bool kByClass = sizeof(R) == 8;
-    Acc<V> d1, d2, f1, f2;
-    V n = V(R(0));
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-        const auto pi = ph(i);
-        V t;
-        if constexpr (kByClass) t = pi; else t = pi - phi;
-        n = i == 1 ? pi * N[i] : fma(pi, N[i], n);
-        const int c[3] = {L::cx(i), L::cy(i), L::cz(i)};
-        if (i < kDiag) d1.add(1, t); else d2.add(1, t);
-#pragma unroll
-        for (int a = 0; a < L::D; ++a) {
-            if (c[a] == 0) continue;
-            if (i < kDiag) f1.add(c[a], fl(i, a)); else f2.add(c[a], fl(i, a));
-        }
-    }
-    V s1 = d1.get(), s2 = d2.get();
-    if (kByClass) {
-        s1 = fma(V(R(1 - kDiag)), phi, s1);
-        s2 = fma(V(R(kDiag - Q)), phi, s2);
-    }
-    V r = fma(V(P.chi[1]), s1, V(P.chi[kDiag]) * s2);
-    r = fma(V(R(L::w(1))), f1.get(), fma(V(R(L::w(kDiag))), f2.get(), r));
-    r = fma(phi, n0, r);
-    r = UNITS ? fma(n, V(R(1) / R(kScaleN)), r) : r + n;
-    if (kByClass) return phi + r;
-    r = r + lo;
-    const V s = phi + r, d = s - phi;
-    lo = (phi - (s - d)) + (r - d);                          // phi + r = s + lo exactly
-    return s;
-}
-
-// The color tile at (x0, y0, z0), one node per thread (early: the ghost kernel
-// follows and may start at once): halo of the color and
-// the flux, the pull of N* while it is in flight.  A node that is not fluid
-// keeps its value (ghost nodes their ghost color, read back as it was used).
-template <int Q, int V, typename T, typename S>
-__device__ __forceinline__ void color_tile(const StepParams<T>& P, const StepBuffers<T, S>& b, T* s_phi, T* s_f, int x0,
-                                           int y0, int z0, int early, const CUtensorMap* tm_phi = nullptr,
-                                           const CUtensorMap* tm_f = nullptr, uint64_t* bar = nullptr) {
-    using Tl = Tile<Q, V>;
-    using L = Lattice<Q>;
-    using PS = PopStore<S>;
-    using Sc = typename ScalarOf<T>::type;
-    const bool tma = tm_phi != nullptr;
-    const int x = x0 + threadIdx.x, y = y0 + threadIdx.y, z = z0 + threadIdx.z;
-    const bool in_grid = x < P.nx && y < P.ny && z < P.nz;
-    const int node = in_grid ? idx_checked(x + P.px * (y + P.ny * z), P.plane, b.err) : 0;
-    const uint32_t m = in_grid ? __ldg(b.mask + node) : MASK_NOT_FLUID;
-    pdl_wait();
-    if (early) pdl_trigger();
-    HaloFix<Tl, T, true> fx;
-    if (!halo_issue<Tl, T, true>(P, b.phi, b.flux, b.err, s_phi, s_f, x0, y0, z0, tm_phi, tm_f, bar, fx)) return;
-    T N[Q], n0 = T(0);
-    if (in_grid) {
-        pull_streaming<Q, T, S>(P, b.Nout, node, x, y, z, N, b.err);
-        n0 = (T)PS::load_rest(PS::rest(static_cast<const S*>(b.Nout)), node);
-    }
-    const bool fluid = !(m & MASK_NOT_FLUID);
-    if (fluid && (m & MASK_DIRS)) pull_bounce_back<Q, T, S>(P, b.Nout, m, node, N, b.err);
-    const bool halo_ok = halo_complete<Tl, T>(b.err, tma, bar, s_phi, s_f, fx);
-    __syncthreads();
-    if (!in_grid || !halo_ok) return;
-    const int hc = (threadIdx.x + Tl::XO) +
-                   Tl::HX * ((threadIdx.y + 1) + Tl::HY * (Tl::D == 2 ? 0 : threadIdx.z + 1));
-    const T phi = s_phi[idx_checked(hc, Tl::HN, b.err)];
-    if (!fluid) {
-        b.phi_out[node] = phi;
-        return;
-    }
-    Sc Ns[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) Ns[i] = Sc(N[i]);
-    auto from = [&](int i) { return idx_checked(hc - Tl::off(L::cx(i), L::cy(i), L::cz(i)), Tl::HN, b.err); };
-    Sc r, lo = Sc(T(0));
-    if (sizeof(T) == 4) lo = Sc(b.phi_lo[node]);
-    if (!(m & MASK_DIRS)) {
-        auto ph = [&](int i) { return Sc(s_phi[from(i)]); };
-        auto fl = [&](int i, int a) { return Sc(s_f[a * Tl::HN + from(i)]); };
-        r = color_update<Q, !PS::kExact, Sc>(P, Sc(phi), Sc(n0), Ns, ph, fl, lo);
-    } else {
-        // a direction that bounces back carries the node's own B* of the opposite direction
-        auto ph = [&](int i) { return Sc((m >> i) & 1u ? phi : s_phi[from(i)]); };
-        auto fl = [&](int i, int a) {
-            const T* f = s_f + a * Tl::HN;
-            return Sc((m >> i) & 1u ? -f[hc] : f[from(i)]);
-        };
-        r = color_update<Q, !PS::kExact, Sc>(P, Sc(phi), Sc(n0), Ns, ph, fl, lo);
-    }
-    b.phi_out[node] = r.v;
-    if (sizeof(T) == 4) b.phi_lo[node] = lo.v;
-}
-
-template <int Q, typename T, typename S, int V = 0>
-__global__ void __launch_bounds__(Tile<Q, V>::THREADS)
-    k_color(StepParams<T> P, StepBuffers<T, S> b, const __grid_constant__ CUtensorMap tm_phi,
-            const __grid_constant__ CUtensorMap tm_f, int tma, int early) {
-    using Tl = Tile<Q, V>;
-    __shared__ __align__(128) T s_phi[Tl::HN];
-    __shared__ __align__(128) T s_f[Tl::D * Tl::HN];
-    __shared__ __align__(8) uint64_t s_bar;
-    // tiles in the reverse of k_step's order: the N* and f that k_step wrote last
-    // are still in L2 when this kernel starts
-    const int x0 = (gridDim.x - 1 - blockIdx.x) * Tl::TX, y0 = (gridDim.y - 1 - blockIdx.y) * Tl::TY,
-              z0 = (gridDim.z - 1 - blockIdx.z) * Tl::TZ;
-    const bool interior = tma && y0 >= 1 && y0 + Tl::TY + 1 <= P.ny &&
-                          (Tl::D == 2 || (z0 >= 1 && z0 + Tl::TZ + 1 <= P.nz));
-    if (interior) {
-        if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
-        __syncthreads();
-        color_tile<Q, V, T, S>(P, b, s_phi, s_f, x0, y0, z0, early, &tm_phi, &tm_f, &s_bar);
-    } else {
-        color_tile<Q, V, T, S>(P, b, s_phi, s_f, x0, y0, z0, early);
-    }
 }
 
 // Resident blocks per SM the step kernels are compiled for (registers per
@@ -1313,20 +1238,9 @@ struct BatchEntry {
 template <typename T, typename S>
 __constant__ BatchEntry<T, S> c_batch[kBatchSlots];
 
-// maps: tiled TMA maps of the halo fields for this tile shape, kSlotMaps per
-// slot (phi, then u_in, each for step parity 0 and 1, then the flux, with the
-// box of Tile<Q, V>'s halo), in global memory; used on tiles needing no
-// periodic image in y, z.
-constexpr int kSlotMaps = 5;
-__device__ __forceinline__ const CUtensorMap* slot_phi_map(const CUtensorMap* maps, int slot, int parity) {
-    return maps + kSlotMaps * slot + parity;
-}
-__device__ __forceinline__ const CUtensorMap* slot_u_map(const CUtensorMap* maps, int slot, int parity) {
-    return maps + kSlotMaps * slot + 2 + parity;
-}
-__device__ __forceinline__ const CUtensorMap* slot_flux_map(const CUtensorMap* maps, int slot) {
-    return maps + kSlotMaps * slot + 4;
-}
+// maps: tiled TMA maps of the halo fields for this tile shape, three per slot
+// (phi, then u_in for step parity 0 and 1, with the box of Tile<Q, V>'s halo),
+// in global memory; used on tiles needing no periodic image in y, z.
 template <int Q, typename T, typename S, int V, bool CONTRAST>
 __global__ void __launch_bounds__(Tile<Q, V>::THREADS, (step_min_blocks<T, S, Tile<Q, V>::THREADS>()))
     k_step_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity) {
@@ -1347,38 +1261,40 @@ __global__ void __launch_bounds__(Tile<Q, V>::THREADS, (step_min_blocks<T, S, Ti
     if (tma) {
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();                                      // the barrier exists before anyone waits on it
-        step_tile<Q, V, T, S, CONTRAST>(e.P, e.b[parity], s_phi, s_u, t.y, y0, z0, slot_phi_map(maps, t.x, parity),
-                                        slot_u_map(maps, t.x, parity), &s_bar);
+        step_tile<Q, V, T, S, CONTRAST>(e.P, e.b[parity], s_phi, s_u, t.y, y0, z0, maps + 3 * t.x,
+                                        maps + 3 * t.x + 1 + parity, &s_bar);
     } else {
         step_tile<Q, V, T, S, CONTRAST>(e.P, e.b[parity], s_phi, s_u, t.y, y0, z0);
     }
 }
 
 template <int Q, typename T, typename S, int V>
-__global__ void __launch_bounds__(Tile<Q, V>::THREADS)
-    k_color_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity, int early) {
-    using Tl = Tile<Q, V>;
-    __shared__ __align__(128) T s_phi[Tl::HN];
-    __shared__ __align__(128) T s_f[Tl::D * Tl::HN];
-    __shared__ __align__(8) uint64_t s_bar;
-    const int4 t = __ldg(tiles + (gridDim.x - 1 - blockIdx.x));     // reverse order, as k_color
+__global__ void __launch_bounds__(Tile<Q, V>::THREADS) k_phi_batched(const int4* __restrict__ tiles, int parity,
+                                                                             int early) {
+    const int4 t = __ldg(tiles + (gridDim.x - 1 - blockIdx.x));     // reverse order, as k_phi
     const BatchEntry<T, S>& e = c_batch<T, S>[idx_checked(t.x, kBatchSlots, c_batch<T, S>[0].b[0].err)];
-    const int y0 = t.z, z0 = t.w;
-    if (kDebugBounds && !(idx_ok(t.y, e.P.nx, e.b[0].err) && idx_ok(y0, e.P.ny, e.b[0].err) &&
-                          idx_ok(z0, e.P.nz, e.b[0].err))) {
-        pdl_wait();
-        return;                                         // a tile outside its domain
+    // this step's output B* is the buffer the step kernel wrote
+    phi_node<Q, T, S>(e.P, e.b[parity].Bout, e.b[parity].mask, e.b[parity].phi, t.y + threadIdx.x, t.z + threadIdx.y,
+                      t.w + threadIdx.z, early, e.b[parity].err);
+}
+
+// Color kernel of a batch over row chunks: a block takes kPhiChunk
+// consecutive nodes of one z plane of one domain in the padded row order
+// (tile {slot, x0, y0, z}: the chunk starts at (x0, y0)), crossing rows where
+// a row ends, so that only the padding columns and a plane's last chunk leave
+// threads idle (box tiles idle at the ragged x end of every row of a small
+// domain), and every pull of the block reads one contiguous run per direction.
+template <int Q, typename T, typename S>
+__global__ void __launch_bounds__(kPhiChunk) k_phi_rows_batched(const int4* __restrict__ tiles, int parity, int early) {
+    const int4 t = __ldg(tiles + (gridDim.x - 1 - blockIdx.x));     // reverse order, as k_phi
+    const BatchEntry<T, S>& e = c_batch<T, S>[idx_checked(t.x, kBatchSlots, c_batch<T, S>[0].b[0].err)];
+    int x = t.y + (int)threadIdx.x, y = t.z;
+    while (x >= e.P.px) {                         // at most kPhiChunk / px + 1 rows on
+        x -= e.P.px;
+        ++y;
     }
-    const bool tma = maps != nullptr && e.tma && y0 >= 1 && y0 + Tl::TY + 1 <= e.P.ny &&
-                     (Tl::D == 2 || (z0 >= 1 && z0 + Tl::TZ + 1 <= e.P.nz));
-    if (tma) {
-        if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
-        __syncthreads();
-        color_tile<Q, V, T, S>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0, early, slot_phi_map(maps, t.x, parity),
-                               slot_flux_map(maps, t.x), &s_bar);
-    } else {
-        color_tile<Q, V, T, S>(e.P, e.b[parity], s_phi, s_f, t.y, y0, z0, early);
-    }
+    // padding columns and threads past the plane's end drop out there
+    phi_node<Q, T, S>(e.P, e.b[parity].Bout, e.b[parity].mask, e.b[parity].phi, x, y, t.w, early, e.b[parity].err);
 }
 
 // Ghost tables of all domains: ghost g of the batch belongs to the domain d with
@@ -1390,7 +1306,7 @@ struct GhostTable {
     const int32_t* corner;
     const T* wt;
     T exp_eps, eps;
-    T* phi[2];                     // by step parity
+    T* phi;
     int rule;
     int64_t plane;                 // entries of phi (bounds of node and corner indices)
     int* err;                      // the domain's error word
@@ -1399,7 +1315,7 @@ struct GhostTable {
 template <int GK, typename T>
 __global__ void __launch_bounds__(256) k_ghost_batched(const GhostTable<T>* __restrict__ tabs,
                                                        const int64_t* __restrict__ ghost_begin, int ndom,
-                                                       int64_t total, int parity) {
+                                                       int64_t total) {
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (g >= total) {
         pdl_wait();
@@ -1426,10 +1342,9 @@ __global__ void __launch_bounds__(256) k_ghost_batched(const GhostTable<T>* __re
     pdl_wait();
     pdl_trigger();
     if (!ok) return;
-    T* const phi = t.phi[parity];
     T phiF = T(0);
 #pragma unroll
-    for (int c = 0; c < GK; ++c) phiF += wt[c] * phi[corner[c]];
+    for (int c = 0; c < GK; ++c) phiF += wt[c] * t.phi[corner[c]];
     T phiG;
     if (t.rule == 0) {
         phiG = phiF / (phiF + (T(1) - phiF) * t.exp_eps);
@@ -1437,7 +1352,7 @@ __global__ void __launch_bounds__(256) k_ghost_batched(const GhostTable<T>* __re
         const T a = T(1) + T(0.5) * t.eps;
         phiG = T(4) * phiF / (a + sqrt(a * a - T(2) * t.eps * phiF)) - phiF;
     }
-    if (idx_ok(gn, t.plane, t.err)) phi[gn] = phiG;
+    if (idx_ok(gn, t.plane, t.err)) t.phi[gn] = phiG;
 }
 
 }  // namespace lbmgpu

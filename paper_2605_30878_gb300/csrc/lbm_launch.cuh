@@ -28,36 +28,26 @@ struct StepConfig {
     double exp_eps;
     double eps;                    // -(4/W) cos(theta)
     int ghost_rule;                // lbm_ghost_rule
-    bool pair = false;             // float arithmetic: the two-node kernels (k_step_pair, k_color_pair)
-    int pair_width = 32;           // nodes along x of their tiles, 32 or 64
+    bool pair = false;             // float arithmetic: the two-node step kernel (k_step_pair)
+    int pair_width = 32;           // nodes along x of its tiles, 32 or 64
 };
 
 struct StepPtrs {
     const void* Nin;
+    const void* Bin;
     void* Nout;
-    const void* phi;               // color the step reads
-    void* phi_out;                 // color after the step
-    void* phi_lo;
+    void* Bout;
+    void* phi;
     const void* u_in;
     void* u_out;
     void* p;
-    void* flux;
     const uint32_t* mask;
     int* err;
-    // tiled maps of phi, u_in and the flux for the halo copies (the box of the
-    // domain's step and color kernels), or none
+    // tiled maps of phi and of u_in for the halo copies (the box of the domain's
+    // step kernel), or none
     const CUtensorMap* tm_phi = nullptr;
     const CUtensorMap* tm_u = nullptr;
-    const CUtensorMap* tm_flux = nullptr;
 };
-
-// Single-domain tile of the one-node kernels: shape 0 in float; in FP64 shape
-// 3, 128-thread tiles.  FP64 is bound by its arithmetic rate per SM, so what
-// counts is that every SM has blocks and the last ones are short.  Against
-// 256-thread tiles (shape 0): 64^2 19.7 -> 13.3 us per step, 300^2 54.9 -> 47.2,
-// 24^3 41.2 -> 25.6, equal from 500 x 300 and 64^3 on; one-warp tiles gain
-// nothing more (13.1, 47.2, 26.6).
-template <typename T> constexpr int kSingleTile = sizeof(T) == 8 ? 3 : 0;
 
 template <typename T, typename S>
 struct Launch {
@@ -71,20 +61,15 @@ struct Launch {
     template <int Q>
     static void step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
     static void step(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
-    template <int Q>
-    static void color_q(const StepConfig& c, const StepPtrs& p, int early, cudaStream_t s);
     // ghosts_follow: the next kernel on the stream is the ghost kernel
-    static void color(const StepConfig& c, const StepPtrs& p, bool ghosts_follow, cudaStream_t s);
-    static StepBuffers<T, S> buffers(const StepPtrs& p);
+    static void phi(const StepConfig& c, const void* Bst, const uint32_t* mask, void* phi, bool ghosts_follow, int* err,
+                    cudaStream_t s);
     static void ghost(int GK, int rule, int64_t ng, const int32_t* node, const int32_t* corner, const void* wt,
                       double exp_eps, double eps, void* phi, int64_t plane, int* err, cudaStream_t s);
     static unsigned flat_blocks(const Dims& d);
     static void init_phi(const StepConfig& c, const uint8_t* cls, void* phi, int mode, const double ctr[3], double R0,
                          double ghost_value, cudaStream_t s);
     static void init_pops(const StepConfig& c, const uint8_t* cls, const void* phi, void* N, void* B, cudaStream_t s);
-    // B of the last step into B (storage form), from its color, N* and flux
-    static void rebuild_B(const StepConfig& c, const uint8_t* cls, const void* phi, const void* N, const void* flux,
-                          void* B, cudaStream_t s);
     static void build_mask(const StepConfig& c, const uint8_t* cls, uint32_t* mask, cudaStream_t s);
     static void expand_classes(const StepConfig& c, int W, const uint64_t* F, const uint64_t* G, uint8_t* cls,
                                cudaStream_t s);
@@ -101,26 +86,21 @@ struct Launch {
     template <int Qc, int V>
     static void step_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast, int parity,
                                cudaStream_t s);
-    // the step kernels of every domain (the ghost update precedes them) on tile
-    // shape V; tiles[0, ncontrast) belong to domains with density contrast
-    static void step_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
-                             int parity, cudaStream_t s);
-    template <int Qc, int V>
-    static void color_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int parity, int early,
-                                cudaStream_t s);
-    // the color kernel of every domain on tile shape V
-    static void color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int parity,
-                              bool ghosts_follow, cudaStream_t s);
+    // step kernels then color kernel of every domain (the ghost update precedes them);
+    // tiles[0, ncontrast) belong to domains with density contrast; the color
+    // kernel runs on phi_tiles of shape Vphi, or of row chunks (Vphi == kPhiRows)
+    static void step_phi_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
+                                 int Vphi, const int4* phi_tiles, int phi_ntiles, int parity, bool ghosts_follow,
+                                 cudaStream_t s);
     // Slot tables: entry_size() bytes per domain, filled by fill_entry, copied
     // to slots [slot0, slot0 + n) of the constant table by upload_entries.
     static size_t entry_size() { return sizeof(BatchEntry<T, S>); }
     static void fill_entry(void* out, const StepConfig& c, const StepPtrs p[2], bool tma);
     static cudaError_t upload_entries(int slot0, const void* entries, int n);
-    static void ghost_batched(int GK, const void* tabs, const int64_t* begin, int ndom, int64_t total, int parity,
-                              cudaStream_t s);
+    static void ghost_batched(int GK, const void* tabs, const int64_t* begin, int ndom, int64_t total, cudaStream_t s);
     static size_t ghost_table_size() { return sizeof(GhostTable<T>); }
     static void fill_ghost_table(void* out, int64_t n, const int32_t* node, const int32_t* corner, const void* wt,
-                                 double exp_eps, double eps, void* const phi[2], int rule, int64_t plane, int* err);
+                                 double exp_eps, double eps, void* phi, int rule, int64_t plane, int* err);
     static int diag_blocks(const Dims& d);
     static void diag(const StepConfig& c, const uint32_t* mask, const void* Nst, const void* phi, const void* u,
                      const void* p, const ProbeDev& pr, double* partial, double* out, cudaStream_t s);

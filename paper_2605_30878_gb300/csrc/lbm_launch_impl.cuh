@@ -67,7 +67,6 @@ StepParams<T> Launch<T, S>::params(const StepConfig& c) {
     P.chi_err[1] = (T)(c.chi[1] - chi[1]);
     P.chi_err[2] = (T)(c.chi[diag] - chi[diag]);
     P.c2chi = (T)c.c2chi;
-    P.kappa = (T)(c.chi[1] / (c.Q == 9 ? Lattice<9>::w(1) : Lattice<19>::w(1)));
     P.exp_eps = (T)c.exp_eps;
     return P;
 }
@@ -93,20 +92,13 @@ dim3 Launch<T, S>::pair_grid(const Dims& d) {
 }
 
 template <typename T, typename S>
-StepBuffers<T, S> Launch<T, S>::buffers(const StepPtrs& p) {
-    StepBuffers<T, S> b;
-    b.Nin = (const S*)p.Nin; b.Nout = (S*)p.Nout;
-    b.phi = (const T*)p.phi; b.phi_out = (T*)p.phi_out; b.phi_lo = (T*)p.phi_lo;
-    b.u_in = (const T*)p.u_in; b.u_out = (T*)p.u_out; b.p = (T*)p.p; b.flux = (T*)p.flux;
-    b.mask = p.mask; b.err = p.err;
-    return b;
-}
-
-template <typename T, typename S>
 template <int Q>
 void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s) {
     const StepParams<T> P = params(c);
-    const StepBuffers<T, S> b = buffers(p);
+    StepBuffers<T, S> b;
+    b.Nin = (const S*)p.Nin; b.Bin = (const S*)p.Bin; b.Nout = (S*)p.Nout; b.Bout = (S*)p.Bout;
+    b.phi = (T*)p.phi; b.u_in = (const T*)p.u_in; b.u_out = (T*)p.u_out; b.p = (T*)p.p;
+    b.mask = p.mask; b.err = p.err;
     CUtensorMap tm_phi{}, tm_u{};
     const int tma = p.tm_phi && p.tm_u;
     if (tma) {
@@ -127,7 +119,12 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s
             return;
         }
     }
-    constexpr int V = kSingleTile<T>;
+    // FP64: 128-thread tiles.  It is bound by its arithmetic rate per SM, so what
+    // counts is that every SM has blocks and the last ones are short.  Against
+    // 256-thread tiles (shape 0): 64^2 19.7 -> 13.3 us per step, 300^2 54.9 -> 47.2,
+    // 24^3 41.2 -> 25.6, equal from 500 x 300 and 64^3 on; one-warp tiles gain
+    // nothing more (13.1, 47.2, 26.6).
+    constexpr int V = sizeof(T) == 8 ? 3 : 0;
     if (c.contrast)
         launch_pdl(k_step<Q, T, S, true, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma);
     else
@@ -140,34 +137,28 @@ void Launch<T, S>::step(const StepConfig& c, const StepPtrs& p, cudaStream_t s) 
 }
 
 template <typename T, typename S>
-template <int Q>
-void Launch<T, S>::color_q(const StepConfig& c, const StepPtrs& p, int early, cudaStream_t s) {
+void Launch<T, S>::phi(const StepConfig& c, const void* Bst, const uint32_t* mask, void* phi, bool ghosts_follow,
+                       int* err, cudaStream_t s) {
     const StepParams<T> P = params(c);
-    const StepBuffers<T, S> b = buffers(p);
-    CUtensorMap tm_phi{}, tm_f{};
-    const int tma = p.tm_phi && p.tm_flux;
-    if (tma) {
-        tm_phi = *p.tm_phi;
-        tm_f = *p.tm_flux;
-    }
+    const int early = ghosts_follow;
     if constexpr (sizeof(T) == 4) {
         if (c.pair) {
-            auto run = [&](auto tile) {
+            auto run = [&](auto q, auto tile) {
                 using Tl = decltype(tile);
-                launch_pdl(k_color_pair<Q, S, Tl::TX, Tl::TY>, pair_grid<Tl>(c.d), dim3(Tl::BX, Tl::TY, Tl::TZ), s, P, b,
-                           tm_phi, tm_f, tma, early);
+                launch_pdl(k_phi_pair<decltype(q)::value, S, Tl::TX, Tl::TY>, pair_grid<Tl>(c.d),
+                           dim3(Tl::BX, Tl::TY, Tl::TZ), s, P, (const S*)Bst, mask, (T*)phi, early, err);
             };
-            if (c.pair_width == 64) run(PairTile<Q>{}); else run(NarrowTile<Q>{});
+            const std::integral_constant<int, 9> q9;
+            const std::integral_constant<int, 19> q19;
+            if (c.Q == 9) c.pair_width == 64 ? run(q9, PairTile<9>{}) : run(q9, NarrowTile<9>{});
+            else c.pair_width == 64 ? run(q19, PairTile<19>{}) : run(q19, NarrowTile<19>{});
             return;
         }
     }
-    constexpr int V = kSingleTile<T>;
-    launch_pdl(k_color<Q, T, S, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_f, tma, early);
-}
-
-template <typename T, typename S>
-void Launch<T, S>::color(const StepConfig& c, const StepPtrs& p, bool ghosts_follow, cudaStream_t s) {
-    if (c.Q == 9) color_q<9>(c, p, ghosts_follow, s); else color_q<19>(c, p, ghosts_follow, s);
+    if (c.Q == 9)
+        launch_pdl(k_phi<9, T, S>, step_grid<9>(c.d), step_block<9>(), s, P, (const S*)Bst, mask, (T*)phi, early, err);
+    else
+        launch_pdl(k_phi<19, T, S>, step_grid<19>(c.d), step_block<19>(), s, P, (const S*)Bst, mask, (T*)phi, early, err);
 }
 
 template <typename T, typename S>
@@ -208,18 +199,6 @@ void Launch<T, S>::init_pops(const StepConfig& c, const uint8_t* cls, const void
         k_init_pops<9, T, S><<<flat_blocks(c.d), 256, 0, s>>>(c.d, P, cls, (const T*)phi, (S*)N, (S*)B);
     else
         k_init_pops<19, T, S><<<flat_blocks(c.d), 256, 0, s>>>(c.d, P, cls, (const T*)phi, (S*)N, (S*)B);
-}
-
-template <typename T, typename S>
-void Launch<T, S>::rebuild_B(const StepConfig& c, const uint8_t* cls, const void* phi, const void* N, const void* flux,
-                             void* B, cudaStream_t s) {
-    const StepParams<T> P = params(c);
-    if (c.Q == 9)
-        k_rebuild_B<9, T, S><<<flat_blocks(c.d), 256, 0, s>>>(c.d, P, cls, (const T*)phi, (const S*)N, (const T*)flux,
-                                                              (S*)B);
-    else
-        k_rebuild_B<19, T, S><<<flat_blocks(c.d), 256, 0, s>>>(c.d, P, cls, (const T*)phi, (const S*)N, (const T*)flux,
-                                                               (S*)B);
 }
 
 template <typename T, typename S>
@@ -300,62 +279,53 @@ void Launch<T, S>::step_batched_v(const int4* tiles, const CUtensorMap* maps, in
     }
 }
 
+// step kernels then color kernel of every domain (the ghost update precedes them);
+// tiles[0, ncontrast) belong to domains with density contrast
 template <typename T, typename S>
-template <int Qc, int V>
-void Launch<T, S>::color_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int parity, int early,
-                                   cudaStream_t s) {
-    using Tl = Tile<Qc, V>;
-    if constexpr ((V == 5 || V == 3 || V == 0) && sizeof(T) == 4) {
-        constexpr int TXn = Tl::TX, TYn = Tl::TY;
-        using Pt = PairTile<Qc, TXn, TYn>;
-        launch_pdl(k_color_pair_batched<Qc, S, TXn, TYn>, ntiles, dim3(Pt::BX, Pt::TY, Pt::TZ), s, tiles, maps, parity,
-                   early);
-    } else {
-        launch_pdl(k_color_batched<Qc, T, S, V>, ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), s, tiles, maps, parity, early);
-    }
-}
-
-// f(lattice, shape) with both as compile-time constants
-template <class F>
-void with_shape(int Q, int V, F&& f) {
-    auto shapes = [&](auto q) {
-        switch (V) {
-        case 0: f(q, std::integral_constant<int, 0>{}); break;
-        case 1: f(q, std::integral_constant<int, 1>{}); break;
-        case 2: f(q, std::integral_constant<int, 2>{}); break;
-        case 3: f(q, std::integral_constant<int, 3>{}); break;
-        case 4: f(q, std::integral_constant<int, 4>{}); break;
-        default: f(q, std::integral_constant<int, 5>{}); break;
-        }
+void Launch<T, S>::step_phi_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
+                                    int Vphi, const int4* phi_tiles, int phi_ntiles, int parity, bool ghosts_follow,
+                                    cudaStream_t s) {
+    if (ntiles == 0) return;
+    const int early = ghosts_follow;
+    auto steps = [&](auto q) {
+        constexpr int Qc = decltype(q)::value;
+        if (V == 0) step_batched_v<Qc, 0>(tiles, maps, ntiles, ncontrast, parity, s);
+        if (V == 1) step_batched_v<Qc, 1>(tiles, maps, ntiles, ncontrast, parity, s);
+        if (V == 2) step_batched_v<Qc, 2>(tiles, maps, ntiles, ncontrast, parity, s);
+        if (V == 3) step_batched_v<Qc, 3>(tiles, maps, ntiles, ncontrast, parity, s);
+        if (V == 4) step_batched_v<Qc, 4>(tiles, maps, ntiles, ncontrast, parity, s);
+        if (V == 5) step_batched_v<Qc, 5>(tiles, maps, ntiles, ncontrast, parity, s);
+        // the color kernel on its own tile list (it needs no halo, so its shape
+        // need not be the step's)
+        auto phi = [&](auto v) {
+            constexpr int Vc = decltype(v)::value;
+            using Tl = Tile<Qc, Vc>;
+            launch_pdl(k_phi_batched<Qc, T, S, Vc>, phi_ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), s, phi_tiles, parity, early);
+        };
+        if (Vphi == 0) phi(std::integral_constant<int, 0>{});
+        if (Vphi == 1) phi(std::integral_constant<int, 1>{});
+        if (Vphi == 2) phi(std::integral_constant<int, 2>{});
+        if (Vphi == 3) phi(std::integral_constant<int, 3>{});
+        if (Vphi == 4) phi(std::integral_constant<int, 4>{});
+        if (Vphi == 5) phi(std::integral_constant<int, 5>{});
+        if (Vphi == kPhiRows)
+            launch_pdl(k_phi_rows_batched<Qc, T, S>, phi_ntiles, kPhiChunk, s, phi_tiles, parity, early);
     };
-    if (Q == 9) shapes(std::integral_constant<int, 9>{});
-    else shapes(std::integral_constant<int, 19>{});
-}
-
-template <typename T, typename S>
-void Launch<T, S>::step_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
-                                int parity, cudaStream_t s) {
-    if (ntiles == 0) return;
-    with_shape(Q, V, [&](auto q, auto v) {
-        step_batched_v<decltype(q)::value, decltype(v)::value>(tiles, maps, ntiles, ncontrast, parity, s);
-    });
-}
-
-template <typename T, typename S>
-void Launch<T, S>::color_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int parity,
-                                 bool ghosts_follow, cudaStream_t s) {
-    if (ntiles == 0) return;
-    with_shape(Q, V, [&](auto q, auto v) {
-        color_batched_v<decltype(q)::value, decltype(v)::value>(tiles, maps, ntiles, parity, ghosts_follow, s);
-    });
+    if (Q == 9) steps(std::integral_constant<int, 9>{});
+    else steps(std::integral_constant<int, 19>{});
 }
 
 template <typename T, typename S>
 void Launch<T, S>::fill_entry(void* out, const StepConfig& c, const StepPtrs p[2], bool tma) {
     BatchEntry<T, S> e;
     e.P = params(c);
-    for (int k = 0; k < 2; ++k) e.b[k] = buffers(p[k]);
-    e.tma = tma ? 1 : 0;
+    for (int k = 0; k < 2; ++k) {
+        StepBuffers<T, S>& b = e.b[k];
+        b.Nin = (const S*)p[k].Nin; b.Bin = (const S*)p[k].Bin; b.Nout = (S*)p[k].Nout; b.Bout = (S*)p[k].Bout;
+        b.phi = (T*)p[k].phi; b.u_in = (const T*)p[k].u_in; b.u_out = (T*)p[k].u_out; b.p = (T*)p[k].p;
+        b.mask = p[k].mask; b.err = p[k].err;
+    }
+    e.tma = (sizeof(T) == 4 && tma) ? 1 : 0;
     std::memcpy(out, &e, sizeof(e));
 }
 
@@ -366,20 +336,19 @@ cudaError_t Launch<T, S>::upload_entries(int slot0, const void* entries, int n) 
 }
 
 template <typename T, typename S>
-void Launch<T, S>::ghost_batched(int GK, const void* tabs, const int64_t* begin, int ndom, int64_t total, int parity,
-                                 cudaStream_t s) {
+void Launch<T, S>::ghost_batched(int GK, const void* tabs, const int64_t* begin, int ndom, int64_t total, cudaStream_t s) {
     if (total == 0) return;
     const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (GK == 4) launch_pdl(k_ghost_batched<4, T>, blocks, 256, s, (const GhostTable<T>*)tabs, begin, ndom, total, parity);
-    else launch_pdl(k_ghost_batched<8, T>, blocks, 256, s, (const GhostTable<T>*)tabs, begin, ndom, total, parity);
+    if (GK == 4) launch_pdl(k_ghost_batched<4, T>, blocks, 256, s, (const GhostTable<T>*)tabs, begin, ndom, total);
+    else launch_pdl(k_ghost_batched<8, T>, blocks, 256, s, (const GhostTable<T>*)tabs, begin, ndom, total);
 }
 
 template <typename T, typename S>
 void Launch<T, S>::fill_ghost_table(void* out, int64_t n, const int32_t* node, const int32_t* corner, const void* wt,
-                             double exp_eps, double eps, void* const phi[2], int rule, int64_t plane, int* err) {
+                             double exp_eps, double eps, void* phi, int rule, int64_t plane, int* err) {
     GhostTable<T> g;
     g.n = n; g.node = node; g.corner = corner; g.wt = (const T*)wt; g.exp_eps = (T)exp_eps; g.eps = (T)eps;
-    g.phi[0] = (T*)phi[0]; g.phi[1] = (T*)phi[1]; g.rule = rule; g.plane = plane; g.err = err;
+    g.phi = (T*)phi; g.rule = rule; g.plane = plane; g.err = err;
     std::memcpy(out, &g, sizeof(g));
 }
 

@@ -99,3 +99,30 @@ def test_fields_read_back_whole(shape, precision):
             v[2 * nx * ny:] = 0.0
         d.write(f, v)
         assert np.array_equal(d.read(f).reshape(-1), v.astype(kind).astype(np.float64)), f
+
+
+@pytest.mark.parametrize("precision", [lbm.FP64, lbm.FP32, lbm.FP16])
+@pytest.mark.parametrize("ratio", [1.0, 1000.0])
+@pytest.mark.parametrize("shape", [(1, 33, 65), (17, 18, 70)])
+def test_steps_in_one_call_equal_single_steps(shape, ratio, precision):
+    """A run of steps in one call (captured eight at a time, from either buffer
+    parity) leaves the state of as many single steps, every field, alone and in
+    a batch."""
+    cfg = _case(shape, ratio)
+    P = dict(cfg["params"], precision=precision)
+    doms = [lbm.Domain(P, cfg["solid"], cfg["ghosts"]) for _ in range(3)]
+    for d in doms:
+        d.init_droplet(cfg["center"], cfg["R0"])
+    one, many, mate = doms
+    b = lbm.Batch([mate])
+    for n in (8, 1, 19):
+        for _ in range(n):
+            one.step(1)
+        many.step(n)
+        b.step(n)
+        b.sync()
+        for f in ("N", "B", "phi", "u", "p"):
+            want = one.read(f)
+            assert np.array_equal(many.read(f), want), (n, f)
+            assert np.array_equal(mate.read(f), want), (n, f, "batch")
+    b.close()
