@@ -587,7 +587,7 @@ lbm_status prepare_ghosts(lbm_domain* d, const lbm_ghost* ghosts) {
 }
 
 // ev: optional events {before ghost, before step, before phi, after phi}
-void launch_one_step(lbm_domain* d, int cur, cudaStream_t s, cudaEvent_t* ev = nullptr) {
+void launch_one_step(lbm_domain* d, int cur, bool last, cudaStream_t s, cudaEvent_t* ev = nullptr) {
     const Layout& L = d->lay;
     if (ev) cudaEventRecord(ev[0], s);
     if (d->ng > 0) {
@@ -604,7 +604,7 @@ void launch_one_step(lbm_domain* d, int cur, cudaStream_t s, cudaEvent_t* ev = n
     sp.mask = d->mask(); sp.err = d->errflag();
     if (d->tma) { sp.tm_phi = &d->tm_phi; sp.tm_u = &d->tm_u[cur]; }
     if (ev) cudaEventRecord(ev[1], s);
-    dispatch(d, [&](auto Lx) { decltype(Lx)::step(d->cfg, sp, s); });
+    dispatch(d, [&](auto Lx) { decltype(Lx)::step(d->cfg, sp, last, s); });
     if (ev) cudaEventRecord(ev[2], s);
     dispatch(d, [&](auto Lx) { decltype(Lx)::phi(d->cfg, d->B(1 - cur), d->mask(), d->phi(), d->ng > 0, d->errflag(), s); });
     if (ev) cudaEventRecord(ev[3], s);
@@ -614,7 +614,7 @@ lbm_status capture(lbm_domain* d, int start, int nsteps, cudaGraphExec_t* out) {
     cudaGraph_t g = nullptr;
     CUDA_TRY(d, cudaStreamBeginCapture(d->cap, cudaStreamCaptureModeThreadLocal));
     int c = start;
-    for (int k = 0; k < nsteps; ++k) { launch_one_step(d, c, d->cap); c ^= 1; }
+    for (int k = 0; k < nsteps; ++k) { launch_one_step(d, c, k == nsteps - 1, d->cap); c ^= 1; }
     cudaError_t e = cudaStreamEndCapture(d->cap, &g);
     if (e != cudaSuccess) return fail(d, LBM_ERR_CUDA, std::string("stream capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(out, g, 0);
@@ -964,11 +964,11 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     c.eps = -(4.0 / P.W) * std::cos(P.theta);
     c.exp_eps = std::exp(c.eps);
     c.ghost_rule = P.ghost_rule;
-    // Float arithmetic: the two-node step kernel (half the load/store and
-    // address instructions per node of the one-node kernel; at 192^3 0.967
-    // against 0.919 of the measured copy peak with FP32 storage, 0.667 against
-    // 0.658 of its roofline with FP16 storage).  LBM_STEP_KERNEL=pair|single
-    // overrides; both kernels give the same results to the bit.
+    // Float arithmetic: the two-node kernels (half the load and store
+    // instructions per node of the one-node kernels; 192^3 349 us per step
+    // against 367 with FP32 and 232 against 304 with FP16 storage, 128^3 packing
+    // 120 against 135).  LBM_STEP_KERNEL=pair|single overrides; both give the
+    // same results to the bit.
     const char* step_kernel = std::getenv("LBM_STEP_KERNEL");
     c.pair = P.precision != LBM_FP64 && (step_kernel == nullptr || std::strcmp(step_kernel, "pair") == 0);
 
@@ -1165,7 +1165,7 @@ lbm_status lbm_profile_steps(lbm_domain* d, int64_t n, double kernel_ms[3]) {
     for (int k = 0; k < 4; ++k) CUDA_TRY(d, cudaEventCreate(&ev[k]));
     lbm_status st = LBM_OK;
     for (int64_t t = 0; t < n && st == LBM_OK; ++t) {
-        launch_one_step(d, d->cur, d->stream, ev);
+        launch_one_step(d, d->cur, true, d->stream, ev);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[3]);
         if (e != cudaSuccess) { st = fail(d, LBM_ERR_CUDA, std::string("profiled step: ") + cudaGetErrorString(e)); break; }
@@ -1520,7 +1520,7 @@ void append_tiles(int Q, int V, const lbm_params& P, int i, std::vector<int4>& o
             for (int x = 0; x < P.nx; x += TX) out.push_back(make_int4(i, x, y, z));
 }
 
-void batch_launch_step(lbm_batch* b, int parity, cudaStream_t s) {
+void batch_launch_step(lbm_batch* b, int parity, bool last, cudaStream_t s) {
     const int V = b->variant;
     bdispatch(b->precision, [&](auto Lx) {
         using L = decltype(Lx);
@@ -1529,7 +1529,7 @@ void batch_launch_step(lbm_batch* b, int parity, cudaStream_t s) {
         const int4* pt = Vp == kPhiRows ? b->phi_rows : b->tiles[Vp];
         const int np = Vp == kPhiRows ? b->nphi_rows : b->ntiles[Vp];
         L::step_phi_batched(b->Q, V, b->tiles[V], b->maps + (size_t)V * kBatchSlots * 3, b->ntiles[V],
-                            b->ncontrast[V], Vp, pt, np, parity, b->total_ghosts > 0, s);
+                            b->ncontrast[V], Vp, pt, np, parity, last, b->total_ghosts > 0, s);
     });
 }
 
@@ -1540,8 +1540,8 @@ lbm_status batch_capture(lbm_batch* b) {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return bfail(b, LBM_ERR_CUDA, cudaGetErrorString(e));
-        if (k < 2) batch_launch_step(b, k, b->cap);
-        else for (int t = 0; t < 8; ++t) batch_launch_step(b, t & 1, b->cap);
+        if (k < 2) batch_launch_step(b, k, true, b->cap);
+        else for (int t = 0; t < 8; ++t) batch_launch_step(b, t & 1, t == 7, b->cap);
         const cudaError_t le = cudaGetLastError();          // a launch the capture refused
         e = cudaStreamEndCapture(b->cap, &g);
         if (le != cudaSuccess) {
@@ -1770,7 +1770,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int32_t steps_per_trial, int32_t* chosen
     int best_v = 0;
     for (int V = 0; V < kTileVariants; ++V) {
         b->variant = V;
-        batch_launch_step(b, b->parity, b->stream);        // warm-up step of this shape
+        batch_launch_step(b, b->parity, true, b->stream);  // warm-up step of this shape
         b->parity ^= 1;
         const cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) {
@@ -1781,7 +1781,7 @@ lbm_status lbm_batch_tune(lbm_batch* b, int32_t steps_per_trial, int32_t* chosen
         }
         cudaEventRecord(e0, b->stream);
         for (int t = 0; t < steps_per_trial; ++t) {
-            batch_launch_step(b, b->parity, b->stream);
+            batch_launch_step(b, b->parity, true, b->stream);
             b->parity ^= 1;
         }
         cudaEventRecord(e1, b->stream);

@@ -137,10 +137,10 @@ __device__ __forceinline__ void pull_pair(const StepParams<float>& P, const S* _
 
 // The pair tile at (x0, y0, z0); maps != nullptr: tiled halo copies (the
 // caller checked the tile needs no periodic image in y and z and initialised
-// the barrier).
+// the barrier).  last: as for step_node.
 template <int Q, typename S, bool CONTRAST, int TXn = 64, int TYn = 0>
 __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const StepBuffers<float, S>& b,
-                                               float* s_phi, float* s_u, int x0, int y0, int z0,
+                                               float* s_phi, float* s_u, int x0, int y0, int z0, int last,
                                                const CUtensorMap* tm_phi, const CUtensorMap* tm_u,
                                                uint64_t* bar) {
     using Tl = PairTile<Q, TXn, TYn>;
@@ -204,8 +204,9 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
             *reinterpret_cast<float2*>(PS::rest(b.Nout) + nodeP) = zero;
             *reinterpret_cast<float2*>(PS::rest(b.Bout) + nodeP) = zero;
 #pragma unroll
-            for (int a = 0; a < D; ++a) *reinterpret_cast<float2*>(b.u_out + a * pl + nodeP) = zero;
-            *reinterpret_cast<float2*>(b.p + nodeP) = zero;
+            for (int a = 0; a < D; ++a)
+                if (CONTRAST || last) *reinterpret_cast<float2*>(b.u_out + a * pl + nodeP) = zero;
+            if (last) *reinterpret_cast<float2*>(b.p + nodeP) = zero;
         }
     }
     if (!(fluidA || fluidB) || !halo_ok) return;
@@ -245,9 +246,11 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
     // (the velocity halo reads 0 at solid nodes)
 #pragma unroll
     for (int a = 0; a < D; ++a)
-        *reinterpret_cast<float2*>(b.u_out + a * pl + nodeA) =
-            make_float2(fluidA ? n2.u[a].lo() : 0.f, fluidB ? n2.u[a].hi() : 0.f);
-    *reinterpret_cast<float2*>(b.p + nodeA) = make_float2(fluidA ? n2.p.lo() : 0.f, fluidB ? n2.p.hi() : 0.f);
+        if (CONTRAST || last)
+            *reinterpret_cast<float2*>(b.u_out + a * pl + nodeA) =
+                make_float2(fluidA ? n2.u[a].lo() : 0.f, fluidB ? n2.u[a].hi() : 0.f);
+    if (last)
+        *reinterpret_cast<float2*>(b.p + nodeA) = make_float2(fluidA ? n2.p.lo() : 0.f, fluidB ? n2.p.hi() : 0.f);
     if ((fluidA && !(n2.uu.lo() < 1e30f)) || (fluidB && !(n2.uu.hi() < 1e30f))) atomicOr(err, kErrNonFinite);
 
     auto* __restrict__ NmA = PS::moving(b.Nout, pl) + pop_at<Q>(nodeA);
@@ -282,7 +285,7 @@ template <int Q, typename S, bool CONTRAST, int TXn = 64, int TYn = 0>
 __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
                                   (PairBlocks<PairTile<Q, TXn, TYn>::THREADS>::value))
     k_step_pair(StepParams<float> P, StepBuffers<float, S> b, const __grid_constant__ CUtensorMap tm_phi,
-                const __grid_constant__ CUtensorMap tm_u, int tma) {
+                const __grid_constant__ CUtensorMap tm_u, int tma, int last) {
     using Tl = PairTile<Q, TXn, TYn>;
     constexpr int D = Tl::D;
     __shared__ __align__(128) float s_phi[Tl::HN];
@@ -296,7 +299,8 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();                                      // the barrier exists before anyone waits on it
     }
-    step_pair_tile<Q, S, CONTRAST, TXn, TYn>(P, b, s_phi, s_u, x0, y0, z0, interior ? &tm_phi : nullptr, &tm_u, &s_bar);
+    step_pair_tile<Q, S, CONTRAST, TXn, TYn>(P, b, s_phi, s_u, x0, y0, z0, last, interior ? &tm_phi : nullptr,
+                                             &tm_u, &s_bar);
 }
 
 // Color of the pair from the pulled B*, each node's sum in phi_node's order, so
@@ -346,7 +350,7 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS)
 template <int Q, typename S, bool CONTRAST, int TXn = 64, int TYn = 0>
 __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
                                   (PairBlocks<PairTile<Q, TXn, TYn>::THREADS>::value))
-    k_step_pair_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity) {
+    k_step_pair_batched(const int4* __restrict__ tiles, const CUtensorMap* __restrict__ maps, int parity, int last) {
     using Tl = PairTile<Q, TXn, TYn>;
     constexpr int D = Tl::D;
     __shared__ __align__(128) float s_phi[Tl::HN];
@@ -366,7 +370,8 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
         if (threadIdx.x + threadIdx.y + threadIdx.z == 0) mbar_init(&s_bar, 1);
         __syncthreads();                                      // the barrier exists before anyone waits on it
     }
-    step_pair_tile<Q, S, CONTRAST, TXn, TYn>(e.P, e.b[parity], s_phi, s_u, t.y, y0, z0, tma ? maps + 3 * t.x : nullptr,
+    step_pair_tile<Q, S, CONTRAST, TXn, TYn>(e.P, e.b[parity], s_phi, s_u, t.y, y0, z0, last,
+                                             tma ? maps + 3 * t.x : nullptr,
                                         maps + 3 * t.x + 1 + parity, &s_bar);
 }
 

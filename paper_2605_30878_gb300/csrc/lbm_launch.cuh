@@ -59,8 +59,9 @@ struct Launch {
     template <class Tl>
     static dim3 pair_grid(const Dims& d);
     template <int Q>
-    static void step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
-    static void step(const StepConfig& c, const StepPtrs& p, cudaStream_t s);
+    static void step_q(const StepConfig& c, const StepPtrs& p, int last, cudaStream_t s);
+    // last: store the state that only a caller reads (p; u without density contrast)
+    static void step(const StepConfig& c, const StepPtrs& p, bool last, cudaStream_t s);
     // ghosts_follow: the next kernel on the stream is the ghost kernel
     static void phi(const StepConfig& c, const void* Bst, const uint32_t* mask, void* phi, bool ghosts_follow, int* err,
                     cudaStream_t s);
@@ -84,13 +85,13 @@ struct Launch {
                            cudaStream_t s);
     // ---- batched launches (one block per tile of a flat tile list)
     template <int Qc, int V>
-    static void step_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast, int parity,
+    static void step_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast, int parity, int last,
                                cudaStream_t s);
     // step kernels then color kernel of every domain (the ghost update precedes them);
     // tiles[0, ncontrast) belong to domains with density contrast; the color
     // kernel runs on phi_tiles of shape Vphi, or of row chunks (Vphi == kPhiRows)
     static void step_phi_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
-                                 int Vphi, const int4* phi_tiles, int phi_ntiles, int parity, bool ghosts_follow,
+                                 int Vphi, const int4* phi_tiles, int phi_ntiles, int parity, bool last, bool ghosts_follow,
                                  cudaStream_t s);
     // Slot tables: entry_size() bytes per domain, filled by fill_entry, copied
     // to slots [slot0, slot0 + n) of the constant table by upload_entries.

@@ -93,7 +93,7 @@ dim3 Launch<T, S>::pair_grid(const Dims& d) {
 
 template <typename T, typename S>
 template <int Q>
-void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s) {
+void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, int last, cudaStream_t s) {
     const StepParams<T> P = params(c);
     StepBuffers<T, S> b;
     b.Nin = (const S*)p.Nin; b.Bin = (const S*)p.Bin; b.Nout = (S*)p.Nout; b.Bout = (S*)p.Bout;
@@ -111,9 +111,9 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s
                 using Tl = decltype(tile);
                 const dim3 block(Tl::BX, Tl::TY, Tl::TZ), grid = pair_grid<Tl>(c.d);
                 if (c.contrast)
-                    launch_pdl(k_step_pair<Q, S, true, Tl::TX, Tl::TY>, grid, block, s, P, b, tm_phi, tm_u, tma);
+                    launch_pdl(k_step_pair<Q, S, true, Tl::TX, Tl::TY>, grid, block, s, P, b, tm_phi, tm_u, tma, last);
                 else
-                    launch_pdl(k_step_pair<Q, S, false, Tl::TX, Tl::TY>, grid, block, s, P, b, tm_phi, tm_u, tma);
+                    launch_pdl(k_step_pair<Q, S, false, Tl::TX, Tl::TY>, grid, block, s, P, b, tm_phi, tm_u, tma, last);
             };
             if (c.pair_width == 64) run(PairTile<Q>{}); else run(NarrowTile<Q>{});
             return;
@@ -126,14 +126,14 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, cudaStream_t s
     // nothing more (13.1, 47.2, 26.6).
     constexpr int V = sizeof(T) == 8 ? 3 : 0;
     if (c.contrast)
-        launch_pdl(k_step<Q, T, S, true, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma);
+        launch_pdl(k_step<Q, T, S, true, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma, last);
     else
-        launch_pdl(k_step<Q, T, S, false, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma);
+        launch_pdl(k_step<Q, T, S, false, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma, last);
 }
 
 template <typename T, typename S>
-void Launch<T, S>::step(const StepConfig& c, const StepPtrs& p, cudaStream_t s) {
-    if (c.Q == 9) step_q<9>(c, p, s); else step_q<19>(c, p, s);
+void Launch<T, S>::step(const StepConfig& c, const StepPtrs& p, bool last, cudaStream_t s) {
+    if (c.Q == 9) step_q<9>(c, p, last, s); else step_q<19>(c, p, last, s);
 }
 
 template <typename T, typename S>
@@ -254,7 +254,7 @@ void Launch<T, S>::gather_dir(const StepConfig& c, const uint8_t* cls, int i, bo
 // ---- batched launches (one block per tile of a flat tile list)
 template <typename T, typename S>
 template <int Qc, int V>
-void Launch<T, S>::step_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast, int parity,
+void Launch<T, S>::step_batched_v(const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast, int parity, int last,
                                   cudaStream_t s) {
     using Tl = Tile<Qc, V>;
     const dim3 block(Tl::TX, Tl::TY, Tl::TZ);     // the tile shape, as in the single-domain kernels
@@ -266,16 +266,15 @@ void Launch<T, S>::step_batched_v(const int4* tiles, const CUtensorMap* maps, in
         static_assert(Pt::TX == Tl::TX && Pt::TY == Tl::TY && Pt::TZ == Tl::TZ, "the pair tile covers the shape's tile");
         const dim3 pblock(Pt::BX, Pt::TY, Pt::TZ);
         if (ncontrast > 0)
-            launch_pdl(k_step_pair_batched<Qc, S, true, TXn, TYn>, ncontrast, pblock, s, tiles, maps, parity);
+            launch_pdl(k_step_pair_batched<Qc, S, true, TXn, TYn>, ncontrast, pblock, s, tiles, maps, parity, last);
         if (ntiles > ncontrast)
             launch_pdl(k_step_pair_batched<Qc, S, false, TXn, TYn>, ntiles - ncontrast, pblock, s, tiles + ncontrast,
-                                                                                             maps, parity);
+                                                                                             maps, parity, last);
     } else {
         if (ncontrast > 0)
-            launch_pdl(k_step_batched<Qc, T, S, V, true>, ncontrast, block, s, tiles, maps, parity);
+            launch_pdl(k_step_batched<Qc, T, S, V, true>, ncontrast, block, s, tiles, maps, parity, last);
         if (ntiles > ncontrast)
-            launch_pdl(k_step_batched<Qc, T, S, V, false>, ntiles - ncontrast, block, s, tiles + ncontrast, maps,
-                                                                                    parity);
+            launch_pdl(k_step_batched<Qc, T, S, V, false>, ntiles - ncontrast, block, s, tiles + ncontrast, maps, parity, last);
     }
 }
 
@@ -283,18 +282,18 @@ void Launch<T, S>::step_batched_v(const int4* tiles, const CUtensorMap* maps, in
 // tiles[0, ncontrast) belong to domains with density contrast
 template <typename T, typename S>
 void Launch<T, S>::step_phi_batched(int Q, int V, const int4* tiles, const CUtensorMap* maps, int ntiles, int ncontrast,
-                                    int Vphi, const int4* phi_tiles, int phi_ntiles, int parity, bool ghosts_follow,
+                                    int Vphi, const int4* phi_tiles, int phi_ntiles, int parity, bool last, bool ghosts_follow,
                                     cudaStream_t s) {
     if (ntiles == 0) return;
     const int early = ghosts_follow;
     auto steps = [&](auto q) {
         constexpr int Qc = decltype(q)::value;
-        if (V == 0) step_batched_v<Qc, 0>(tiles, maps, ntiles, ncontrast, parity, s);
-        if (V == 1) step_batched_v<Qc, 1>(tiles, maps, ntiles, ncontrast, parity, s);
-        if (V == 2) step_batched_v<Qc, 2>(tiles, maps, ntiles, ncontrast, parity, s);
-        if (V == 3) step_batched_v<Qc, 3>(tiles, maps, ntiles, ncontrast, parity, s);
-        if (V == 4) step_batched_v<Qc, 4>(tiles, maps, ntiles, ncontrast, parity, s);
-        if (V == 5) step_batched_v<Qc, 5>(tiles, maps, ntiles, ncontrast, parity, s);
+        if (V == 0) step_batched_v<Qc, 0>(tiles, maps, ntiles, ncontrast, parity, last, s);
+        if (V == 1) step_batched_v<Qc, 1>(tiles, maps, ntiles, ncontrast, parity, last, s);
+        if (V == 2) step_batched_v<Qc, 2>(tiles, maps, ntiles, ncontrast, parity, last, s);
+        if (V == 3) step_batched_v<Qc, 3>(tiles, maps, ntiles, ncontrast, parity, last, s);
+        if (V == 4) step_batched_v<Qc, 4>(tiles, maps, ntiles, ncontrast, parity, last, s);
+        if (V == 5) step_batched_v<Qc, 5>(tiles, maps, ntiles, ncontrast, parity, last, s);
         // the color kernel on its own tile list (it needs no halo, so its shape
         // need not be the step's)
         auto phi = [&](auto v) {
