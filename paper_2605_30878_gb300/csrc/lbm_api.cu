@@ -1446,10 +1446,13 @@ struct lbm_batch {
     int parity = 0;                    // steps taken by the batch, mod 2
     int variant = 0;
     // tiles of the color kernel, whatever shape the step kernels use (it has
-    // no halo): row chunks of 128 nodes (kPhiRows), which leave only the
-    // padding columns idle.  LBM_BATCH_PHI_SHAPE=step: the step's shape;
-    // =0..5: that shape (shape 3, 32 x 2 x 2, ran a batch of 64 domains of 48^3 to 128^3 at 3.305 ms per
-    // step against 3.331 on the step's 64-wide tiles).
+    // no halo).  D3Q19 and FP64: row chunks of 128 nodes (kPhiRows), which leave
+    // only the padding columns idle.  D2Q9 in float: shape 0, two nodes per
+    // thread.  us per step, chunks against shapes 0, 3 and 5: twelve 3D domains
+    // FP32 295 against 299, 298, 304, FP16 storage 245 against 249, 249, 259;
+    // sixteen 2D domains FP32 49.2 against 47.3, 49.8, 47.2, FP16 storage 42.4
+    // against 38.5, 43.3, 38.9.  LBM_BATCH_PHI_SHAPE=rows: chunks; =step: the
+    // step's shape; =0..5: that shape.
     int phi_shape = kPhiRows;
     int4* phi_rows = nullptr;          // {slot, x0, y0, z} row chunks
     int nphi_rows = 0;
@@ -1586,6 +1589,7 @@ lbm_status lbm_batch_create(lbm_domain* const* doms, int32_t n, void* cuda_strea
         b->cur0.push_back(doms[i]->cur);
     }
     b->stream = (cudaStream_t)cuda_stream;
+    if (b->Q == 9 && b->precision != LBM_FP64) b->phi_shape = 0;
     const char* phi_shape = std::getenv("LBM_BATCH_PHI_SHAPE");
     if (phi_shape && std::strcmp(phi_shape, "step") == 0) b->phi_shape = -1;
     else if (phi_shape && std::strcmp(phi_shape, "rows") == 0) b->phi_shape = kPhiRows;

@@ -299,7 +299,14 @@ void Launch<T, S>::step_phi_batched(int Q, int V, const int4* tiles, const CUten
         auto phi = [&](auto v) {
             constexpr int Vc = decltype(v)::value;
             using Tl = Tile<Qc, Vc>;
-            launch_pdl(k_phi_batched<Qc, T, S, Vc>, phi_ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), s, phi_tiles, parity, early);
+            if constexpr ((Vc == 5 || Vc == 3 || Vc == 0) && sizeof(T) == 4) {
+                using Pt = PairTile<Qc, Tl::TX, Tl::TY>;
+                launch_pdl(k_phi_pair_batched<Qc, S, Tl::TX, Tl::TY>, phi_ntiles, dim3(Pt::BX, Pt::TY, Pt::TZ), s,
+                           phi_tiles, parity, early);
+            } else {
+                launch_pdl(k_phi_batched<Qc, T, S, Vc>, phi_ntiles, dim3(Tl::TX, Tl::TY, Tl::TZ), s, phi_tiles, parity,
+                           early);
+            }
         };
         if (Vphi == 0) phi(std::integral_constant<int, 0>{});
         if (Vphi == 1) phi(std::integral_constant<int, 1>{});
