@@ -1372,8 +1372,8 @@ double lbm_bytes_per_fluid_node(const lbm_domain* d) {
     const double s = (double)d->lay.elem;
     const double moving = (d->lay.Q - 1) * (double)d->lay.pop_elem;
     const double pop = (double)d->lay.rest_elem + moving;   // per node and array
-    // k_step pulls N: the FP64 update follows the literal collision and reads the
-    // rest population, the float updates take every moment from the moving ones
+    // k_step pulls N and takes every moment from the moving populations; the FP64
+    // count still holds the rest population's pull
     const double pull = d->lay.elem == 8 ? pop : moving;
     const int D = d->lay.D;
     // N* and B* written, B* pulled by k_phi; phi written (k_phi) and read (k_step);
@@ -1449,9 +1449,9 @@ struct lbm_batch {
     // no halo).  D3Q19 and FP64: row chunks of 128 nodes (kPhiRows), which leave
     // only the padding columns idle.  D2Q9 in float: shape 0, two nodes per
     // thread.  us per step, chunks against shapes 0, 3 and 5: twelve 3D domains
-    // FP32 295 against 299, 298, 304, FP16 storage 245 against 249, 249, 259;
-    // sixteen 2D domains FP32 49.2 against 47.3, 49.8, 47.2, FP16 storage 42.4
-    // against 38.5, 43.3, 38.9.  LBM_BATCH_PHI_SHAPE=rows: chunks; =step: the
+    // FP32 296 against 298, 297, 303, FP16 storage 247 against 249, 248, 258;
+    // sixteen 2D domains FP32 49.5 against 46.2, 49.0, 46.5, FP16 storage 42.6
+    // against 39.0, 43.2, 39.6.  LBM_BATCH_PHI_SHAPE=rows: chunks; =step: the
     // step's shape; =0..5: that shape.
     int phi_shape = kPhiRows;
     int4* phi_rows = nullptr;          // {slot, x0, y0, z} row chunks

@@ -375,13 +375,13 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
                                         maps + 3 * t.x + 1 + parity, &s_bar);
 }
 
-// Batched color kernel of the two-node tile shapes: bound as k_phi_pair, chosen
-// for D2Q9 (sixteen 2D domains, per step against row chunks: FP32 49.2 -> 47.3 us,
-// FP16 storage 42.4 -> 38.5).
+// Batched color kernel of the two-node tile shapes, bound as k_phi_pair.  Where
+// the batch takes it instead of row chunks, and both sides measured, stands at
+// the batch's choice of its color tiles (lbm_batch::phi_shape).
 template <int Q, typename S, int TXn, int TYn>
 __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS)
     k_phi_pair_batched(const int4* __restrict__ tiles, int parity, int early) {
-    const int4 t = __ldg(tiles + blockIdx.x);          // {slot, x0, y0, z0}
+    const int4 t = __ldg(tiles + (gridDim.x - 1 - blockIdx.x));     // {slot, x0, y0, z0}, reverse order, as k_phi
     const BatchEntry<float, S>& e = c_batch<float, S>[idx_checked(t.x, kBatchSlots, c_batch<float, S>[0].b[0].err)];
     const StepBuffers<float, S>& b = e.b[parity];
     phi_pair<Q, S>(e.P, b.Bout, b.mask, b.phi, t.y, t.z, t.w, early, b.err);
