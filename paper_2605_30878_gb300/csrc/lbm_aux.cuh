@@ -162,7 +162,7 @@ __global__ void k_init_pops(Dims d, StepParams<T> P, const uint8_t* __restrict__
             const T e = P.chi_err[i == 0 ? 0 : (L::cx(i) * L::cx(i) + L::cy(i) * L::cy(i) + L::cz(i) * L::cz(i) == 1
                                                     ? 1 : 2)];
             pop_store<Q, S, T>(Nst, i, pl, nd, kShift ? e : P.chi[i], kScaleN);
-            pop_store<Q, S, T>(Bst, i, pl, nd, PopStore<S>::kShiftB ? (ph - T(0.5)) * P.chi[i] + ph * e : ph * P.chi[i], kScaleB);
+            pop_store<Q, S, T>(Bst, i, pl, nd, kShift ? (ph - T(0.5)) * P.chi[i] + ph * e : ph * P.chi[i], kScaleB);
         }
     }
 }

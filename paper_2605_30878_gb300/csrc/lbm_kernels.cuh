@@ -59,14 +59,16 @@ struct StepParams {
     T exp_eps;               // exp(eps), eps = -(4/W) cos(theta)
 };
 
-// Population storage.  N is stored as its deviation from the rest state,
-// N_i - chi_i, in every mode; the step computes directly in these deviations,
-// an exact rewrite because sum chi = 1, sum c chi = 0 and chi is isotropic, and
-// it keeps the small pressure of a dense liquid (p = p_h/rho ~ 1e-8 at density
-// ratio 1000) representable.  B: full values in S = double (FP64 mode),
-// B_i - chi_i/2 in S = float (FP32 mode).  S = __half: the same deviations, the rest
+// Population storage.  S = double (FP64 mode): full values, the ones the state
+// transfer hands out, so that a state read and written back goes on to the bit
+// (N_i - chi_i holds bits that N_i in double does not).  S = float (FP32 mode):
+// deviations from the rest state, N_i - chi_i and B_i - chi_i/2, which keep the
+// small pressure of a dense liquid (p = p_h/rho ~ 1e-8 at density ratio 1000)
+// representable.  S = __half: the same deviations, the rest
 // populations (i = 0, whose B deviation reaches chi_0/2 ~ 0.46) as float in the
 // first plane, the moving ones times 2^16 (N) and 2^7 (B) as FP16 after it.
+// The step computes in deviations of N in every mode, an exact rewrite because
+// sum chi = 1, sum c chi = 0 and chi is isotropic.
 constexpr float kScaleN = 65536.0f;
 constexpr float kScaleB = 128.0f;
 
@@ -116,10 +118,10 @@ template <typename V> struct PlainStore {
     __device__ static void store_units(V* m, int idx, V v, V&) { m[idx] = v; }
 };
 template <> struct PopStore<double> : PlainStore<double> {
-    static constexpr bool kShift = true, kShiftB = false, kExact = true;
+    static constexpr bool kShift = false, kExact = true;
 };
 template <> struct PopStore<float> : PlainStore<float> {
-    static constexpr bool kShift = true, kShiftB = true, kExact = true;
+    static constexpr bool kShift = true, kExact = true;
     // two adjacent nodes (idx even, so 8-byte aligned): values in storage units
     __device__ static float2 load_units2(const float* m, int idx) {
         return __ldg(reinterpret_cast<const float2*>(m + idx));
@@ -130,7 +132,7 @@ template <> struct PopStore<float> : PlainStore<float> {
     __device__ static void store_zero2(float* m) { *reinterpret_cast<float2*>(m) = make_float2(0.f, 0.f); }
 };
 template <> struct PopStore<__half> {
-    static constexpr bool kShift = true, kShiftB = true, kExact = false;     // moving populations are rounded on store
+    static constexpr bool kShift = true, kExact = false;     // moving populations are rounded on store
     static constexpr int kRestBytes = 4, kMovingBytes = 2;
     __device__ static const float* rest(const __half* p) { return reinterpret_cast<const float*>(p); }
     __device__ static float* rest(__half* p) { return reinterpret_cast<float*>(p); }
@@ -441,16 +443,16 @@ __device__ __forceinline__ void phi_node(const StepParams<T>& P, const S* __rest
     // a grid coarse enough for their float sum to be exact, so the node's color
     // comes back as k_step wrote it.
     const T rest = (T)PS::load_rest(PS::rest(Bst), node);
-    T s = PS::kShiftB ? T(0) : rest;
+    T s = PS::kShift ? T(0) : rest;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const bool back = (m >> i) & 1u;
         const int from = idx_checked(back ? node : node + W.off(-L::cx(i), -L::cy(i), -L::cz(i)), P.plane, err);
         PS::accumulate(mv + pop_at<Q>(from), back ? pop_dir(L::opp(i)) : pop_dir(i), s);
     }
-    if (PS::kShiftB) s = rest + (PS::kExact ? s : s * T(1.0 / kScaleB));
+    if (PS::kShift) s = rest + (PS::kExact ? s : s * T(1.0 / kScaleB));
     // stored deviations B_i - chi_i/2 sum to phi - 1/2
-    phi[node] = PS::kShiftB ? T(0.5) + s : s;
+    phi[node] = PS::kShift ? T(0.5) + s : s;
 }
 
 template <int Q, typename T, typename S>
@@ -700,15 +702,16 @@ struct Acc {
 // ---------------------------------------------------------------------------
 // FP64 runs it too: this GPU's FP64 rate (two lanes per clock and SM) makes the
 // FP64 step bound by its FP64 instructions alone, so what counts is how few a
-// node takes: ~580 in D3Q19 and ~280 in D2Q9 in this form, against ~2400 and
+// node takes: ~600 in D3Q19 and ~290 in D2Q9 in this form, against ~2400 and
 // ~1150 for the model's expressions evaluated as printed (a division by each
-// constant, no fused multiply-add): 64^3 1237 -> 240 us per step, 500 x 300
-// 308 -> 71 us.
+// constant, no fused multiply-add): 64^3 1092 -> 246 us per step, 500 x 300
+// 288 -> 70 us.  N stored as its deviation would save 16 of them (237 and 69 us),
+// but a state read and written back would then not go on to the bit.
 //
 // Arithmetic of one fluid node (V = SF, or SD in FP64), or of the two nodes of a
 // pair (V = F2, one packed lane each), written once so that the one-node and the
-// two-node kernels round alike.  Inputs: the pulled populations N
-// (deviations, in storage units with FP16 storage), the color phi at the node
+// two-node kernels round alike.  Inputs: the pulled populations N as stored
+// (deviations, in storage units with FP16 storage; full values in FP64), the color phi at the node
 // and its isotropic stencils gp = grad phi, lap = lap phi and gu[a][b] = d_a u_b
 // (the stencil weights carry the 3 and the 6).
 //
@@ -727,23 +730,27 @@ struct NodeUpdate {
     // (the stress projections, the weights, phi, kseg) and the scaled values
     // round exactly as the unscaled ones would.
     static constexpr R sN = UNITS ? kScaleN : 1, sB = UNITS ? kScaleB : 1;
-    // B is stored in full in FP64, as its deviation from chi/2 in float
-    static constexpr bool kFullB = sizeof(R) == 8;
+    // N and B are stored in full in FP64, as deviations from chi and chi/2 in float
+    static constexpr bool kFull = sizeof(R) == 8;
     V phi, u[3], uu, p;
     V F[3], gp[3];
     V A0, A1, Axy, Axz, Ayz;                   // stress projections of N - Neq, times (1 - 1/tau)
     V base0, base1, base2, three_p, halfF;
     V common1, common2, krc1, krc2;            // per direction class (1 axis, 2 diagonal/edge)
-    V shb1, shb2;                              // (phi - 1/2) chi_i per class, in B's units (FP64: phi chi_i)
+    V shb1, shb2;                              // (phi - 1/2) chi_i per class, in B's units (float)
+    R chi1, chi2;                              // chi_i per class (FP64)
     V phiB;
 
-    // raw moments of the pulled N (storage units): sum, first and second moments
+    // raw moments of the pulled N's deviations (storage units): sum, first and second moments
     V m_sum, m_u0[3], m_xx, m_yy, m_zz, m_xy, m_xz, m_yz;
 
     // The moments need only the pulled populations, not the halo: the two-node
     // kernel takes them before its barrier, so that the pulled values are not
-    // held across the stencils.
-    __device__ __forceinline__ void moments(const V (&N)[Q]) {
+    // held across the stencils.  Full values give the deviations' sum as
+    // (N_i - 2 chi_i) + N_opp and their difference as N_i - N_opp: near the rest
+    // state both are exact (but for the last bit of N_i - 2 chi_i where it crosses a
+    // power of two), at one operation more per pair.
+    __device__ __forceinline__ void moments(const StepParams<R>& P, const V (&N)[Q]) {
         // force-free velocity and the moments of Eq. (pressureUpdate) and the collision
         Acc<V> u0s[3], sm, Pxx, Pyy, Pzz, Pxy, Pxz, Pyz;
 #pragma unroll
@@ -751,7 +758,8 @@ struct NodeUpdate {
             const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
             // odd moments from N_i - N_opp, even ones from N_i + N_opp
             if (L::opp(i) < i) continue;
-            const V sp = N[i] + N[L::opp(i)], dp = N[i] - N[L::opp(i)];
+            const V sp = (kFull ? fma(V(R(-2.0)), V(P.chi[i]), N[i]) : N[i]) + N[L::opp(i)];
+            const V dp = N[i] - N[L::opp(i)];
             sm.add(1, sp);
             u0s[0].add(cx, dp);
             u0s[1].add(cy, dp);
@@ -772,7 +780,7 @@ struct NodeUpdate {
 
     __device__ __forceinline__ void compute(const StepParams<R>& P, const V (&N)[Q], V phi_, const V (&gp_)[3],
                                             V lap, const V (&gu)[3][3]) {
-        moments(N);
+        moments(P, N);
         compute(P, phi_, gp_, lap, gu);
     }
 
@@ -870,9 +878,11 @@ struct NodeUpdate {
         const V kseg = V(P.two_over_W) * phi * (V(R(1.0)) - phi) * inv_gn;
         const V ksegB = UNITS ? kseg * V(sB) : kseg;                        // recoloring in B's units
         phiB = UNITS ? phi * V(sB / sN) : phi;                              // phi N*, from N's units to B's
-        const V phmB = kFullB ? phi : (UNITS ? (phi - V(R(0.5))) * V(sB) : phi - V(R(0.5)));
+        const V phmB = UNITS ? (phi - V(R(0.5))) * V(sB) : phi - V(R(0.5));
         shb1 = phmB * V(P.chi[1]);
         shb2 = phmB * V(P.chi[D == 2 ? 5 : 7]);
+        chi1 = P.chi[1];
+        chi2 = P.chi[D == 2 ? 5 : 7];
         three_p = V(R(3.0)) * p;
         halfF = V(R(1.5)) * inv_rho;   // (1/2) F_i = (3/2) w_i (c_i . F)/rho
         const V common = fma(V(R(-1.5)), uu, three_p);
@@ -889,7 +899,8 @@ struct NodeUpdate {
     // Direction i (opp(i) > i) and its opposite o, in storage units: the
     // post-collision N*_i - chi_i, N*_o - chi_o (they share the even part and
     // flip the odd part) and B*_i - chi_i/2, B*_o - chi_o/2 with
-    // B* = phi N* + recolor, i.e. phi dN* + (phi - 1/2) chi_i + recolor.
+    // B* = phi N* + recolor, i.e. phi dN* + (phi - 1/2) chi_i + recolor.  FP64: the
+    // full values, chi_i added to the even part.
     __device__ __forceinline__ void dir(int i, V& ni, V& no, V& bi, V& bo) const {
         const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
         const R wiN = R(L::w(i)) * sN;
@@ -913,22 +924,29 @@ struct NodeUpdate {
         const bool axis = cx * cx + cy * cy + cz * cz == 1;
         const V krc = axis ? krc1 : krc2, g = cg.get();                // recoloring krc (c . grad phi), odd in c
         const V c3 = cu3.get();
-        const V even = fma(V(wiN), fma(V(R(0.5)) * c3, c3, axis ? common1 : common2), proj.get());
+        V even = fma(V(wiN), fma(V(R(0.5)) * c3, c3, axis ? common1 : common2), proj.get());
+        if constexpr (kFull) even = even + V(axis ? chi1 : chi2);
         const V odd = fma(halfF, cF.get(), c3);                        // the odd part over wiN
         ni = fma(V(wiN), odd, even);
         no = fma(V(-wiN), odd, even);
-        const V shift_b = axis ? shb1 : shb2;                          // (phi - 1/2) chi_i
-        bi = fma(krc, g, fma(phiB, ni, shift_b));
-        bo = fma(-krc, g, fma(phiB, no, shift_b));
+        if constexpr (kFull) {
+            bi = fma(krc, g, phiB * ni);
+            bo = fma(-krc, g, phiB * no);
+        } else {
+            const V shift_b = axis ? shb1 : shb2;                      // (phi - 1/2) chi_i
+            bi = fma(krc, g, fma(phiB, ni, shift_b));
+            bo = fma(-krc, g, fma(phiB, no, shift_b));
+        }
     }
 
     // Rest direction (no forcing, no stress projection, no recoloring, c_0 = 0),
-    // stored exactly (FP32): N*_0 - chi_0 and B*_0 - chi_0/2.
+    // stored exactly: N*_0 - chi_0 and B*_0 - chi_0/2 (FP32), N*_0 and B*_0 (FP64).
     __device__ __forceinline__ V rest_N(const StepParams<R>& P) const {
-        return fma(V(-R(1.5 * w0)), uu, fma(V(-R(1.0 - w0)), three_p, V(P.chi_err[0])));
+        return fma(V(-R(1.5 * w0)), uu, fma(V(-R(1.0 - w0)), three_p, V(kFull ? P.chi[0] : P.chi_err[0])));
     }
     __device__ __forceinline__ V rest_B(const StepParams<R>& P, V nst0) const {
-        return fma(phi, nst0, (kFullB ? phi : phi - V(R(0.5))) * V(P.chi[0]));
+        if constexpr (kFull) return phi * nst0;
+        return fma(phi, nst0, (phi - V(R(0.5))) * V(P.chi[0]));
     }
     // With FP16 storage the float rest populations take the node totals the
     // collision fixes less the moving populations as stored (sumN, sumB in
@@ -962,7 +980,6 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
     // every store index below follows from this node
     if (!idx_ok(node, P.plane, err)) return;
     using PS = PopStore<S>;
-    constexpr bool kShift = PS::kShift;
 
     // isotropic stencils: grad f = 3 sum_i w_i c_i f(x+c_i), lap f = 6 sum_i w_i (f(x+c_i) - f(x)),
     // summed over +/- pairs (half the multiply-adds)
@@ -996,7 +1013,7 @@ __device__ __forceinline__ void step_node(const StepParams<T>& P, const StepBuff
             }
         }
     }
-    static_assert(kShift, "the node update runs on deviations");
+    static_assert(PS::kShift == (sizeof(T) == 4), "NodeUpdate takes full values in FP64, deviations in float");
     constexpr bool kUnits = !PS::kExact;
     using Sc = typename ScalarOf<T>::type;
     using FN = NodeUpdate<Q, kUnits, CONTRAST, Sc>;

@@ -169,7 +169,7 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
         F2 N2[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) N2[i] = F2(NA[i], NB[i]);
-        n2.moments(N2);
+        n2.moments(P, N2);
     }
     const bool halo_ok = halo_complete<Tl, float, S>(b, interior, bar, s_phi, s_u, fx);
     __syncthreads();

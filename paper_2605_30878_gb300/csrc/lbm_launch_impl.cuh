@@ -218,7 +218,7 @@ void Launch<T, S>::build_mask(const StepConfig& c, const uint8_t* cls, uint32_t*
 // base subtracted from direction i of N (is_b = false) or B (true) in storage
 template <typename T, typename S>
 double Launch<T, S>::storage_base(const StepConfig& c, int i, bool is_b) {
-    if (!(is_b ? PopStore<S>::kShiftB : PopStore<S>::kShift)) return 0.0;
+    if (!PopStore<S>::kShift) return 0.0;
     double chi[19];                     // the deviations are taken from the chi the kernels use
     if (sizeof(T) == 4) chi_for_float(c.chi, chi);
     else std::memcpy(chi, c.chi, sizeof(chi));

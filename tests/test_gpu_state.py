@@ -1,0 +1,52 @@
+"""State taken out of a domain and put back, and reads from several threads."""
+import math
+
+import numpy as np
+import pytest
+
+from paper_2605_30878_gb300 import lbm
+from paper_2605_30878_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+FIELDS = ("N", "B", "phi", "u", "p")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2605_30878_gb300 import build
+    build.build()
+    lbm.load()
+
+
+def _drop(shape, ratio, precision, **where):
+    nz, ny, nx = shape
+    Q = 9 if nz == 1 else 19
+    small = min(n for n in shape if n > 1)
+    center = (0.5 * nx, 0.45 * ny, 0.5 * nz if nz > 1 else 0.0)
+    solid, ghosts = wl.sphere_domain(Q, shape, center, 0.2 * small)
+    params = dict(lattice=Q, nx=nx, ny=ny, nz=nz, periodic=7, rho_l=ratio, rho_g=1.0, mu_l=0.1 * ratio ** 0.5, mu_g=0.1,
+                  sigma=0.005, W=4.0, M_phi=0.02, theta=math.radians(70.0), g=(1e-6, -2e-6, 0.0), precision=precision)
+    d = lbm.Domain(params, solid, ghosts, **where)
+    d.init_droplet((center[0], center[1] + 0.25 * small, center[2]), 0.2 * small)
+    return d
+
+
+@pytest.mark.parametrize("ratio", [1.0, 1000.0])
+@pytest.mark.parametrize("shape", [(1, 33, 41), (18, 19, 22)])
+def test_fp64_state_written_back_goes_on_to_the_bit(shape, ratio):
+    """A run stopped, its fields written into a fresh domain and gone on with
+    (either buffer parity) is the run that was not stopped."""
+    one = _drop(shape, ratio, lbm.FP64)
+    for n in (5, 12):
+        one.step(n)
+        two = _drop(shape, ratio, lbm.FP64)
+        for f in FIELDS:
+            two.write(f, one.read(f))
+        one.step(7)
+        two.step(7)
+        for f in FIELDS:
+            assert np.array_equal(one.read(f), two.read(f)), (n, f)
