@@ -705,7 +705,7 @@ struct Acc {
 // node takes: ~600 in D3Q19 and ~290 in D2Q9 in this form, against ~2400 and
 // ~1150 for the model's expressions evaluated as printed (a division by each
 // constant, no fused multiply-add): 64^3 1092 -> 246 us per step, 500 x 300
-// 288 -> 70 us.  N stored as its deviation would save 16 of them (237 and 69 us),
+// 288 -> 71 us.  N stored as its deviation would save 16 of them (237 and 69 us),
 // but a state read and written back would then not go on to the bit.
 //
 // Arithmetic of one fluid node (V = SF, or SD in FP64), or of the two nodes of a
@@ -792,9 +792,20 @@ struct NodeUpdate {
         for (int a = 0; a < 3; ++a) gp[a] = gp_[a];
 
         // mixture density and viscosity (Sec. II), relaxation time (Appendix A)
-        const V rho = fma(V(P.drho), phi, V(P.rho_g));
+        V rho, inv_nu;                                   // 1/nu = phi/nu_l + (1-phi)/nu_g
+        if constexpr (kFull) {
+            // sums of positive terms: in the float form below a large viscosity or
+            // small density of the liquid is the difference of two large numbers
+            // (nu_l/nu_g = 1000: 1/nu 2e-14 off); 3 operations more per node
+            const V gas = V(R(1.0)) - phi;
+            rho = fma(V(P.rho_l), phi, V(P.rho_g) * gas);
+            inv_nu = fma(phi, V(P.inv_nu_l), gas * V(P.inv_nu_g));
+        } else {
+            rho = fma(V(P.drho), phi, V(P.rho_g));
+            inv_nu = fma(phi, V(P.inv_nu_l - P.inv_nu_g), V(P.inv_nu_g));
+        }
         const V inv_rho = rcp(rho);
-        const V nu = rcp(fma(phi, V(P.inv_nu_l - P.inv_nu_g), V(P.inv_nu_g)));   // 1 / (phi/nu_l + (1-phi)/nu_g)
+        const V nu = rcp(inv_nu);
         const V tau = fma(V(R(3.0)), nu, V(R(0.5)));
 
         // FP16 storage: N came in storage units (times sN = 2^16); the moments are
