@@ -743,7 +743,9 @@ lbm_status upload_as(lbm_domain* d, void* dst, const double* src) {
 // per device, made on first use and kept: a copy into it runs at the link's
 // rate and beside the conversion of the half before, and neither pages of a
 // fresh buffer nor the driver's own staging cost anything.  One read uses it at
-// a time; lbm_release_cached_memory gives it back.
+// a time, from the copy it queues behind its domain's steps to the last value;
+// a read that finds it taken goes through a buffer of its own and waits for
+// nothing but its own domain.  lbm_release_cached_memory gives it back.
 struct ReadStage {
     static constexpr size_t kHalf = (size_t)4 << 20;
     std::mutex use;
@@ -800,8 +802,9 @@ lbm_status download_as(lbm_domain* d, double* dst, const V* src, int planes, int
     const int64_t nx = d->prm.nx, px = L.px, rows = L.nn_dense / nx;
     const int64_t row_bytes = px * (int64_t)sizeof(V);
     ReadStage& st = read_stage();
-    std::lock_guard<std::mutex> one_read(st.use);
-    if (row_bytes > (int64_t)ReadStage::kHalf || !st.ready()) {
+    std::unique_lock<std::mutex> one_read(st.use, std::try_to_lock);
+    if (!one_read.owns_lock() || row_bytes > (int64_t)ReadStage::kHalf || !st.ready()) {
+        if (one_read.owns_lock()) one_read.unlock();
         std::vector<V> tmp((size_t)L.nn);
         for (int a = 0; a < planes; ++a) {
             CUDA_TRY(d, cudaMemcpyAsync(tmp.data(), src + a * src_step, tmp.size() * sizeof(V), cudaMemcpyDeviceToHost,
@@ -1422,12 +1425,15 @@ lbm_status lbm_release_cached_memory(void) {
             return LBM_ERR_CUDA;
         }
     }
+    // a stage in use is waited for, with no lock held that a read elsewhere takes
+    std::vector<std::pair<int, ReadStage*>> stages;
     {
         std::lock_guard<std::mutex> ls(g_stage_mutex);
-        for (auto& kv : g_stages) {
-            cudaSetDevice(kv.first);
-            kv.second->release();
-        }
+        for (auto& kv : g_stages) stages.push_back({kv.first, kv.second.get()});
+    }
+    for (auto& s : stages) {
+        cudaSetDevice(s.first);
+        s.second->release();
     }
     cudaSetDevice(cur);
     return LBM_OK;

@@ -1,5 +1,7 @@
 """State taken out of a domain and put back, and reads from several threads."""
 import math
+import threading
+import time
 
 import numpy as np
 import pytest
@@ -50,3 +52,33 @@ def test_fp64_state_written_back_goes_on_to_the_bit(shape, ratio):
         two.step(7)
         for f in FIELDS:
             assert np.array_equal(one.read(f), two.read(f)), (n, f)
+
+
+@pytest.mark.parametrize("precision", [lbm.FP64, lbm.FP32])
+def test_read_of_an_idle_domain_does_not_wait_for_another_domain(precision):
+    """One thread reads a domain with a second or so of steps queued; meanwhile the
+    read of an idle domain on another stream returns, with the right values."""
+    import torch
+    busy_stream, idle_stream = torch.cuda.Stream(), torch.cuda.Stream()
+    shape = (48, 96, 96)
+    busy, idle = _drop(shape, 10.0, precision, stream=busy_stream), _drop(shape, 10.0, precision, stream=idle_stream)
+    idle.step(8)
+    want = {f: idle.read(f) for f in ("phi", "u")}
+    busy.step(8)
+    for f in want:
+        assert np.array_equal(busy.read(f), want[f])
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record(busy_stream)
+    busy.step(80)
+    end.record(busy_stream)
+    busy.sync()
+    busy.step(int(80 * 1200.0 / start.elapsed_time(end)))          # about 1.2 s
+    reader = threading.Thread(target=busy.read, args=("phi",))
+    reader.start()
+    time.sleep(0.2)
+    got = {f: idle.read(f) for f in want}
+    still_running = not busy_stream.query()
+    reader.join()
+    assert still_running
+    for f in want:
+        assert np.array_equal(got[f], want[f])
