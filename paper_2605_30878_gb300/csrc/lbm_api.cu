@@ -9,7 +9,6 @@
 #include <cstring>
 #include <functional>
 #include <map>
-#include <memory>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -23,6 +22,7 @@
 #include "lbm.h"
 #include "lbm_domain_access.h"
 #include "lbm_launch.cuh"
+#include "lbm_read_stage.h"
 
 using namespace lbmgpu;
 
@@ -739,61 +739,6 @@ lbm_status upload_as(lbm_domain* d, void* dst, const double* src) {
     return LBM_OK;
 }
 
-// Pinned memory that fields are read back through, two halves of kHalf bytes
-// per device, made on first use and kept: a copy into it runs at the link's
-// rate and beside the conversion of the half before, and neither pages of a
-// fresh buffer nor the driver's own staging cost anything.  One read uses it at
-// a time, from the copy it queues behind its domain's steps to the last value;
-// a read that finds it taken goes through a buffer of its own and waits for
-// nothing but its own domain.  lbm_release_cached_memory gives it back.
-struct ReadStage {
-    static constexpr size_t kHalf = (size_t)4 << 20;
-    std::mutex use;
-    char* half[2] = {nullptr, nullptr};
-    cudaEvent_t landed[2] = {nullptr, nullptr};
-    bool ready() {
-        if (half[0]) return true;
-        void* p = nullptr;
-        if (cudaHostAlloc(&p, 2 * kHalf, cudaHostAllocPortable) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        for (auto& e : landed)
-            if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
-                cudaGetLastError();
-                release_events();
-                cudaFreeHost(p);
-                return false;
-            }
-        half[0] = (char*)p;
-        half[1] = half[0] + kHalf;
-        return true;
-    }
-    void release_events() {
-        for (auto& e : landed) {
-            if (e) cudaEventDestroy(e);
-            e = nullptr;
-        }
-    }
-    void release() {
-        std::lock_guard<std::mutex> lk(use);
-        if (!half[0]) return;
-        release_events();
-        cudaFreeHost(half[0]);
-        half[0] = half[1] = nullptr;
-    }
-};
-std::mutex g_stage_mutex;
-std::map<int, std::unique_ptr<ReadStage>> g_stages;
-ReadStage& read_stage() {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    std::lock_guard<std::mutex> lk(g_stage_mutex);
-    auto& s = g_stages[dev];
-    if (!s) s.reset(new ReadStage());
-    return *s;
-}
-
 // `planes` whole fields, src_step elements apart on the device (rows padded to
 // px), into dense host arrays of doubles one after the other.
 template <typename V>
@@ -801,7 +746,7 @@ lbm_status download_as(lbm_domain* d, double* dst, const V* src, int planes, int
     const Layout& L = d->lay;
     const int64_t nx = d->prm.nx, px = L.px, rows = L.nn_dense / nx;
     const int64_t row_bytes = px * (int64_t)sizeof(V);
-    ReadStage& st = read_stage();
+    ReadStage& st = ReadStage::of(d->stream);
     std::unique_lock<std::mutex> one_read(st.use, std::try_to_lock);
     if (!one_read.owns_lock() || row_bytes > (int64_t)ReadStage::kHalf || !st.ready()) {
         if (one_read.owns_lock()) one_read.unlock();
@@ -1425,16 +1370,7 @@ lbm_status lbm_release_cached_memory(void) {
             return LBM_ERR_CUDA;
         }
     }
-    // a stage in use is waited for, with no lock held that a read elsewhere takes
-    std::vector<std::pair<int, ReadStage*>> stages;
-    {
-        std::lock_guard<std::mutex> ls(g_stage_mutex);
-        for (auto& kv : g_stages) stages.push_back({kv.first, kv.second.get()});
-    }
-    for (auto& s : stages) {
-        cudaSetDevice(s.first);
-        s.second->release();
-    }
+    ReadStage::release_all();
     cudaSetDevice(cur);
     return LBM_OK;
 }
