@@ -586,9 +586,16 @@ lbm_status prepare_ghosts(lbm_domain* d, const lbm_ghost* ghosts) {
     return LBM_OK;
 }
 
-// ev: optional events {before ghost, before step, before phi, after phi}
-void launch_one_step(lbm_domain* d, int cur, bool last, cudaStream_t s, cudaEvent_t* ev = nullptr) {
+// ev: optional events {before ghost, before step, before phi, after phi}.
+// Returns the error of the first launch that was refused (under capture the
+// launches after it fail with another one).
+cudaError_t launch_one_step(lbm_domain* d, int cur, bool last, cudaStream_t s, cudaEvent_t* ev = nullptr) {
     const Layout& L = d->lay;
+    cudaError_t first = cudaSuccess;
+    auto launched = [&]() {
+        const cudaError_t e = cudaGetLastError();
+        if (first == cudaSuccess) first = e;
+    };
     if (ev) cudaEventRecord(ev[0], s);
     if (d->ng > 0) {
         const void* wt = d->at<void>(L.off_gwt);
@@ -597,6 +604,7 @@ void launch_one_step(lbm_domain* d, int cur, bool last, cudaStream_t s, cudaEven
                                 d->at<int32_t>(L.off_gcorner), wt, d->cfg.exp_eps, d->cfg.eps, d->phi(), L.plane,
                                 d->errflag(), s);
         });
+        launched();
     }
     StepPtrs sp;
     sp.Nin = d->N(cur); sp.Bin = d->B(cur); sp.Nout = d->N(1 - cur); sp.Bout = d->B(1 - cur);
@@ -605,18 +613,27 @@ void launch_one_step(lbm_domain* d, int cur, bool last, cudaStream_t s, cudaEven
     if (d->tma) { sp.tm_phi = &d->tm_phi; sp.tm_u = &d->tm_u[cur]; }
     if (ev) cudaEventRecord(ev[1], s);
     dispatch(d, [&](auto Lx) { decltype(Lx)::step(d->cfg, sp, last, s); });
+    launched();
     if (ev) cudaEventRecord(ev[2], s);
     dispatch(d, [&](auto Lx) { decltype(Lx)::phi(d->cfg, d->B(1 - cur), d->mask(), d->phi(), d->ng > 0, d->errflag(), s); });
+    launched();
     if (ev) cudaEventRecord(ev[3], s);
+    return first;
 }
 
 lbm_status capture(lbm_domain* d, int start, int nsteps, cudaGraphExec_t* out) {
     cudaGraph_t g = nullptr;
     CUDA_TRY(d, cudaStreamBeginCapture(d->cap, cudaStreamCaptureModeThreadLocal));
     int c = start;
-    for (int k = 0; k < nsteps; ++k) { launch_one_step(d, c, k == nsteps - 1, d->cap); c ^= 1; }
+    cudaError_t le = cudaSuccess;
+    for (int k = 0; k < nsteps && le == cudaSuccess; ++k) { le = launch_one_step(d, c, k == nsteps - 1, d->cap); c ^= 1; }
     cudaError_t e = cudaStreamEndCapture(d->cap, &g);
-    if (e != cudaSuccess) return fail(d, LBM_ERR_CUDA, std::string("stream capture: ") + cudaGetErrorString(e));
+    if (le != cudaSuccess || e != cudaSuccess) {
+        cudaGetLastError();
+        if (g) cudaGraphDestroy(g);
+        return fail(d, LBM_ERR_CUDA, le != cudaSuccess ? std::string("step launch: ") + cudaGetErrorString(le)
+                                                       : std::string("stream capture: ") + cudaGetErrorString(e));
+    }
     e = cudaGraphInstantiate(out, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return fail(d, LBM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
@@ -1113,8 +1130,7 @@ lbm_status lbm_profile_steps(lbm_domain* d, int64_t n, double kernel_ms[3]) {
     for (int k = 0; k < 4; ++k) CUDA_TRY(d, cudaEventCreate(&ev[k]));
     lbm_status st = LBM_OK;
     for (int64_t t = 0; t < n && st == LBM_OK; ++t) {
-        launch_one_step(d, d->cur, true, d->stream, ev);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_one_step(d, d->cur, true, d->stream, ev);
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[3]);
         if (e != cudaSuccess) { st = fail(d, LBM_ERR_CUDA, std::string("profiled step: ") + cudaGetErrorString(e)); break; }
         for (int k = 0; k < 3; ++k) {

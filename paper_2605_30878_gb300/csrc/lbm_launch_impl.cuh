@@ -26,6 +26,8 @@ inline void chi_for_float(const double* chi, double* out) {
     out[0] = rest;
 }
 
+constexpr unsigned kMaxGridY = 65535;         // blocks along y (and z) of a launch
+
 // Launches a kernel of the step chain with programmatic stream serialization:
 // it may start before the work in front of it on the stream has finished, and
 // waits for it in pdl_wait().
@@ -123,12 +125,22 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, int last, cuda
     // counts is that every SM has blocks and the last ones are short.  Against
     // 256-thread tiles (shape 0): 64^2 19.7 -> 13.3 us per step, 300^2 54.9 -> 47.2,
     // 24^3 41.2 -> 25.6, equal from 500 x 300 and 64^3 on; one-warp tiles gain
-    // nothing more (13.1, 47.2, 26.6).
-    constexpr int V = sizeof(T) == 8 ? 3 : 0;
-    if (c.contrast)
-        launch_pdl(k_step<Q, T, S, true, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma, last);
-    else
-        launch_pdl(k_step<Q, T, S, false, V>, step_grid<Q, V>(c.d), step_block<Q, V>(), s, P, b, tm_phi, tm_u, tma, last);
+    // nothing more (13.1, 47.2, 26.6).  They are half as high: a grid too tall for
+    // 65535 of them (ny above 262140 in 2D, 131070 in 3D) runs on shape 0, whose
+    // results are the same to the bit.
+    auto run = [&](auto v) {
+        constexpr int V = decltype(v)::value;
+        const dim3 grid = step_grid<Q, V>(c.d), block = step_block<Q, V>();
+        if (c.contrast) launch_pdl(k_step<Q, T, S, true, V>, grid, block, s, P, b, tm_phi, tm_u, tma, last);
+        else launch_pdl(k_step<Q, T, S, false, V>, grid, block, s, P, b, tm_phi, tm_u, tma, last);
+    };
+    if constexpr (sizeof(T) == 8) {
+        if (step_grid<Q, 3>(c.d).y <= kMaxGridY) {
+            run(std::integral_constant<int, 3>{});
+            return;
+        }
+    }
+    run(std::integral_constant<int, 0>{});
 }
 
 template <typename T, typename S>
