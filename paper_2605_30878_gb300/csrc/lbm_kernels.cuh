@@ -98,6 +98,42 @@ template <int Q> __host__ __device__ constexpr unsigned pop_at(int node) {
 }
 __host__ __device__ constexpr int pop_dir(int d) { return (d - 1) * kGroup; }
 
+// How a kernel of the step chain loads populations.  Fresh: what the kernel in
+// front writes, which may still run when this one's blocks start (pdl_wait), so
+// that it is not constant for this kernel's life: ordinary loads, which stay
+// behind pdl_wait (both are volatile).  Constant: what was complete before this
+// kernel could start, over the read-only path.
+enum class Ld { Fresh, Constant };
+__device__ __forceinline__ float ld_fresh(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_fresh(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_fresh(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ __half ld_fresh(const __half* p) {
+    unsigned short v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __ushort_as_half(v);
+}
+__device__ __forceinline__ __half2 ld_fresh(const __half2* p) {
+    __half2 v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(*reinterpret_cast<unsigned*>(&v)) : "l"(p));
+    return v;
+}
+template <Ld how, typename V> __device__ __forceinline__ V ld(const V* p) {
+    if constexpr (how == Ld::Fresh) return ld_fresh(p);
+    else return __ldg(p);
+}
+
 template <typename S> struct PopStore;
 template <typename V> struct PlainStore {
     static constexpr int kRestBytes = sizeof(V), kMovingBytes = sizeof(V);
@@ -112,8 +148,8 @@ template <typename V> struct PlainStore {
     __device__ static void store_rest(V* r, int idx, V v) { r[idx] = v; }
     __device__ static void store_moving(V* m, int idx, V v, float) { m[idx] = v; }
     // in storage units: the value itself
-    __device__ static V load_units(const V* m, int idx) { return __ldg(m + idx); }
-    __device__ static void accumulate(const V* m, int idx, V& acc) { acc += __ldg(m + idx); }
+    template <Ld how> __device__ static V load_units(const V* m, int idx) { return ld<how>(m + idx); }
+    template <Ld how> __device__ static void accumulate(const V* m, int idx, V& acc) { acc += ld<how>(m + idx); }
     // stores v; exact storage leaves nothing to account for, acc is untouched
     __device__ static void store_units(V* m, int idx, V v, V&) { m[idx] = v; }
 };
@@ -123,8 +159,8 @@ template <> struct PopStore<double> : PlainStore<double> {
 template <> struct PopStore<float> : PlainStore<float> {
     static constexpr bool kShift = true, kExact = true;
     // two adjacent nodes (idx even, so 8-byte aligned): values in storage units
-    __device__ static float2 load_units2(const float* m, int idx) {
-        return __ldg(reinterpret_cast<const float2*>(m + idx));
+    template <Ld how> __device__ static float2 load_units2(const float* m, int idx) {
+        return ld<how>(reinterpret_cast<const float2*>(m + idx));
     }
     __device__ static void store_units2(float* m, int idx, float va, float vb, float&, float&) {
         *reinterpret_cast<float2*>(m + idx) = make_float2(va, vb);
@@ -148,8 +184,10 @@ template <> struct PopStore<__half> {
     }
     // in storage units (value x scale): the step kernels fold the power-of-two
     // scales into their arithmetic instead of scaling every population
-    __device__ static float load_units(const __half* m, int idx) { return __half2float(__ldg(m + idx)); }
-    __device__ static void accumulate(const __half* m, int idx, float& acc) { acc = add_f16_f32(__ldg(m + idx), acc); }
+    template <Ld how> __device__ static float load_units(const __half* m, int idx) { return __half2float(ld<how>(m + idx)); }
+    template <Ld how> __device__ static void accumulate(const __half* m, int idx, float& acc) {
+        acc = add_f16_f32(ld<how>(m + idx), acc);
+    }
     // stores v (already scaled) and adds the value stored to acc
     __device__ static void store_units(__half* m, int idx, float v, float& acc) {
         const __half h = __float2half_rn(v);
@@ -158,8 +196,8 @@ template <> struct PopStore<__half> {
     }
     // two adjacent nodes (idx even, so 4-byte aligned): one 32-bit load or
     // store for both, each value rounded as store_units rounds it
-    __device__ static float2 load_units2(const __half* m, int idx) {
-        return __half22float2(__ldg(reinterpret_cast<const __half2*>(m + idx)));
+    template <Ld how> __device__ static float2 load_units2(const __half* m, int idx) {
+        return __half22float2(ld<how>(reinterpret_cast<const __half2*>(m + idx)));
     }
     __device__ static void store_units2(__half* m, int idx, float va, float vb, float& accA, float& accB) {
         const __half2 h = __floats2half2_rn(va, vb);
@@ -423,7 +461,7 @@ __device__ __forceinline__ void load_halo(const StepParams<T>& P, const T* __res
 // thread in float, k_phi_pair).
 // ---------------------------------------------------------------------------
 template <int Q, typename T, typename S>
-__device__ __forceinline__ void phi_node(const StepParams<T>& P, const S* __restrict__ Bst,
+__device__ __forceinline__ void phi_node(const StepParams<T>& P, const S* Bst,
                                          const uint32_t* __restrict__ mask, T* __restrict__ phi, int x, int y, int z,
                                          int early, int* err) {
     using L = Lattice<Q>;
@@ -442,13 +480,13 @@ __device__ __forceinline__ void phi_node(const StepParams<T>& P, const S* __rest
     // add the rest population last: with FP16 storage the moving values lie on
     // a grid coarse enough for their float sum to be exact, so the node's color
     // comes back as k_step wrote it.
-    const T rest = (T)PS::load_rest(PS::rest(Bst), node);
+    const T rest = (T)ld<Ld::Fresh>(PS::rest(Bst) + node);
     T s = PS::kShift ? T(0) : rest;
 #pragma unroll
     for (int i = 1; i < Q; ++i) {
         const bool back = (m >> i) & 1u;
         const int from = idx_checked(back ? node : node + W.off(-L::cx(i), -L::cy(i), -L::cz(i)), P.plane, err);
-        PS::accumulate(mv + pop_at<Q>(from), back ? pop_dir(L::opp(i)) : pop_dir(i), s);
+        PS::template accumulate<Ld::Fresh>(mv + pop_at<Q>(from), back ? pop_dir(L::opp(i)) : pop_dir(i), s);
     }
     if (PS::kShift) s = rest + (PS::kExact ? s : s * T(1.0 / kScaleB));
     // stored deviations B_i - chi_i/2 sum to phi - 1/2
@@ -456,7 +494,7 @@ __device__ __forceinline__ void phi_node(const StepParams<T>& P, const S* __rest
 }
 
 template <int Q, typename T, typename S>
-__global__ void __launch_bounds__(Tile<Q>::THREADS) k_phi(StepParams<T> P, const S* __restrict__ Bst,
+__global__ void __launch_bounds__(Tile<Q>::THREADS) k_phi(StepParams<T> P, const S* Bst,
                                                           const uint32_t* __restrict__ mask, T* __restrict__ phi,
                                                           int early, int* err) {
     using Tl = Tile<Q>;
@@ -536,7 +574,9 @@ __device__ __forceinline__ float inv_norm_floor(float g2, float floor) {
 // only through phi = sum B, which k_phi computed.  Values come in storage
 // units (times kScaleN with FP16 storage).  In the deviation form the pressure
 // and every moment come from the moving populations (Eq. pressureUpdate), so
-// N[0] is not read.
+// N[0] is not read.  N is constant for the step kernel's whole life: the step
+// before wrote it, and the color kernel in between let nothing start before it
+// had waited for that step.
 template <int Q, typename T, typename S>
 __device__ __forceinline__ void pull_streaming(const StepParams<T>& P, const S* __restrict__ Nin, int node, int x,
                                                int y, int z, T (&N)[Q], int* err) {
@@ -548,8 +588,8 @@ __device__ __forceinline__ void pull_streaming(const StepParams<T>& P, const S* 
     const auto* mv = PS::moving(Nin, pl);
 #pragma unroll
     for (int i = 1; i < Q; ++i)
-        N[i] = (T)PS::load_units(mv + pop_at<Q>(idx_checked(node + Wr.off(-L::cx(i), -L::cy(i), -L::cz(i)), P.plane,
-                                                            err)), pop_dir(i));
+        N[i] = (T)PS::template load_units<Ld::Constant>(
+            mv + pop_at<Q>(idx_checked(node + Wr.off(-L::cx(i), -L::cy(i), -L::cz(i)), P.plane, err)), pop_dir(i));
 }
 template <int Q, typename T, typename S>
 __device__ __forceinline__ void pull_bounce_back(const StepParams<T>& P, const S* __restrict__ Nin, uint32_t m,
@@ -561,7 +601,7 @@ __device__ __forceinline__ void pull_bounce_back(const StepParams<T>& P, const S
     const auto* const at = mv + pop_at<Q>(idx_checked(node, P.plane, err));
 #pragma unroll
     for (int i = 1; i < Q; ++i)
-        if ((m >> i) & 1u) N[i] = (T)PS::load_units(at, pop_dir(L::opp(i)));
+        if ((m >> i) & 1u) N[i] = (T)PS::template load_units<Ld::Constant>(at, pop_dir(L::opp(i)));
 }
 
 // Value types of the float node update.  SF is a float whose every

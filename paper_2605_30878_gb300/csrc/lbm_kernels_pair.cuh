@@ -90,9 +90,10 @@ struct PairNode {
 };
 
 // The pair's moving populations after streaming, in storage units (the
-// deviation form never reads N[0]).
-template <int Q, typename S>
-__device__ __forceinline__ void pull_pair(const StepParams<float>& P, const S* __restrict__ N, const PairNode& pn,
+// deviation form never reads N[0]).  how: Ld::Constant for N in the step kernels,
+// Ld::Fresh for B* in the color kernels.
+template <int Q, Ld how, typename S>
+__device__ __forceinline__ void pull_pair(const StepParams<float>& P, const S* N, const PairNode& pn,
                                           float (&NA)[Q], float (&NB)[Q], int* err) {
     using L = Lattice<Q>;
     using PS = PopStore<S>;
@@ -110,15 +111,15 @@ __device__ __forceinline__ void pull_pair(const StepParams<float>& P, const S* _
         const int cx = L::cx(i), cy = L::cy(i), cz = L::cz(i);
         const int row = nodeA + W.off(0, -cy, -cz);
         if (cx == 0) {
-            const float2 v = PS::load_units2(at(row), pop_dir(i));
+            const float2 v = PS::template load_units2<how>(at(row), pop_dir(i));
             NA[i] = v.x;
             NB[i] = v.y;
         } else if (cx > 0) {
-            NA[i] = (float)PS::load_units(at(row + dl), pop_dir(i));
-            NB[i] = (float)PS::load_units(at(row), pop_dir(i));
+            NA[i] = (float)PS::template load_units<how>(at(row + dl), pop_dir(i));
+            NB[i] = (float)PS::template load_units<how>(at(row), pop_dir(i));
         } else {
-            const float v = (float)PS::load_units(at(row), pop_dir(i) + 1);      // B's column: A is even
-            NB[i] = (float)PS::load_units(at(row + dr), pop_dir(i));
+            const float v = (float)PS::template load_units<how>(at(row), pop_dir(i) + 1);      // B's column: A is even
+            NB[i] = (float)PS::template load_units<how>(at(row + dr), pop_dir(i));
             NA[i] = pn.b_in ? v : NB[i];
         }
     }
@@ -126,12 +127,12 @@ __device__ __forceinline__ void pull_pair(const StepParams<float>& P, const S* _
     if (pn.fluidA && (pn.m.x & ~MASK_NOT_FLUID)) {
 #pragma unroll
         for (int i = 1; i < Q; ++i)
-            if ((pn.m.x >> i) & 1u) NA[i] = (float)PS::load_units(at(nodeA), pop_dir(L::opp(i)));
+            if ((pn.m.x >> i) & 1u) NA[i] = (float)PS::template load_units<how>(at(nodeA), pop_dir(L::opp(i)));
     }
     if (pn.fluidB && (pn.m.y & ~MASK_NOT_FLUID)) {
 #pragma unroll
         for (int i = 1; i < Q; ++i)
-            if ((pn.m.y >> i) & 1u) NB[i] = (float)PS::load_units(at(nodeA), pop_dir(L::opp(i)) + 1);
+            if ((pn.m.y >> i) & 1u) NB[i] = (float)PS::template load_units<how>(at(nodeA), pop_dir(L::opp(i)) + 1);
     }
 }
 
@@ -160,7 +161,7 @@ __device__ __forceinline__ void step_pair_tile(const StepParams<float>& P, const
     // the pair's populations, pulled while the halo is in flight
     const int pl = (int)P.plane;
     float NA[Q], NB[Q];
-    pull_pair<Q, S>(P, b.Nin, pn, NA, NB, err);
+    pull_pair<Q, Ld::Constant>(P, b.Nin, pn, NA, NB, err);
     // the moments of both nodes (one packed lane each) while the halo copy
     // completes; the pulled values are then dead, which keeps them out of the
     // registers the stencils need
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS,
 // of B*, mask and color); 1000 x 600 17.0 -> 15.9 us per step; a 128^3 packing,
 // a third solid, 34.9 -> 36.2.
 template <int Q, typename S>
-__device__ __forceinline__ void phi_pair(const StepParams<float>& P, const S* __restrict__ Bst,
+__device__ __forceinline__ void phi_pair(const StepParams<float>& P, const S* Bst,
                                          const uint32_t* __restrict__ mask, float* __restrict__ phi, int x0, int y0,
                                          int z0, int early, int* err) {
     using PS = PopStore<S>;
@@ -319,8 +320,8 @@ __device__ __forceinline__ void phi_pair(const StepParams<float>& P, const S* __
     if (early) pdl_trigger();
     if (!(pn.fluidA || pn.fluidB)) return;
     float BA[Q], BB[Q];
-    pull_pair<Q, S>(P, Bst, pn, BA, BB, err);
-    const float2 rest = *reinterpret_cast<const float2*>(PS::rest(Bst) + pn.nodeA);
+    pull_pair<Q, Ld::Fresh>(P, Bst, pn, BA, BB, err);
+    const float2 rest = ld<Ld::Fresh>(reinterpret_cast<const float2*>(PS::rest(Bst) + pn.nodeA));
     F2 s(0.f);
 #pragma unroll
     for (int i = 1; i < Q; ++i) s = s + F2(BA[i], BB[i]);
@@ -336,7 +337,7 @@ __device__ __forceinline__ void phi_pair(const StepParams<float>& P, const S* __
 
 template <int Q, typename S, int TXn = 64, int TYn = 0>
 __global__ void __launch_bounds__(PairTile<Q, TXn, TYn>::THREADS)
-    k_phi_pair(StepParams<float> P, const S* __restrict__ Bst, const uint32_t* __restrict__ mask,
+    k_phi_pair(StepParams<float> P, const S* Bst, const uint32_t* __restrict__ mask,
                float* __restrict__ phi, int early, int* err) {
     using Tl = PairTile<Q, TXn, TYn>;
     // tiles in the reverse of the step's order, as k_phi
