@@ -436,7 +436,7 @@ void stencil_offsets(int Q, std::vector<int>& ox, std::vector<int>& oy, std::vec
 }
 
 // Color weights chi (Appendix A / Eq. ChiTerm) and alpha from M_phi at p = 0.
-void color_weights(int Q, double M_phi, double chi[19], double& alpha, double& c2chi) {
+void color_weights(int Q, double M_phi, double chi[19], double& alpha) {
     const double cs2 = 1.0 / 3.0;
     const double w0 = Q == 9 ? 4.0 / 9.0 : 1.0 / 3.0;
     alpha = 1.0 - 2.0 * M_phi * (1.0 - w0) / cs2;
@@ -449,7 +449,6 @@ void color_weights(int Q, double M_phi, double chi[19], double& alpha, double& c
             chi[i] = (1.0 - alpha) * Lattice<19>::w(i) / (1.0 - w0);          // same rule in 3D
         }
     }
-    c2chi = (1.0 - alpha) * cs2 / (1.0 - w0);
 }
 
 // f(k) for every fluid node k (dense index) of the domain, from the row bits
@@ -692,10 +691,10 @@ bool encode_halo_maps(const lbm_domain* d, CUtensorMap out[3]) {
 template <int Q>
 bool make_halo_maps(lbm_domain* d) {
     CUtensorMap m[3];
-    if (!(!d->cfg.pair ? encode_halo_maps<Q, 0>(d, m)
-          : d->cfg.pair_width == 64 ? encode_halo_maps_tile<PairTile<Q>>(d, m)
-                                    : encode_halo_maps_tile<NarrowTile<Q>>(d, m)))
-        return false;
+    bool ok = false;
+    if (d->cfg.pair) with_pair_tile<Q>(d->cfg, [&](auto tile) { ok = encode_halo_maps_tile<decltype(tile)>(d, m); });
+    else ok = encode_halo_maps<Q, 0>(d, m);
+    if (!ok) return false;
     d->tm_phi = m[0];
     d->tm_u[0] = m[1];
     d->tm_u[1] = m[2];
@@ -914,9 +913,9 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     d->ng = n_ghosts;
     d->stream = (cudaStream_t)cuda_stream;
 
-    double alpha, c2chi;
+    double alpha;
     StepConfig& c = d->cfg;
-    color_weights(P.lattice, P.M_phi, c.chi, alpha, c2chi);
+    color_weights(P.lattice, P.M_phi, c.chi, alpha);
     if (!(alpha > 0.0 && alpha < 1.0)) { delete d; return fail(nullptr, LBM_ERR_ARG, "M_phi gives alpha outside (0,1)"); }
     c.Q = P.lattice;
     c.contrast = d->contrast;
@@ -925,7 +924,6 @@ lbm_status lbm_create_domain(const lbm_params* params, const uint8_t* solid, con
     c.nu_l = P.mu_l / P.rho_l; c.nu_g = P.mu_g / P.rho_g;
     c.sigma = P.sigma; c.W = P.W;
     for (int a = 0; a < 3; ++a) c.g[a] = (L.D == 2 && a == 2) ? 0.0 : P.g[a];
-    c.c2chi = c2chi;
     c.eps = -(4.0 / P.W) * std::cos(P.theta);
     c.exp_eps = std::exp(c.eps);
     c.ghost_rule = P.ghost_rule;

@@ -45,9 +45,8 @@ struct StepParams {
     int px;                  // row pitch: node = x + px * (y + ny * z), px = nx rounded up to 4
     int64_t plane;           // elements between consecutive planes of a field
     T rho_l, rho_g, drho;    // drho = rho_l - rho_g
-    T inv_nu_l, inv_nu_g;    // 1/nu_l, 1/nu_g
-    T sigma, W;
-    T nu_l, nu_g;            // kinematic viscosities
+    T inv_nu_l, inv_nu_g;    // 1/nu_l, 1/nu_g (kinematic)
+    T sigma;
     T k48W, k3W2, two_over_W;   // 48/W, 3W/2, 2/W
     T g[3];
     T chi[19];               // float arithmetic: the storage reference, on a 2^-24 grid, summing to exactly 1
@@ -55,8 +54,6 @@ struct StepParams {
     // diagonal/edge): zero in FP64; in float arithmetic the equilibrium and the
     // pressure's zero are taken at the exact chi through these corrections
     T chi_err[3];
-    T c2chi;                 // sum_i chi_i c_ix^2 = (1-alpha) c_s^2/(1-w_0)
-    T exp_eps;               // exp(eps), eps = -(4/W) cos(theta)
 };
 
 // Population storage.  S = double (FP64 mode): full values, the ones the state
@@ -136,7 +133,6 @@ template <Ld how, typename V> __device__ __forceinline__ V ld(const V* p) {
 
 template <typename S> struct PopStore;
 template <typename V> struct PlainStore {
-    static constexpr int kRestBytes = sizeof(V), kMovingBytes = sizeof(V);
     using Rest = V;
     using Moving = V;
     __device__ static const V* rest(const V* p) { return p; }
@@ -169,7 +165,6 @@ template <> struct PopStore<float> : PlainStore<float> {
 };
 template <> struct PopStore<__half> {
     static constexpr bool kShift = true, kExact = false;     // moving populations are rounded on store
-    static constexpr int kRestBytes = 4, kMovingBytes = 2;
     __device__ static const float* rest(const __half* p) { return reinterpret_cast<const float*>(p); }
     __device__ static float* rest(__half* p) { return reinterpret_cast<float*>(p); }
     __device__ static const __half* moving(const __half* p, int plane) { return p + 2 * plane; }
@@ -698,24 +693,11 @@ struct H2 {
     bool odd;                                   // a constant once the direction loops are unrolled
     __device__ __forceinline__ operator F2() const { return F2(v.x, v.y); }
 };
-__device__ __forceinline__ F2 operator+(F2 a, H2 b) {
-    return b.odd ? F2(__fadd_rn(a.lo(), b.v.x), __fadd_rn(a.hi(), b.v.y)) : a + F2(b);
-}
-__device__ __forceinline__ F2 operator-(F2 a, H2 b) {
-    return b.odd ? F2(__fsub_rn(a.lo(), b.v.x), __fsub_rn(a.hi(), b.v.y)) : a - F2(b);
-}
 __device__ __forceinline__ F2 operator-(H2 a, F2 b) {
     return a.odd ? F2(__fsub_rn(a.v.x, b.lo()), __fsub_rn(a.v.y, b.hi())) : F2(a) - b;
 }
 __device__ __forceinline__ F2 operator-(H2 a, H2 b) {
     return a.odd ? F2(__fsub_rn(a.v.x, b.v.x), __fsub_rn(a.v.y, b.v.y)) : F2(a) - F2(b);
-}
-__device__ __forceinline__ F2 operator-(H2 a) { return -F2(a); }
-__device__ __forceinline__ F2 operator*(H2 a, F2 b) {
-    return a.odd ? F2(__fmul_rn(a.v.x, b.lo()), __fmul_rn(a.v.y, b.hi())) : F2(a) * b;
-}
-__device__ __forceinline__ F2 fma(H2 a, F2 b, F2 c) {
-    return a.odd ? F2(fmaf(a.v.x, b.lo(), c.lo()), fmaf(a.v.y, b.hi(), c.hi())) : fma(F2(a), b, c);
 }
 
 // a + k t for an integer coefficient k that is a constant once the direction
@@ -901,7 +883,7 @@ struct NodeUpdate {
         uu = D == 2 ? fma(u[0], u[0], u[1] * u[1]) : fma(u[0], u[0], fma(u[1], u[1], u[2] * u[2]));
         p = fma(V(-R(0.5 * w0)), uu, pres_base) * inv_1mw0;
 
-        // collision: traceless second moments of N - Neq, with sum Neq c c = (c2chi + p) I + u u,
+        // collision: traceless second moments of N - Neq, with sum Neq c c = (sum chi c_x^2 + p) I + u u,
         // in N's storage units (the moments are raw, the u u terms take the scale)
         const V omega1 = V(R(1.0)) - rcp(tau);                                        // 1 - s_nu
         const V o4 = omega1 * V(R(0.25));

@@ -45,8 +45,8 @@ struct PairTile {
     __host__ __device__ static constexpr int off(int cx, int cy, int cz) { return cx + HX * (cy + HY * cz); }
 };
 
-// 32 nodes wide, as batch shape 0.
-template <int Q> using NarrowTile = PairTile<Q, 32, Q == 9 ? 8 : 4>;
+// 32 nodes wide, as batch shape 0 (D3Q19).
+using NarrowTile = PairTile<19, 32, 4>;
 
 // Resident blocks per SM the pair kernel is compiled for (registers per thread
 // <= 65536 / (THREADS * blocks)): 7 (72 registers; FP32 storage with density

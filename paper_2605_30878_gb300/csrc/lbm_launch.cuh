@@ -24,13 +24,24 @@ struct StepConfig {
     double rho_l, rho_g, nu_l, nu_g, sigma, W;
     double g[3];
     double chi[19];
-    double c2chi;
     double exp_eps;
     double eps;                    // -(4/W) cos(theta)
     int ghost_rule;                // lbm_ghost_rule
     bool pair = false;             // float arithmetic: the two-node step kernel (k_step_pair)
-    int pair_width = 32;           // nodes along x of its tiles, 32 or 64
+    int pair_width = 64;           // nodes along x of its tiles, 64 or (D3Q19) 32
 };
+
+// f of the tile of a domain's two-node kernels (narrow ones in 3D only).
+template <int Q, typename F>
+void with_pair_tile(const StepConfig& c, F&& f) {
+    if constexpr (Q == 19) {
+        if (c.pair_width == 32) {
+            f(NarrowTile{});
+            return;
+        }
+    }
+    f(PairTile<Q>{});
+}
 
 struct StepPtrs {
     const void* Nin;

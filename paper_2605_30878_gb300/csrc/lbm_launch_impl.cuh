@@ -54,8 +54,6 @@ StepParams<T> Launch<T, S>::params(const StepConfig& c) {
     P.rho_l = (T)c.rho_l; P.rho_g = (T)c.rho_g; P.drho = (T)(c.rho_l - c.rho_g);
     P.inv_nu_l = (T)(1.0 / c.nu_l); P.inv_nu_g = (T)(1.0 / c.nu_g);
     P.sigma = (T)c.sigma;
-    P.W = (T)c.W;
-    P.nu_l = (T)c.nu_l; P.nu_g = (T)c.nu_g;
     P.k48W = (T)(48.0 / c.W); P.k3W2 = (T)(1.5 * c.W); P.two_over_W = (T)(2.0 / c.W);
     for (int a = 0; a < 3; ++a) P.g[a] = (T)c.g[a];
     double chi[19];
@@ -68,8 +66,6 @@ StepParams<T> Launch<T, S>::params(const StepConfig& c) {
     P.chi_err[0] = (T)(c.chi[0] - chi[0]);
     P.chi_err[1] = (T)(c.chi[1] - chi[1]);
     P.chi_err[2] = (T)(c.chi[diag] - chi[diag]);
-    P.c2chi = (T)c.c2chi;
-    P.exp_eps = (T)c.exp_eps;
     return P;
 }
 
@@ -117,7 +113,7 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, int last, cuda
                 else
                     launch_pdl(k_step_pair<Q, S, false, Tl::TX, Tl::TY>, grid, block, s, P, b, tm_phi, tm_u, tma, last);
             };
-            if (c.pair_width == 64) run(PairTile<Q>{}); else run(NarrowTile<Q>{});
+            with_pair_tile<Q>(c, run);
             return;
         }
     }
@@ -155,15 +151,13 @@ void Launch<T, S>::phi(const StepConfig& c, const void* Bst, const uint32_t* mas
     const int early = ghosts_follow;
     if constexpr (sizeof(T) == 4) {
         if (c.pair) {
-            auto run = [&](auto q, auto tile) {
+            auto run = [&](auto tile) {
                 using Tl = decltype(tile);
-                launch_pdl(k_phi_pair<decltype(q)::value, S, Tl::TX, Tl::TY>, pair_grid<Tl>(c.d),
+                launch_pdl(k_phi_pair<Tl::D == 2 ? 9 : 19, S, Tl::TX, Tl::TY>, pair_grid<Tl>(c.d),
                            dim3(Tl::BX, Tl::TY, Tl::TZ), s, P, (const S*)Bst, mask, (T*)phi, early, err);
             };
-            const std::integral_constant<int, 9> q9;
-            const std::integral_constant<int, 19> q19;
-            if (c.Q == 9) c.pair_width == 64 ? run(q9, PairTile<9>{}) : run(q9, NarrowTile<9>{});
-            else c.pair_width == 64 ? run(q19, PairTile<19>{}) : run(q19, NarrowTile<19>{});
+            if (c.Q == 9) with_pair_tile<9>(c, run);
+            else with_pair_tile<19>(c, run);
             return;
         }
     }
