@@ -195,6 +195,16 @@ def k_step_bytes_per_fluid_node(Q, D, s, contrast, moving=None, rest=None):
     return (Q - 1) * moving + 2 * pop + s + (D * s if contrast else 0) + D * s + s + 4
 
 
+def run_bytes_per_fluid_node(step_bytes, steps, before, D, s, contrast):
+    """Algorithmic bytes per fluid node and step of a run of `steps` steps in one
+    call, `before` steps after the state was set: step_bytes (a step by itself)
+    less the p, and without a density contrast the u, that the first seven of
+    eight captured steps do not store.  Runs of eight start at an even step."""
+    head = min(before % 2, steps)
+    stored = head + (steps - head) // 8 + (steps - head) % 8
+    return step_bytes - (1.0 - stored / steps) * s * (1 if contrast else 1 + D)
+
+
 def workload(theta, precision, n=N_GRID):
     from paper_2605_30878_gb300 import workloads as wl
     scale = n / float(N_GRID)
@@ -706,7 +716,7 @@ def run_ours(args):
     traffic = recorded_traffic(fluid, fp16=prec == lbm.FP16)
     share = kms / kms.sum()
     launches = dom.launches_per_step()
-    bytes_step = dom.bytes_per_fluid_node()
+    bytes_step = run_bytes_per_fluid_node(dom.bytes_per_fluid_node(), args.steps, args.warmup, D, s, True)
     dom.close()
     del dom
     torch.cuda.empty_cache()

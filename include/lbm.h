@@ -226,7 +226,10 @@ lbm_status lbm_ghost_table(lbm_domain* dom, int64_t* corner, double* weight, int
 int64_t lbm_ghost_fallbacks(const lbm_domain* dom);
 
 /* Kernel launches one lbm_step(dom, 1) issues, and the algorithmic device
- * bytes one step moves per fluid node (populations, fields, node type). */
+ * bytes that step moves per fluid node (populations, fields, node type).  A run
+ * of n >= 8 steps moves less: of eight captured steps only the last stores p,
+ * and u where no density contrast makes the next step read it.  The LBM_FP64
+ * count holds a read of the rest population that the kernels do not make. */
 int32_t lbm_launches_per_step(const lbm_domain* dom);
 double  lbm_bytes_per_fluid_node(const lbm_domain* dom);
 int64_t lbm_fluid_nodes(const lbm_domain* dom);

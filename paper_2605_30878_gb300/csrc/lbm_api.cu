@@ -832,8 +832,8 @@ lbm_status init_state(lbm_domain* d, int mode, const double ctr[3], double R0) {
     // (init_pops) and the velocity of the first step's stencil, 0.  Population
     // slots of non-fluid nodes are never read (every pull of a fluid node reads
     // a fluid source or the node's own slots, as the diagnostics and state
-    // transfer do), the second velocity buffer is written at every fluid node
-    // by the first step, and the velocity of non-fluid nodes stays 0 from the
+    // transfer do), a velocity buffer is written at every fluid node before a
+    // later step or the caller reads it, and the velocity of non-fluid nodes stays 0 from the
     // domain's creation (no kernel writes it but as 0).  So of the state only
     // the first velocity buffer and p (state read back as 0 before a step) are
     // cleared.
@@ -1335,12 +1335,13 @@ double lbm_bytes_per_fluid_node(const lbm_domain* d) {
     const double moving = (d->lay.Q - 1) * (double)d->lay.pop_elem;
     const double pop = (double)d->lay.rest_elem + moving;   // per node and array
     // k_step pulls N and takes every moment from the moving populations; the FP64
-    // count still holds the rest population's pull
+    // count also holds a pull of the rest population, which the kernel does not make
     const double pull = d->lay.elem == 8 ? pop : moving;
     const int D = d->lay.D;
     // N* and B* written, B* pulled by k_phi; phi written (k_phi) and read (k_step);
     // u written, and read when the density contrast makes F_visc active; p written; the 4-byte
-    // bounce-back mask read by k_step and k_phi
+    // bounce-back mask read by k_step and k_phi.  (In a captured run of eight steps
+    // the first seven do not store p, nor u without a contrast.)
     return pull + 3.0 * pop + 2.0 * s + (d->contrast ? 2.0 : 1.0) * D * s + s + 8.0;
 }
 
