@@ -1124,6 +1124,9 @@ lbm_status lbm_profile_steps(lbm_domain* d, int64_t n, double kernel_ms[3]) {
     if (!d || !kernel_ms) return fail(d, LBM_ERR_ARG, "NULL argument");
     if (n < 1) return fail(d, LBM_ERR_ARG, "n must be >= 1");
     if (d->poisoned) return fail(d, LBM_ERR_TIMEOUT, kPoisonedMsg);
+    // what wrote the state is done before a step kernel, launched outside a graph,
+    // may be resident (it reads N as constant)
+    CUDA_TRY(d, cudaStreamSynchronize(d->stream));
     cudaEvent_t ev[4];
     for (int k = 0; k < 4; ++k) CUDA_TRY(d, cudaEventCreate(&ev[k]));
     lbm_status st = LBM_OK;
@@ -1727,6 +1730,14 @@ lbm_status lbm_batch_tune(lbm_batch* b, int32_t steps_per_trial, int32_t* chosen
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return bfail(b, LBM_ERR_CUDA, "cudaEventCreate failed");
+    // what wrote the states is done before a step kernel, launched outside a graph,
+    // may be resident (it reads N as constant)
+    const cudaError_t done = cudaStreamSynchronize(b->stream);
+    if (done != cudaSuccess) {
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        return bfail(b, LBM_ERR_CUDA, cudaGetErrorString(done));
+    }
     double best = 1e300;
     int best_v = 0;
     for (int V = 0; V < kTileVariants; ++V) {

@@ -571,7 +571,8 @@ __device__ __forceinline__ float inv_norm_floor(float g2, float floor) {
 // and every moment come from the moving populations (Eq. pressureUpdate), so
 // N[0] is not read.  N is constant for the step kernel's whole life: the step
 // before wrote it, and the color kernel in between let nothing start before it
-// had waited for that step.
+// had waited for that step; what wrote the state before the first step is done
+// when a graph starts, and waited for where steps are launched without one.
 template <int Q, typename T, typename S>
 __device__ __forceinline__ void pull_streaming(const StepParams<T>& P, const S* __restrict__ Nin, int node, int x,
                                                int y, int z, T (&N)[Q], int* err) {
@@ -727,14 +728,15 @@ struct Acc {
 // node takes: ~600 in D3Q19 and ~290 in D2Q9 in this form, against ~2400 and
 // ~1150 for the model's expressions evaluated as printed (a division by each
 // constant, no fused multiply-add): 64^3 1092 -> 246 us per step, 500 x 300
-// 288 -> 71 us.  N stored as its deviation would save 16 of them (237 and 69 us),
-// but a state read and written back would then not go on to the bit.
+// 288 -> 71 us.  N stored as its deviation would save 16 of them (237 and 69 us) and
+// keep u and p to 1e-15 instead of 2e-13 (relative, after 20 steps), but a state
+// read and written back would not go on to the bit: doubles near chi end at 1e-18.
 //
 // Arithmetic of one fluid node (V = SF, or SD in FP64), or of the two nodes of a
 // pair (V = F2, one packed lane each), written once so that the one-node and the
 // two-node kernels round alike.  Inputs: the pulled populations N as stored
-// (deviations, in storage units with FP16 storage; full values in FP64), the color phi at the node
-// and its isotropic stencils gp = grad phi, lap = lap phi and gu[a][b] = d_a u_b
+// (deviations, in storage units with FP16 storage; full values in FP64), the color
+// phi at the node and its isotropic stencils gp = grad phi, lap = lap phi and gu[a][b] = d_a u_b
 // (the stencil weights carry the 3 and the 6).
 //
 // Every operation of V rounds on its own and fuses only where written as fma,

@@ -119,9 +119,9 @@ void Launch<T, S>::step_q(const StepConfig& c, const StepPtrs& p, int last, cuda
     }
     // FP64: 128-thread tiles.  It is bound by its arithmetic rate per SM, so what
     // counts is that every SM has blocks and the last ones are short.  Against
-    // 256-thread tiles (shape 0): 64^2 19.7 -> 13.3 us per step, 300^2 54.9 -> 47.2,
-    // 24^3 41.2 -> 25.6, equal from 500 x 300 and 64^3 on; one-warp tiles gain
-    // nothing more (13.1, 47.2, 26.6).  They are half as high: a grid too tall for
+    // 256-thread tiles (shape 0): 64^2 21.5 -> 13.6 us per step, 300^2 55.0 -> 46.9,
+    // 24^3 41.3 -> 24.9, equal from 500 x 300 (71.5, 71.2) and 64^3 (248, 247) on;
+    // one-warp tiles gained nothing more.  They are half as high: a grid too tall for
     // 65535 of them (ny above 262140 in 2D, 131070 in 3D) runs on shape 0, whose
     // results are the same to the bit.
     auto run = [&](auto v) {

@@ -27,3 +27,13 @@ def test_color_kernels_load_populations_fresh(file, name):
     loads = re.findall(r"\b(?:PS::(?:template )?(?:load_\w+|accumulate)|pull_pair|ld)\b[^(]*\(", body)
     assert len(loads) == 2 and all("Ld::Fresh" in x for x in loads), loads
     assert not re.search(r"[=+]\s*\*", body), "a plain dereference on the right-hand side"
+
+
+@pytest.mark.parametrize("entry,launch", [("lbm_profile_steps", "launch_one_step("), ("lbm_batch_tune", "batch_launch_step(")])
+def test_steps_launched_without_a_graph_wait_for_the_state(entry, launch):
+    """The step kernels read N over the read-only path: the kernel that wrote the
+    first step's N must have completed before one can be resident."""
+    with open(os.path.join(build.CSRC, "lbm_api.cu")) as f:
+        s = f.read()
+    start = s.index("lbm_status %s(" % entry)
+    assert "cudaStreamSynchronize(" in s[start:s.index(launch, start)]
