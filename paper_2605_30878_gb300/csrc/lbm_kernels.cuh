@@ -44,8 +44,12 @@ struct StepParams {
     int nx, ny, nz;
     int px;                  // row pitch: node = x + px * (y + ny * z), px = nx rounded up to 4
     int64_t plane;           // elements between consecutive planes of a field
-    T rho_l, rho_g, drho;    // drho = rho_l - rho_g
+    T rho_g, drho;           // drho = rho_l - rho_g
     T inv_nu_l, inv_nu_g;    // 1/nu_l, 1/nu_g (kinematic)
+    // FP64: the smaller of the phases' densities and what the other has more, and
+    // whether the smaller one is the liquid's; the same of 1/nu
+    T rho_low, rho_more, inv_nu_low, inv_nu_more;
+    int rho_low_liquid, inv_nu_low_liquid;
     T sigma;
     T k48W, k3W2, two_over_W;   // 48/W, 3W/2, 2/W
     T g[3];
@@ -728,7 +732,7 @@ struct Acc {
 // node takes: ~600 in D3Q19 and ~290 in D2Q9 in this form, against ~2400 and
 // ~1150 for the model's expressions evaluated as printed (a division by each
 // constant, no fused multiply-add): 64^3 1092 -> 246 us per step, 500 x 300
-// 288 -> 71 us.  N stored as its deviation would save 16 of them (237 and 69 us) and
+// 288 -> 70 us.  N stored as its deviation would save 16 of them (237 and 69 us) and
 // keep u and p to 1e-15 instead of 2e-13 (relative, after 20 steps), but a state
 // read and written back would not go on to the bit: doubles near chi end at 1e-18.
 //
@@ -818,12 +822,12 @@ struct NodeUpdate {
         // mixture density and viscosity (Sec. II), relaxation time (Appendix A)
         V rho, inv_nu;                                   // 1/nu = phi/nu_l + (1-phi)/nu_g
         if constexpr (kFull) {
-            // sums of positive terms: in the float form below a large viscosity or
-            // small density of the liquid is the difference of two large numbers
-            // (nu_l/nu_g = 1000: 1/nu 2e-14 off); 3 operations more per node
+            // sums of positive terms, from the phase that has less: in the float form
+            // below a large viscosity or small density of the liquid is the
+            // difference of two large numbers (nu_l/nu_g = 1000: 1/nu 2e-14 off)
             const V gas = V(R(1.0)) - phi;
-            rho = fma(V(P.rho_l), phi, V(P.rho_g) * gas);
-            inv_nu = fma(phi, V(P.inv_nu_l), gas * V(P.inv_nu_g));
+            rho = fma(V(P.rho_more), P.rho_low_liquid ? gas : phi, V(P.rho_low));
+            inv_nu = fma(P.inv_nu_low_liquid ? gas : phi, V(P.inv_nu_more), V(P.inv_nu_low));
         } else {
             rho = fma(V(P.drho), phi, V(P.rho_g));
             inv_nu = fma(phi, V(P.inv_nu_l - P.inv_nu_g), V(P.inv_nu_g));

@@ -3,9 +3,9 @@
 // Launch<T, S> (and so every kernel) once each.
 #pragma once
 
-#include <type_traits>
-
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "lbm_launch.cuh"
 
@@ -51,8 +51,11 @@ StepParams<T> Launch<T, S>::params(const StepConfig& c) {
     P.nx = c.d.nx; P.ny = c.d.ny; P.nz = c.d.nz;
     P.px = c.d.px;
     P.plane = c.d.plane;
-    P.rho_l = (T)c.rho_l; P.rho_g = (T)c.rho_g; P.drho = (T)(c.rho_l - c.rho_g);
+    P.rho_g = (T)c.rho_g; P.drho = (T)(c.rho_l - c.rho_g);
     P.inv_nu_l = (T)(1.0 / c.nu_l); P.inv_nu_g = (T)(1.0 / c.nu_g);
+    P.rho_low = (T)std::min(c.rho_l, c.rho_g); P.rho_more = (T)std::fabs(c.rho_l - c.rho_g);
+    P.inv_nu_low = std::min(P.inv_nu_l, P.inv_nu_g); P.inv_nu_more = (T)std::fabs(P.inv_nu_l - P.inv_nu_g);
+    P.rho_low_liquid = c.rho_l < c.rho_g; P.inv_nu_low_liquid = P.inv_nu_l < P.inv_nu_g;
     P.sigma = (T)c.sigma;
     P.k48W = (T)(48.0 / c.W); P.k3W2 = (T)(1.5 * c.W); P.two_over_W = (T)(2.0 / c.W);
     for (int a = 0; a < 3; ++a) P.g[a] = (T)c.g[a];
