@@ -566,7 +566,7 @@ def run_packing_bench(lbm, steps, checkpoints=10, fp64_steps=200):
     seed 1): liquid slab 0 <= x < 16 (tanh, periodic image included) in the
     sphere-free reservoir, theta = 45 deg, density and viscosity ratio 1,
     sigma = 0.01, all periodic.  FP32 and FP16 population storage run `steps`
-    steps; FP64 (about 45x slower on this GPU, whose FP64 units are few) runs
+    steps; FP64 (about 13x slower on this GPU, whose FP64 units are few) runs
     the first `fp64_steps` as the reference.  Reported: the liquid saturation
     of the packing region (sum of phi over its fluid nodes / their count) at
     each checkpoint, its deviation from FP64 and from FP32, the phase-mass

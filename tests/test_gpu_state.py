@@ -60,7 +60,7 @@ def test_read_of_an_idle_domain_does_not_wait_for_another_domain(precision):
     read of an idle domain on another stream returns, with the right values."""
     import torch
     busy_stream, idle_stream = torch.cuda.Stream(), torch.cuda.Stream()
-    shape = (48, 96, 96)
+    shape = (160, 160, 160)                      # few launches in a second: none blocks on a full queue
     busy, idle = _drop(shape, 10.0, precision, stream=busy_stream), _drop(shape, 10.0, precision, stream=idle_stream)
     idle.step(8)
     want = {f: idle.read(f) for f in ("phi", "u")}
